@@ -152,7 +152,12 @@ def _scene(case, seed):
     else:
         u = normal(64, 3)
         centres = u / u.norm(dim=1, keepdim=True) * 10.0 * uniform(64, 1) ** (1.0 / 3.0)
-        rots = torch.linalg.qr(normal(64, 3, 3))[0] * (uniform(64, 1, 3) * 1.7 + 0.3)
+        w, x, y, z = torch.nn.functional.normalize(normal(64, 4)).unbind(1)
+        rots = torch.stack([
+            1 - 2 * (y * y + z * z), 2 * (x * y - w * z), 2 * (x * z + w * y),
+            2 * (x * y + w * z), 1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
+            2 * (x * z - w * y), 2 * (y * z + w * x), 1 - 2 * (x * x + y * y)], 1).view(-1, 3, 3)
+        rots = rots * (uniform(64, 1, 3) * 1.7 + 0.3)  # axis standard deviations
         k = torch.randint(0, 64, (n,), generator=g, device=dev)
         means = centres[k] + torch.einsum("nij,nj->ni", rots[k], normal(n, 3))
         r = means.norm(dim=1, keepdim=True)
