@@ -22,7 +22,8 @@
 //      super-tile and per-tile counts; scans over segments and over all
 //      tiles give every tile's list start (the ranges);
 //   7. expansion: each segment writes its rows into the lists of the tiles
-//      they cover, ranked by warp ballots, which keeps the depth order.
+//      they cover, a warp per tile row, ranked by warp scans, which keeps the
+//      depth order.
 // The result is exactly the order of a 64-bit (tile << 32 | depth) key sort
 // with ties by Gaussian id.
 //
@@ -221,6 +222,15 @@ __device__ __forceinline__ int4 view_rect(const int* __restrict__ rect, unsigned
   r.w = min(r.w, c.TY);
   if (r.z <= r.x || r.w <= r.y) r = make_int4(0, 0, 0, 0);
   return r;
+}
+
+// The descriptor of a rect inside a super-tile, in tiles relative to the
+// super-tile's origin: bit r set when it covers tile row r, bit 8 + c when it
+// covers tile column c (x0 < 8, x1 > 0, y0 < 8, y1 > 0: the rect meets it).
+__device__ __forceinline__ unsigned rect_masks(int x0, int x1, int y0, int y1) {
+  const unsigned cols = (0xffu << max(x0, 0)) & (0xffu >> (8 - min(x1, 8)));
+  const unsigned rows = (0xffu << max(y0, 0)) & (0xffu >> (8 - min(y1, 8)));
+  return rows | (cols << 8);
 }
 
 // Super-tile span [x0, x1) x [y0, y1) of a non-empty tile rect.
@@ -860,11 +870,9 @@ __global__ void __launch_bounds__(kScanThreads) rows_expand_kernel(
       }
       unsigned key = (unsigned)(id0 + y * stx + x);
       if (packed) {
-        // the row's rect inside this super-tile: x0 | x1 << 4 | y0 << 8 | y1 << 12
+        // the rows and columns of this super-tile that the rect covers
         const int ox = 8 * (q.x + x), oy = 8 * (q.y + y);
-        const unsigned dx0 = (unsigned)max(r.x - ox, 0), dx1 = (unsigned)min(r.z - ox, 8);
-        const unsigned dy0 = (unsigned)max(r.y - oy, 0), dy1 = (unsigned)min(r.w - oy, 8);
-        key |= (dx0 | (dx1 << 4) | (dy0 << 8) | (dy1 << 12)) << 16;
+        key |= rect_masks(r.x - ox, r.z - ox, r.y - oy, r.w - oy) << 16;
       }
       kk[t] = key;
       vv[t] = row;
@@ -946,11 +954,11 @@ __global__ void __launch_bounds__(256) ranges_kernel(const unsigned* __restrict_
 // of the super-tile (64), the count of rows covering the tile; per tile, the
 // exclusive scan of those counts over the super-tile's segments; per tile,
 // the list start (scan over all tiles); then every segment writes each of
-// its rows into the lists of the tiles it covers, ranks from warp ballots,
-// so each list keeps the depth order of the rows.
+// its rows into the lists of the tiles it covers, in the rows' order, so
+// each list keeps their depth order.
 // ----------------------------------------------------------------------------
 constexpr int kSeg = 1024;
-static_assert(kSeg % 256 == 0, "st_count_kernel loads a segment in groups of 256");
+static_assert(kSeg % 256 == 0, "a segment is loaded in groups of 256");
 
 __device__ __forceinline__ int view_of_st(const CamTable& ct, int s) {
   int v = 0;
@@ -958,17 +966,39 @@ __device__ __forceinline__ int view_of_st(const CamTable& ct, int s) {
   return v;
 }
 
+// A segment as st_segments_kernel lists it: its items [b, e), the global id of
+// its super-tile's first tile, and (packed) the view's tiles per row and the
+// tile columns and rows of the super-tile that lie in the view.
+struct __align__(16) Segment {
+  unsigned b, e;
+  int tile;
+  unsigned shape;  // TX | columns << 16 | rows << 20
+  __device__ __forceinline__ int tx() const { return (int)(shape & 0xffffu); }
+  __device__ __forceinline__ int cols() const { return (int)((shape >> 16) & 15u); }
+  __device__ __forceinline__ int rows() const { return (int)(shape >> 20); }
+};
+
+__device__ __forceinline__ Segment load_segment(const Segment* __restrict__ segs, long long g) {
+  const uint4 v = __ldg(reinterpret_cast<const uint4*>(segs + g));
+  return Segment{v.x, v.y, (int)v.z, v.w};
+}
+
 // Segments of every super-tile: seg_first[s] (exclusive scan of
-// ceil(len_s / kSeg)), seg_first[S] = total, seg_st[g] = super-tile of g.
+// ceil(len_s / kSeg)), seg_first[S] = total, segs[g] and (when not NULL)
+// seg_st[g] = super-tile of g.
 // One CTA of 1024 threads.
 __global__ void __launch_bounds__(1024) st_segments_kernel(uint2* __restrict__ st_ranges,
                                                            int S, const unsigned* __restrict__ totals,
                                                            const long long* __restrict__ q_eff,
                                                            unsigned* __restrict__ seg_first,
+                                                           Segment* __restrict__ segs,
                                                            unsigned* __restrict__ seg_st,
+                                                           const CamTable ct,
                                                            long long* __restrict__ n_seg) {
   __shared__ unsigned s_w[32];
   __shared__ unsigned s_carry;
+  __shared__ Segment s_seg[1024];    // the super-tile's whole range, tile and shape
+  __shared__ unsigned s_first[1024];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (totals) {
     // one radix pass sorted the items by super-tile (S <= 512): the per-digit
@@ -1006,11 +1036,9 @@ __global__ void __launch_bounds__(1024) st_segments_kernel(uint2* __restrict__ s
   __syncthreads();
   for (int base = 0; base < S; base += 1024) {
     const int s = base + tid;
-    unsigned cnt = 0u;
-    if (s < S) {
-      const uint2 r = st_ranges[s];
-      cnt = (r.y - r.x + kSeg - 1) / kSeg;
-    }
+    uint2 r = make_uint2(0u, 0u);
+    if (s < S) r = st_ranges[s];
+    const unsigned cnt = (r.y - r.x + kSeg - 1) / kSeg;
     unsigned incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1030,105 +1058,35 @@ __global__ void __launch_bounds__(1024) st_segments_kernel(uint2* __restrict__ s
       s_w[lane] = ti - t;
     }
     __syncthreads();
-    if (s < S) seg_first[s] = s_carry + s_w[w] + incl - cnt;
+    const unsigned first = s_carry + s_w[w] + incl - cnt;
+    if (s < S) {
+      seg_first[s] = first;
+      const CamInfo& c = ct.c[view_of_st(ct, s)];
+      const int sl = s - c.st_off;
+      const int ox = (sl % c.STX) * kSuperTile, oy = (sl / c.STX) * kSuperTile;
+      s_seg[tid] = Segment{r.x, r.y, c.tile_off + oy * c.TX + ox,
+                           (unsigned)c.TX | (unsigned)min(kSuperTile, c.TX - ox) << 16 |
+                               (unsigned)min(kSuperTile, c.TY - oy) << 20};
+    }
+    s_first[tid] = first;
     __syncthreads();
-    if (tid == 1023) s_carry += s_w[31] + incl;
+    if (tid == 1023) s_carry = first + cnt;
+    // the segments of these super-tiles: a warp per super-tile
+    for (int k = w; k < 1024 && base + k < S; k += 32) {
+      const Segment sg = s_seg[k];
+      const unsigned n = (sg.e - sg.b + kSeg - 1) / kSeg, g0 = s_first[k];
+      for (unsigned j = lane; j < n; j += 32) {
+        const unsigned b = sg.b + j * (unsigned)kSeg;
+        segs[g0 + j] = Segment{b, min(sg.e, b + (unsigned)kSeg), sg.tile, sg.shape};
+        if (seg_st) seg_st[g0 + j] = (unsigned)(base + k);
+      }
+    }
     __syncthreads();
   }
   if (tid == 0) {
     seg_first[S] = s_carry;
     *n_seg = (long long)s_carry;
   }
-  __syncthreads();
-  // the super-tile of every segment: a warp per super-tile
-  for (int s = w; s < S; s += 32) {
-    const unsigned g0 = seg_first[s], g1 = seg_first[s + 1];
-    for (unsigned g = g0 + lane; g < g1; g += 32) seg_st[g] = (unsigned)s;
-  }
-}
-
-// Rows [b, e) of segment g of super-tile s, its view and tile origin.
-struct SegInfo {
-  unsigned b, e;
-  int view, ox, oy;
-};
-
-__device__ __forceinline__ SegInfo seg_info(long long g, const uint2* __restrict__ st_ranges,
-                                            const unsigned* __restrict__ seg_first,
-                                            const unsigned* __restrict__ seg_st,
-                                            const CamTable& ct) {
-  SegInfo si;
-  const int s = (int)seg_st[g];
-  const uint2 rg = st_ranges[s];
-  si.b = rg.x + (unsigned)(g - seg_first[s]) * (unsigned)kSeg;
-  si.e = min(rg.y, si.b + (unsigned)kSeg);
-  si.view = view_of_st(ct, s);
-  const CamInfo& c = ct.c[si.view];
-  const int sl = s - c.st_off;
-  si.ox = (sl % c.STX) * kSuperTile;
-  si.oy = (sl / c.STX) * kSuperTile;
-  return si;
-}
-
-// Ballots of a warp's 32 rows (one per lane) over the rows and the columns of
-// an 8x8 super-tile: B[r] = lanes whose rect covers tile row r, X[c] = lanes
-// whose rect covers tile column c; the lanes covering tile (r, c) are
-// B[r] & X[c].  d = x0 | x1 << 4 | y0 << 8 | y1 << 12 (0: no tile).
-// The descriptor's rows and columns as 8-bit masks (bit k: k in [lo, hi)).
-__device__ __forceinline__ unsigned desc_rows(unsigned d) {
-  return ((1u << ((d >> 12) & 15u)) - 1u) & ~((1u << ((d >> 8) & 15u)) - 1u);
-}
-__device__ __forceinline__ unsigned desc_cols(unsigned d) {
-  return ((1u << ((d >> 4) & 15u)) - 1u) & ~((1u << (d & 15u)) - 1u);
-}
-
-// MASKS: each ballot tests one bit of the rect's 8-bit row or column mask
-// (st_emit_kernel: 1117 -> 1079 us on cfg3); otherwise two comparisons
-// (st_count_kernel: 245 us, against 291 us with the masks, measured
-// back to back in one session).
-template <bool MASKS>
-__device__ __forceinline__ void rect_ballots(unsigned d, unsigned B[8], unsigned X[8]) {
-  if (MASKS) {
-    const unsigned rm = desc_rows(d), cm = desc_cols(d);
-#pragma unroll
-    for (unsigned r = 0; r < 8; ++r) {
-      B[r] = __ballot_sync(0xffffffffu, (rm >> r) & 1u);
-      X[r] = __ballot_sync(0xffffffffu, (cm >> r) & 1u);
-    }
-  } else {
-    const unsigned x0 = d & 15u, x1 = (d >> 4) & 15u, y0 = (d >> 8) & 15u, y1 = (d >> 12) & 15u;
-#pragma unroll
-    for (unsigned r = 0; r < 8; ++r) {
-      B[r] = __ballot_sync(0xffffffffu, y0 <= r && r < y1);
-      X[r] = __ballot_sync(0xffffffffu, x0 <= r && r < x1);
-    }
-  }
-}
-
-// Counts of the warp's rows covering tiles `lane` and `lane + 32` of the
-// super-tile (tile b = 8 row + column).
-// The lanes of the warp's rows covering tiles `lane` and `lane + 32`.
-__device__ __forceinline__ void lane_tile_masks(const unsigned B[8], const unsigned X[8],
-                                                int lane, unsigned& m0, unsigned& m1) {
-  const int r = lane >> 3, c = lane & 7;
-  unsigned b0 = B[0], b1 = B[4], x = X[0];
-#pragma unroll
-  for (int k = 1; k < 4; ++k) {
-    b0 = r == k ? B[k] : b0;
-    b1 = r == k ? B[k + 4] : b1;
-  }
-#pragma unroll
-  for (int k = 1; k < 8; ++k) x = c == k ? X[k] : x;
-  m0 = b0 & x;
-  m1 = b1 & x;
-}
-
-__device__ __forceinline__ void lane_tile_counts(const unsigned B[8], const unsigned X[8],
-                                                 int lane, unsigned& c0, unsigned& c1) {
-  unsigned m0, m1;
-  lane_tile_masks(B, X, lane, m0, m1);
-  c0 = __popc(m0);
-  c1 = __popc(m1);
 }
 
 // Rect of row `row` inside the super-tile with tile origin (ox, oy), as a
@@ -1136,56 +1094,83 @@ __device__ __forceinline__ void lane_tile_counts(const unsigned B[8], const unsi
 __device__ __forceinline__ unsigned st_desc(const int* __restrict__ rect, unsigned row, int N,
                                             const CamTable& ct, int ox, int oy) {
   const int4 r = view_rect(rect, row, N, ct);
-  const int x0 = max(r.x - ox, 0), x1 = min(r.z - ox, kSuperTile);
-  const int y0 = max(r.y - oy, 0), y1 = min(r.w - oy, kSuperTile);
-  if (x1 <= x0 || y1 <= y0) return 0u;  // (not produced by consistent inputs)
-  return (unsigned)(x0 | (x1 << 4) | (y0 << 8) | (y1 << 12));
+  const int x0 = r.x - ox, x1 = r.z - ox, y0 = r.y - oy, y1 = r.w - oy;
+  if (x0 >= kSuperTile || y0 >= kSuperTile || x1 <= 0 || y1 <= 0 || x1 <= x0 || y1 <= y0)
+    return 0u;  // (not produced by consistent inputs)
+  return rect_masks(x0, x1, y0, y1);
 }
 
-// Per segment: the count of rows covering each of the 64 tiles (warp ballots,
-// summed over the CTA's warps).  The rect descriptors travel in the items'
-// keys (bits 16-31) when `packed`; otherwise they are formed here from the
-// rects and stored in desc for the expansion.
+// Per segment: the count of rows covering each of the 64 tiles.  The count of
+// tile (r, c) is the sum over the rows of [covers tile row r] [covers tile
+// column c]: an 8 x 8 product of two 0/1 matrices over up to 1024 rows, which
+// the tensor cores take 16 rows at a time (mma.sync m16n8k16 on bf16 with
+// FP32 sums: whole numbers of at most 4 * 1024, exact).  A lane needs, of four
+// items, the bits of one tile row and one tile column; a set bit moved to bit
+// 14 of its 16-bit half is bf16 2.0, so every covering row adds 4.  The 8
+// unused rows of A are zero.  About 11 instructions per 16 items; counting by
+// row and column ballots took about 60 and was bound by issue (45 M items:
+// 258 -> 97 us; what is left is the latency of the key loads).
+// The descriptors travel in the items' keys (bits 16-31) when `packed`;
+// otherwise they are formed here from the rects and stored in desc for the
+// expansion.
+__device__ __forceinline__ void mma_count(float d[4], unsigned a0, unsigned a2, unsigned b0,
+                                          unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %5}, "
+      "{%7, %8}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a0), "r"(0u), "r"(a2), "r"(b0), "r"(b1));
+}
+
 __global__ void __launch_bounds__(256) st_count_kernel(
     const unsigned* __restrict__ sp_keys, const unsigned* __restrict__ sp_rows,
-    const uint2* __restrict__ st_ranges, const unsigned* __restrict__ seg_first,
-    const unsigned* __restrict__ seg_st, const long long* __restrict__ n_seg, int packed,
-    const int* __restrict__ rect, int N, const CamTable ct, unsigned* __restrict__ desc,
-    unsigned* __restrict__ hist) {
+    const Segment* __restrict__ segs, const unsigned* __restrict__ seg_st,
+    const long long* __restrict__ n_seg, int packed, const int* __restrict__ rect, int N,
+    const CamTable ct, unsigned* __restrict__ desc, unsigned* __restrict__ hist) {
   __shared__ unsigned s_cnt[8][64];
+  constexpr int kPer = kSeg / 8;  // items of a warp
+  __shared__ __align__(16) unsigned short s_desc[8][kPer];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int t = lane & 3, q = lane >> 2;  // the lane's four items of 16; its tile row and column
+  const int sr = 14 - q, sc = 6 - q;      // moves its bits to bit 14 (a rotation by -1 for column 7)
   const long long G = *n_seg;
   for (long long g = blockIdx.x; g < G; g += gridDim.x) {
-    const SegInfo si = seg_info(g, st_ranges, seg_first, seg_st, ct);
-    unsigned a0 = 0u, a1 = 0u;
-    // a segment holds at most kSeg = 4 x 256 items: each warp's (up to) four
-    // groups of 32 are loaded before any is counted
-    constexpr int kGroups = kSeg / 256;
-    unsigned dd[kGroups];
+    const Segment si = load_segment(segs, g);
+    int ox = 0, oy = 0;
+    if (!packed) {
+      const int s = (int)seg_st[g];
+      const CamInfo& c = ct.c[view_of_st(ct, s)];
+      ox = ((s - c.st_off) % c.STX) * kSuperTile;
+      oy = ((s - c.st_off) / c.STX) * kSuperTile;
+    }
+    unsigned dd[kPer / 32];
 #pragma unroll
-    for (int k = 0; k < kGroups; ++k) {
-      const unsigned i = si.b + 32u * w + 256u * k + lane;
+    for (int k = 0; k < kPer / 32; ++k) {
+      const unsigned i = si.b + kPer * w + 32u * k + lane;
       dd[k] = 0u;
       if (i < si.e) {
         if (packed) {
           dd[k] = sp_keys[i] >> 16;
         } else {
-          dd[k] = st_desc(rect, sp_rows[i], N, ct, si.ox, si.oy);
-          desc[i] = dd[k];
+          dd[k] = st_desc(rect, sp_rows[i], N, ct, ox, oy);
+          desc[i] = dd[k] << 16;
         }
       }
     }
 #pragma unroll
-    for (int k = 0; k < kGroups; ++k) {
-      if (si.b + 32u * w + 256u * k >= si.e) break;  // warp-uniform
-      unsigned B[8], X[8], n0, n1;
-      rect_ballots<false>(dd[k], B, X);
-      lane_tile_counts(B, X, lane, n0, n1);
-      a0 += n0;
-      a1 += n1;
+    for (int k = 0; k < kPer / 32; ++k) s_desc[w][32 * k + lane] = (unsigned short)dd[k];
+    __syncwarp();
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < kPer / 16; ++j) {
+      const uint2 v = *reinterpret_cast<const uint2*>(&s_desc[w][16 * j + 4 * t]);
+      mma_count(d, (v.x << sr) & 0x40004000u, (v.y << sr) & 0x40004000u,
+                __funnelshift_l(v.x, v.x, sc) & 0x40004000u,
+                __funnelshift_l(v.y, v.y, sc) & 0x40004000u);
     }
-    s_cnt[w][lane] = a0;
-    s_cnt[w][lane + 32] = a1;
+    // d[0], d[1]: tile row q, columns 2t and 2t + 1
+    *reinterpret_cast<uint2*>(&s_cnt[w][8 * q + 2 * t]) =
+        make_uint2((unsigned)(0.25f * d[0]), (unsigned)(0.25f * d[1]));
     __syncthreads();
     if (tid < 64) {
       unsigned sum = 0u;
@@ -1197,35 +1182,52 @@ __global__ void __launch_bounds__(256) st_count_kernel(
   }
 }
 
-// One CTA per super-tile, 16 groups x 64 tiles: exclusive scan of every
-// tile's counts over the super-tile's segments (in place), and the tile's
-// total list length.
+// One CTA per super-tile, 64 groups of segments x 16 quads of tiles: exclusive
+// scan of every tile's counts over the super-tile's segments (in place), and
+// the tile's total list length.
 __device__ __forceinline__ void tile_scan_dev(const unsigned* __restrict__ tile_cnt, int T,
                                               unsigned* __restrict__ tile_start,
                                               unsigned* __restrict__ ranges);
 
+__device__ __forceinline__ uint4 add4(uint4 a, uint4 b) {
+  return make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
 __global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* __restrict__ seg_first,
                                                        const CamTable ct,
-                                                       unsigned* __restrict__ hist,
+                                                       uint4* __restrict__ hist,
                                                        unsigned* __restrict__ tile_cnt,
                                                        unsigned long long* __restrict__ arrive,
                                                        unsigned* __restrict__ tile_start,
                                                        unsigned* __restrict__ ranges) {
-  __shared__ unsigned s_part[16][64];
+  __shared__ uint4 s_part[64][16];
   const int s = blockIdx.x;
-  const int k = threadIdx.x >> 6, bt = threadIdx.x & 63;
+  const int k = threadIdx.x >> 4, q = threadIdx.x & 15;
   const unsigned g0 = seg_first[s], L = seg_first[s + 1] - g0;
-  const unsigned per = (L + 15u) / 16u;
+  const unsigned per = (L + 63u) / 64u;
   const unsigned a = min(L, (unsigned)k * per), e = min(L, a + per);
-  unsigned sum = 0u;
-  for (unsigned g = a; g < e; ++g) sum += hist[(long long)(g0 + g) * 64 + bt];
-  s_part[k][bt] = sum;
+  constexpr unsigned kBatch = 4;  // counts loaded together
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  uint4 sum = zero;
+  for (unsigned g = a; g < e; g += kBatch) {
+    const uint4* h = hist + (long long)(g0 + g) * 16 + q;
+    uint4 x[kBatch];
+#pragma unroll
+    for (unsigned j = 0; j < kBatch; ++j) x[j] = g + j < e ? h[16 * j] : zero;
+#pragma unroll
+    for (unsigned j = 0; j < kBatch; ++j) sum = add4(sum, x[j]);
+  }
+  s_part[k][q] = sum;
   __syncthreads();
-  if (k == 0) {
+  if (threadIdx.x < 64) {
+    // tile bt: exclusive scan over the 64 groups
+    const int bt = threadIdx.x;
+    unsigned* p = &s_part[0][0].x + bt;
     unsigned run = 0u;
-    for (int kk = 0; kk < 16; ++kk) {
-      const unsigned x = s_part[kk][bt];
-      s_part[kk][bt] = run;
+#pragma unroll 16
+    for (int kk = 0; kk < 64; ++kk) {
+      const unsigned x = p[64 * kk];
+      p[64 * kk] = run;
       run += x;
     }
     const CamInfo& c = ct.c[view_of_st(ct, s)];
@@ -1235,144 +1237,207 @@ __global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* __restric
     if (tx < c.TX && ty < c.TY) tile_cnt[c.tile_off + ty * c.TX + tx] = run;
   }
   __syncthreads();
-  unsigned run = s_part[k][bt];
-  for (unsigned g = a; g < e; ++g) {
-    unsigned* h = hist + (long long)(g0 + g) * 64 + bt;
-    const unsigned x = *h;
-    *h = run;
-    run += x;
+  uint4 run = s_part[k][q];
+  for (unsigned g = a; g < e; g += kBatch) {
+    uint4* h = hist + (long long)(g0 + g) * 16 + q;
+    uint4 x[kBatch];
+#pragma unroll
+    for (unsigned j = 0; j < kBatch; ++j) x[j] = g + j < e ? h[16 * j] : zero;
+#pragma unroll
+    for (unsigned j = 0; j < kBatch; ++j) {
+      if (g + j < e) h[16 * j] = run;
+      run = add4(run, x[j]);
+    }
   }
   if (last_block_arrives(arrive, gridDim.x)) tile_scan_dev(tile_cnt, ct.total_tiles, tile_start, ranges);
 }
 
 // Exclusive scan of the list lengths over all T tiles (one CTA of 1024
-// threads): list starts, and ranges [start, end) ((0, 0) for an empty list).
-// Run by the last CTA of st_scan_kernel (tile_cnt read through L2).
+// threads, 4 consecutive tiles per thread and round): list starts, and ranges
+// [start, end) ((0, 0) for an empty list).  Run by the last CTA of
+// st_scan_kernel (tile_cnt read through L2; it is padded to whole 16 bytes).
 __device__ __forceinline__ void tile_scan_dev(const unsigned* __restrict__ tile_cnt, int T,
                                               unsigned* __restrict__ tile_start,
                                               unsigned* __restrict__ ranges) {
-  __shared__ unsigned s_w[32];
-  __shared__ unsigned s_carry;
+  __shared__ unsigned s_w[2][32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (tid == 0) s_carry = 0u;
-  __syncthreads();
-  for (int base = 0; base < T; base += 1024) {
-    const int t = base + tid;
-    const unsigned cnt = t < T ? __ldcg(tile_cnt + t) : 0u;
-    unsigned incl = cnt;
+  unsigned carry = 0u;
+  int buf = 0;
+  for (int base = 0; base < T; base += 4096, buf ^= 1) {
+    const int t = base + 4 * tid;
+    unsigned c[4] = {0u, 0u, 0u, 0u};
+    if (t < T) {
+      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(tile_cnt + t));
+      c[0] = v.x;
+      c[1] = t + 1 < T ? v.y : 0u;
+      c[2] = t + 2 < T ? v.z : 0u;
+      c[3] = t + 3 < T ? v.w : 0u;
+    }
+    const unsigned sum = c[0] + c[1] + c[2] + c[3];
+    unsigned incl = sum;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += y;
     }
-    if (lane == 31) s_w[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-      const unsigned x = s_w[lane];
-      unsigned xi = x;
+    if (lane == 31) s_w[buf][w] = incl;
+    __syncthreads();  // (two buffers: one barrier per round)
+    unsigned wt = s_w[buf][lane];
+    const unsigned own = wt;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, xi, o);
-        if (lane >= o) xi += y;
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, wt, o);
+      if (lane >= o) wt += y;
+    }
+    unsigned start = carry + __shfl_sync(0xffffffffu, wt - own, w) + incl - sum;
+    carry += __shfl_sync(0xffffffffu, wt, 31);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (t + j < T) {
+        tile_start[t + j] = start;
+        ranges[2ll * (t + j)] = c[j] ? start : 0u;
+        ranges[2ll * (t + j) + 1] = c[j] ? start + c[j] : 0u;
+        start += c[j];
       }
-      s_w[lane] = xi - x;
     }
-    __syncthreads();
-    const unsigned start = s_carry + s_w[w] + incl - cnt;
-    if (t < T) {
-      tile_start[t] = start;
-      ranges[2ll * t] = cnt ? start : 0u;
-      ranges[2ll * t + 1] = cnt ? start + cnt : 0u;
-    }
-    __syncthreads();
-    if (tid == 1023) s_carry = start + cnt;
-    __syncthreads();
   }
 }
 
-// Expansion: per segment, rows in chunks of 256 (one per thread, 8 warps of
-// 32 consecutive rows).  Each warp takes its row and column ballots over the
-// super-tile, counts its rows per tile, a prefix over the warps and the
-// running list positions give every warp its first slot per tile, and the
-// lanes covering tile (r, c) (B[r] & X[c]) write their rows at consecutive
-// slots, so every list receives its rows in the segment's (depth) order with
-// coalesced stores.
+// Inclusive warp scan of four byte fields each (sums stay below 256).
+__device__ __forceinline__ unsigned warp_scan_bytes(unsigned x) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
+        "shfl.sync.up.b32 t|p, %0, %1, 0x0, 0xffffffff;\n\t"
+        "@p add.u32 %0, %0, t;\n\t}"
+        : "+r"(x)
+        : "r"(o));
+  return x;
+}
+
+// Bits 0..3 of x as the low bits of four bytes.
+__device__ __forceinline__ unsigned spread4(unsigned x) {
+  return ((x & 15u) * 0x00204081u) & 0x01010101u;
+}
+
+// Address of the list slot n after the one at address a (one instruction).
+__device__ __forceinline__ unsigned long long slot_after(unsigned long long a, unsigned n) {
+  unsigned long long r;
+  asm("mad.wide.u32 %0, %1, 4, %2;" : "=l"(r) : "r"(n), "l"(a));
+  return r;
+}
+
+// Expansion.  Per segment, the items (row, descriptor) are staged in shared
+// memory and warp r takes tile row r of the super-tile: it walks the items in
+// (depth) order, keeps those that cover its tile row in a ring of its own,
+// and whenever 64 of them are there writes them out to the row's 8 lists, two
+// consecutive items per lane: the ranks of all 8 columns come from one warp
+// scan of byte counters.  (Ranks from ballots take a population count per
+// column and 32 rows, which runs at an eighth of the issue rate and bound this
+// kernel.)  The next slots of the 8 lists stay in registers, so no barrier and
+// no prefix over the warps is needed between the segment's staging and its
+// end, and only the rows that cover the tile row reach the 8 column steps.
+//
+// What bounds it: instruction issue while the lists fit in L2 (21 M pairs: 58
+// -> 43 us against the ballot form), the stores' way to DRAM beyond (351 M
+// pairs: 590 -> 420 us, 3.4 TB/s).  CTAs per SM the register budget targets: 4;
+// left to itself the compiler takes 32 registers, which recomputes addresses
+// (351 M pairs: 567 us).  Grid: up to 64 CTAs per SM, so that most CTAs write
+// one segment and they run in list order (500 us with 8 per SM, whose rounds
+// drift apart and leave a partly empty last one).
+constexpr int kEmitCtas = 4;
+constexpr long long kEmitGrid = 152ll * 64;
 template <bool KEYS>
-__global__ void __launch_bounds__(256) st_emit_kernel(
+__global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
     const unsigned* __restrict__ sp_keys, const unsigned* __restrict__ sp_rows,
-    const unsigned* __restrict__ desc, int packed, const uint2* __restrict__ st_ranges,
-    const unsigned* __restrict__ seg_first, const unsigned* __restrict__ seg_st,
+    const unsigned* __restrict__ desc, int packed, const Segment* __restrict__ segs,
     const long long* __restrict__ n_seg, const unsigned* __restrict__ hist,
-    const unsigned* __restrict__ tile_start, const CamTable ct, const float* __restrict__ depth,
+    const unsigned* __restrict__ tile_start, const float* __restrict__ depth,
     unsigned* __restrict__ out_vals, unsigned long long* __restrict__ out_keys, long long cap) {
-  __shared__ unsigned s_run[64];                   // next list slot per tile of the super-tile
-  __shared__ unsigned s_cnt[8][64];                // per-warp counts per tile
-  __shared__ __align__(16) unsigned s_pos[8][64];  // per-warp first slot per tile
-  __shared__ int s_tile[64];                       // global tile id (-1 outside the view)
+  constexpr unsigned kRing = 128;  // at most 63 waiting + 32 new items
+  __shared__ uint2 s_item[kSeg];                     // row, descriptor
+  __shared__ __align__(16) uint2 s_ring[8][kRing];   // row, columns covered
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const long long G = *n_seg;
+  const unsigned* __restrict__ keys = packed ? sp_keys : desc;
   for (long long g = blockIdx.x; g < G; g += gridDim.x) {
-    const SegInfo si = seg_info(g, st_ranges, seg_first, seg_st, ct);
-    __syncthreads();  // the previous segment's readers of s_run / s_tile are done
-    if (tid < 64) {
-      const CamInfo& c = ct.c[si.view];
-      const int tx = si.ox + (tid & 7), ty = si.oy + (tid >> 3);
-      const bool in = tx < c.TX && ty < c.TY;
-      const int t = in ? c.tile_off + ty * c.TX + tx : -1;
-      s_tile[tid] = t;
-      s_run[tid] = in ? tile_start[t] + hist[g * 64 + tid] : 0u;
+    const Segment si = load_segment(segs, g);
+    const int n = (int)(si.e - si.b);
+    constexpr int kPer = kSeg / 256;
+    uint2 it[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int i = tid + 256 * k;
+      it[k] = make_uint2(0u, 0u);
+      if (i < n) it[k] = make_uint2(sp_rows[si.b + i], keys[si.b + i] >> 16);
     }
-    for (unsigned c0 = si.b; c0 < si.e; c0 += 256) {
-      const unsigned i = c0 + tid;
-      unsigned d = 0u, row = 0u;
-      if (i < si.e) {
-        d = packed ? (sp_keys[i] >> 16) : desc[i];
-        row = sp_rows[i];
+    // the first slots of this warp's tiles (lane c: column c)
+    int tile = -1;
+    unsigned first = 0u;
+    if (lane < si.cols() && w < si.rows()) {
+      tile = si.tile + w * si.tx() + lane;
+      first = tile_start[tile] + hist[g * 64 + 8 * w + lane];
+    }
+    __syncthreads();  // the previous segment's items have been read
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) s_item[tid + 256 * k] = it[k];
+    __syncthreads();
+    unsigned long long run[8];  // address of the next slot of each list
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      run[k] = slot_after(reinterpret_cast<unsigned long long>(out_vals),
+                          __shfl_sync(0xffffffffu, first, k));
+    auto store = [&](unsigned long long at, unsigned row, int tk) {
+      unsigned* p = reinterpret_cast<unsigned*>(at);
+      if (!GS_IN_BOUNDS(p - out_vals, cap, 201)) return;
+      *p = row;
+      if (KEYS)
+        out_keys[p - out_vals] =
+            ((unsigned long long)(unsigned)tk << 32) | __float_as_uint(depth[row]);
+    };
+    // writes out the first `m` (at most 64) of the 64 items from ring position `at`
+    auto flush = [&](unsigned at, unsigned m) {
+      uint4 e = *reinterpret_cast<const uint4*>(&s_ring[w][(at + 2 * lane) & (kRing - 1)]);
+      if (2u * lane >= m) e.y = 0u;
+      if (2u * lane + 1u >= m) e.w = 0u;
+      const unsigned a0 = spread4(e.y), a1 = spread4(e.y >> 4);
+      const unsigned t0 = a0 + spread4(e.w), t1 = a1 + spread4(e.w >> 4);
+      const unsigned i0 = warp_scan_bytes(t0), i1 = warp_scan_bytes(t1);
+      const unsigned x0 = i0 - t0, x1 = i1 - t1;    // ranks of the lane's first item
+      const unsigned y0 = x0 + a0, y1 = x1 + a1;    // and of its second
+      const unsigned n0 = __shfl_sync(0xffffffffu, i0, 31), n1 = __shfl_sync(0xffffffffu, i1, 31);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const unsigned sel = 0x4440u | (k & 3);
+        int tk = 0;
+        if (KEYS) tk = __shfl_sync(0xffffffffu, tile, k);
+        if (e.y & (1u << k))
+          store(slot_after(run[k], __byte_perm(k < 4 ? x0 : x1, 0u, sel)), e.x, tk);
+        if (e.w & (1u << k))
+          store(slot_after(run[k], __byte_perm(k < 4 ? y0 : y1, 0u, sel)), e.z, tk);
+        run[k] = slot_after(run[k], __byte_perm(k < 4 ? n0 : n1, 0u, sel));
       }
-      unsigned B[8], X[8], n0, n1;
-      rect_ballots<true>(d, B, X);
-      lane_tile_counts(B, X, lane, n0, n1);
-      s_cnt[w][lane] = n0;
-      s_cnt[w][lane + 32] = n1;
-      __syncthreads();
-      if (tid < 64) {
-        unsigned run = s_run[tid];
-#pragma unroll
-        for (int ww = 0; ww < 8; ++ww) {
-          s_pos[ww][tid] = run;
-          run += s_cnt[ww][tid];
-        }
-        s_run[tid] = run;
-      }
-      __syncthreads();
-      // this lane's rect in the super-tile, and the column ballots restricted
-      // to the lanes before it (ranks by population counts, no branches per
-      // tile: in the dense case nearly every tile has a covering row)
-      const unsigned rows = desc_rows(d), cols = desc_cols(d);
-      unsigned Xl[8];
-#pragma unroll
-      for (int c = 0; c < 8; ++c) Xl[c] = X[c] & lt;
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        if (B[r] == 0u) continue;  // warp-uniform
-        const uint4 pa = *reinterpret_cast<const uint4*>(&s_pos[w][8 * r]);
-        const uint4 pb = *reinterpret_cast<const uint4*>(&s_pos[w][8 * r + 4]);
-        const unsigned sp[8] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w};
-        const unsigned cov = ((rows >> r) & 1u) ? cols : 0u;
-#pragma unroll
-        for (unsigned c = 0; c < 8; ++c) {
-          // this lane covers tile (r, c): its rank among the covering lanes
-          const unsigned pos = sp[c] + __popc(B[r] & Xl[c]);
-          if ((cov & (1u << c)) && GS_IN_BOUNDS(pos, cap, 201)) {
-            out_vals[pos] = row;
-            if (KEYS)
-              out_keys[pos] = ((unsigned long long)(unsigned)s_tile[8 * r + c] << 32) |
-                              __float_as_uint(depth[row]);
-          }
-        }
+    };
+    unsigned head = 0u, cnt = 0u;  // ring: `cnt` items from position `head`
+    for (int b = 0; b < n; b += 32) {
+      const uint2 e = s_item[b + lane];  // (items past n: descriptor 0)
+      const bool in = (e.y >> w) & 1u;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) s_ring[w][(head + cnt + __popc(m & lt)) & (kRing - 1)] = make_uint2(e.x, e.y >> 8);
+      cnt += __popc(m);
+      if (cnt >= 64u) {
+        __syncwarp();
+        flush(head, 64u);
+        head += 64u;
+        cnt -= 64u;
+        __syncwarp();
       }
     }
+    __syncwarp();
+    if (cnt) flush(head, cnt);
+    __syncwarp();
   }
 }
 
@@ -1398,6 +1463,7 @@ struct Workspace {
   unsigned* hist;                  // radix histograms
   unsigned* st_ranges;             // [2 * super-tiles] rows of each super-tile
   unsigned* seg_first;             // [super-tiles + 1] first segment of each super-tile
+  Segment* segs;                   // the segments
   unsigned* seg_st;                // super-tile of every segment
   unsigned* seg_hist;              // [segments][64] per-tile counts, then bases
   unsigned* tile_cnt;              // [tiles] list lengths
@@ -1462,9 +1528,10 @@ Workspace carve(void* base, long long n_rows, long long cap, long long tiles) {
   w.hist = reinterpret_cast<unsigned*>(take(radix_hist_bytes()));
   w.st_ranges = reinterpret_cast<unsigned*>(take(8ull * (tiles + 1)));
   w.seg_first = reinterpret_cast<unsigned*>(take(4ull * (tiles + 2)));
+  w.segs = reinterpret_cast<Segment*>(take(sizeof(Segment) * ms));
   w.seg_st = reinterpret_cast<unsigned*>(take(4ull * ms));
   w.seg_hist = reinterpret_cast<unsigned*>(take(4ull * 64 * ms));
-  w.tile_cnt = reinterpret_cast<unsigned*>(take(4ull * (tiles + 1)));
+  w.tile_cnt = reinterpret_cast<unsigned*>(take(4ull * (tiles + 4)));
   w.tile_start = reinterpret_cast<unsigned*>(take(4ull * (tiles + 1)));
   w.bytes = off;
   return w;
@@ -1656,28 +1723,28 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     count_launches(1);
   }
   st_segments_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<uint2*>(w.st_ranges), S, st_totals,
-                                         q_eff, w.seg_first, w.seg_st, n_seg);
+                                         q_eff, w.seg_first, w.segs,
+                                         packed ? nullptr : w.seg_st, ct, n_seg);
   const unsigned gs = (unsigned)std::min<long long>(max_segments(q_bound, S), 152ll * 8);
-  st_count_kernel<<<gs, 256, 0, st>>>(sp_keys, sp_rows,
-                                      reinterpret_cast<const uint2*>(w.st_ranges), w.seg_first,
-                                      w.seg_st, n_seg, packed, proj->rect, N, ct, desc,
-                                      w.seg_hist);
-  st_scan_kernel<<<(unsigned)S, 1024, 0, st>>>(w.seg_first, ct, w.seg_hist, w.tile_cnt,
-                                                arrive + 2, w.tile_start, ranges);
+  st_count_kernel<<<gs, 256, 0, st>>>(sp_keys, sp_rows, w.segs, w.seg_st, n_seg, packed,
+                                      proj->rect, N, ct, desc, w.seg_hist);
+  st_scan_kernel<<<(unsigned)S, 1024, 0, st>>>(w.seg_first, ct,
+                                               reinterpret_cast<uint4*>(w.seg_hist), w.tile_cnt,
+                                               arrive + 2, w.tile_start, ranges);
   // 7. every row into the lists of the tiles it covers, in depth order
   {
     const int e = stage_event(GS_STAGE_EXPANSION, false, st);
     if (e != GS_OK) return e;
   }
+  const unsigned ge = (unsigned)std::min<long long>(max_segments(q_bound, S), kEmitGrid);
   if (sorted_keys)
-    st_emit_kernel<true><<<gs, 256, 0, st>>>(
-        sp_keys, sp_rows, desc, packed, reinterpret_cast<const uint2*>(w.st_ranges), w.seg_first,
-        w.seg_st, n_seg, w.seg_hist, w.tile_start, ct, proj->depth, sorted_vals, sorted_keys,
-        cap);
+    st_emit_kernel<true><<<ge, 256, 0, st>>>(sp_keys, sp_rows, desc, packed, w.segs, n_seg,
+                                             w.seg_hist, w.tile_start, proj->depth, sorted_vals,
+                                             sorted_keys, cap);
   else
-    st_emit_kernel<false><<<gs, 256, 0, st>>>(
-        sp_keys, sp_rows, desc, packed, reinterpret_cast<const uint2*>(w.st_ranges), w.seg_first,
-        w.seg_st, n_seg, w.seg_hist, w.tile_start, ct, proj->depth, sorted_vals, nullptr, cap);
+    st_emit_kernel<false><<<ge, 256, 0, st>>>(sp_keys, sp_rows, desc, packed, w.segs, n_seg,
+                                              w.seg_hist, w.tile_start, proj->depth, sorted_vals,
+                                              nullptr, cap);
   {
     const int e = stage_event(GS_STAGE_EXPANSION, true, st);
     if (e != GS_OK) return e;
