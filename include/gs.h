@@ -126,8 +126,9 @@ typedef struct {
     void* ev_begin;                /* optional cudaEvent_t recorded on the stream right before the
                                       blending kernel (for live per-kernel timing) */
     void* ev_end;                  /* optional cudaEvent_t recorded right after it */
-    int pixels_per_thread;         /* 1, 2 or 4 pixels of a column per thread (0 = 2); 4 only
-                                      with 16-pixel tiles */
+    int pixels_per_thread;         /* 1, 2 or 4 pixels of a column per thread (0 = 2, or 1 where
+                                      the views hold too few 16-pixel tiles to fill the GPU);
+                                      4 only with 16-pixel tiles */
     int batch;                     /* list entries staged in shared memory per batch: 256, or
                                       128 with F32 records and 16-pixel tiles (0 = 256) */
     void* zero_beside;             /* gs_render_fwd (optional): device memory that the blending

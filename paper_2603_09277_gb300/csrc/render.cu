@@ -3,9 +3,8 @@
 //
 // One CTA owns one tile of TS x TS pixels (TS = 16, or 8 as in the paper's
 // runs).  A thread owns PPT (1, 2 or 4; 1 or 2 for 8x8 tiles) vertically
-// adjacent pixels of one column, so a warp covers a TS x (32 / TS) PPT block
-// and the column-dependent part of every exponent is shared by the thread's
-// pixels.
+// adjacent pixels of one column, so a warp covers an 8 x 4 PPT block and the
+// column-dependent part of every exponent is shared by the thread's pixels.
 // The tile's list is streamed through shared memory in batches of 256
 // records (gathered with 16-byte vector loads) and every thread walks the
 // batch from shared memory (warp-broadcast reads).  The forward stops a CTA
@@ -23,8 +22,8 @@
 //   dL/dalpha_i = sum_ch g_ch (T_i c_i - S / (1 - alpha_i))
 //               + gH ((-ln w_i - 1) T_i + R / (1 - alpha_i))
 //   S += w_i c_i; R += (ln w_i + 1) w_i    (R starts at (ln T_N+1 + 1) T_N+1)
-//   (only g . S is needed, so it is carried instead of S: g . S += w_i g . c_i;
-//   R and gH are carried in base-2 units, R / ln 2 and gH ln 2)
+//   (only g . S - gH R is needed, so it is carried instead of S and R, see
+//   bwd_pair; L, R and gH are in base-2 units, R / ln 2 and gH ln 2)
 //   then with dd = dalpha alpha (where alpha is not clamped) and (dx, dy)
 //   the pixel centre minus the 2D mean: dsigma = dd / sigma,
 //   dconic = dd (-dx^2/2, -dx dy, -dy^2/2), dmean = dd conic (dx, dy).
@@ -62,9 +61,16 @@ constexpr unsigned kFull = 0xffffffffu;
 // so a finished or outside pixel never passes the alpha_min test again.
 constexpr float kFar = 1e30f;
 
+// A warp takes a block of 8 x 4 PPT pixels of the tile (8 columns, 4 thread
+// rows of PPT pixels each): 8 x 8 at two pixels per thread.  A square block is
+// met by fewer splats than a 16 x 4 strip of the same area.
 template <int TS, int PPT>
 struct TileGeom {
   static constexpr int kThreads = TS * TS / PPT;
+  static constexpr int kBlockH = 4 * PPT;      // block height in pixels
+  static constexpr int kCols = TS / 8;         // blocks per tile row
+  static constexpr int kRows = TS / kBlockH;   // blocks per tile column
+  static_assert(kCols * kRows * 32 == kThreads, "a block per warp");
   int view;
   long long pix0;   // global index of the thread's first pixel
   int W;            // view width (pixel stride of a row)
@@ -72,19 +78,20 @@ struct TileGeom {
   float rx;         // pixel-centre x relative to the tile origin
   float ry0;        // first pixel-centre y relative to the tile origin
   unsigned inside;  // bit k: pixel k lies in the image
-  float xmax;       // largest pixel-centre x of the tile inside the image (relative)
-  unsigned rows;    // bit r: tile row r lies in the image
+  float xmax, ymax; // largest pixel-centre x, y of the tile inside the image (relative)
 };
 
 template <int TS, int PPT>
 __device__ __forceinline__ TileGeom<TS, PPT> tile_geom(const CamTable& ct, int tile) {
-  TileGeom<TS, PPT> g;
+  using G = TileGeom<TS, PPT>;
+  G g;
   g.view = find_view_of_tile(ct, tile);
   const CamInfo& c = ct.c[g.view];
   const int local = tile - c.tile_off;
   const int tx = local % c.TX, ty = local / c.TX;
-  const int lx = threadIdx.x & (TS - 1);
-  const int ly0 = (threadIdx.x / TS) * PPT;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lx = (warp % G::kCols) * 8 + (lane & 7);
+  const int ly0 = (warp / G::kCols) * G::kBlockH + (lane >> 3) * PPT;
   const int px = tx * TS + lx, py0 = ty * TS + ly0;
   g.W = c.W;
   g.pix0 = c.pix_off + (long long)py0 * c.W + px;
@@ -97,59 +104,79 @@ __device__ __forceinline__ TileGeom<TS, PPT> tile_geom(const CamTable& ct, int t
   for (int k = 0; k < PPT; ++k)
     if (px < c.W && py0 + k < c.H) g.inside |= 1u << k;
   g.xmax = (float)(min(TS, c.W - tx * TS) - 1) + 0.5f;
-  const int nrow = min(TS, c.H - ty * TS);
-  g.rows = (1u << nrow) - 1u;
+  g.ymax = (float)(min(TS, c.H - ty * TS) - 1) + 0.5f;
   return g;
 }
 
-// Rows of the tile (bit r: pixel centres at tile-relative y = r + 0.5) in
-// which some pixel centre with x in [0.5, xmax] may pass the alpha_min test.
-// A pixel passes when e = L2S - p^2 - q^2 >= log2(alpha_min), that is when
-// p^2 + q^2 <= rho2 = L2S - log2(alpha_min).  Along one row p^2 + q^2 is a
-// convex quadratic in x; its least value over the segment is taken at the
-// stationary point clamped to the segment.  The limit is widened by a bound
-// on the FP32 rounding of this test and of the per-pixel exponent (32 times
-// the first-order estimate), so a row left out holds no pixel the per-pixel
-// test would blend, and skipping it leaves every output unchanged.
-template <int TS>
-__device__ __forceinline__ unsigned splat_rows(float mx, float my, float f11, float f21, float f22,
-                                               float L2S, float log2_amin, float xmax,
-                                               unsigned rows) {
+// The warps (bit w: block w of the tile) in whose block some pixel centre
+// inside the image may pass the alpha_min test.  A pixel passes when e = L2S -
+// p^2 - q^2 >= log2(alpha_min), that is when p^2 + q^2 <= rho2 = L2S -
+// log2(alpha_min), with p = f11 dx, q = f21 dx + f22 dy.  p^2 + q^2 is convex
+// with its minimum at the mean, so over a block's box of pixel centres its
+// least value lies, unless the mean is inside, on an edge that faces the mean:
+// the column xe of the box nearest to the mean (with the best y on it) or the
+// row ye nearest to it (with the best x).  Both candidates are points of the
+// box in any case, so the smaller of the two is the least value.  The limit is
+// widened by a bound on the FP32 rounding of this test and of the per-pixel
+// exponent (32 times the first-order estimate), so a block left out holds no
+// pixel the per-pixel test would blend, and skipping it leaves every output
+// unchanged.  (About half the work of testing each of the tile's 16 rows.)
+template <int TS, int PPT>
+__device__ __forceinline__ unsigned splat_blocks(float mx, float my, float f11, float f21,
+                                                 float f22, float L2S, float log2_amin, float xmax,
+                                                 float ymax) {
+  using G = TileGeom<TS, PPT>;
   const float rho2 = L2S - log2_amin;
   if (!(rho2 >= 0.f)) return 0u;  // e <= L2S < log2(alpha_min) everywhere
   const float rho = sqrtf(rho2);
-  const float x0 = 0.5f - mx, x1 = xmax - mx;
   const float X =
       (fabsf(f11) + fabsf(f21)) * ((float)TS + fabsf(mx)) + fabsf(f22) * ((float)TS + fabsf(my)) +
       rho;
   const float lim = rho2 + 0x1p-18f * (rho * X + rho2 + 8.f);
   const float a = __fmaf_rn(f11, f11, f21 * f21);
-  const float k = -f21 * f22 / a;  // stationary x of row dy is k dy
-  unsigned m = 0u;
-#pragma unroll 4
-  for (int r = 0; r < TS; ++r) {
-    const float dy = ((float)r + 0.5f) - my;
-    const float dx = fminf(fmaxf(k * dy, x0), x1);
-    const float pv = f11 * dx;
-    const float qv = __fmaf_rn(f21, dx, f22 * dy);
-    if (__fmaf_rn(pv, pv, qv * qv) <= lim) m |= 1u << r;
+  const float kx = -f21 * f22 / a;  // best x on the row dy: kx dy
+  const float ky = -f21 / f22;      // best y on the column dx: ky dx
+  float x0[G::kCols], x1[G::kCols], yb[G::kCols], qx[G::kCols], p2[G::kCols];
+#pragma unroll
+  for (int c = 0; c < G::kCols; ++c) {
+    x0[c] = (8 * c + 0.5f) - mx;
+    x1[c] = fminf(8 * c + 7.5f, xmax) - mx;
+    const float xe = fminf(fmaxf(0.f, x0[c]), x1[c]);
+    yb[c] = ky * xe;
+    qx[c] = f21 * xe;
+    p2[c] = (f11 * xe) * (f11 * xe);
   }
-  return m & rows;
+  unsigned m = 0u;
+#pragma unroll
+  for (int r = 0; r < G::kRows; ++r) {
+    const float y0 = (G::kBlockH * r + 0.5f) - my;
+    const float y1 = fminf(G::kBlockH * r + (G::kBlockH - 0.5f), ymax) - my;
+    const float ye = fminf(fmaxf(0.f, y0), y1);
+    const float xb = kx * ye, qy = f22 * ye;
+    const bool row_in = G::kBlockH * r + 0.5f <= ymax;
+#pragma unroll
+    for (int c = 0; c < G::kCols; ++c) {
+      const float q1 = __fmaf_rn(f22, fminf(fmaxf(yb[c], y0), y1), qx[c]);
+      const float v1 = __fmaf_rn(q1, q1, p2[c]);
+      const float xh = fminf(fmaxf(xb, x0[c]), x1[c]);
+      const float p = f11 * xh, q2 = __fmaf_rn(f21, xh, qy);
+      const float v2 = __fmaf_rn(q2, q2, p * p);
+      // (not a number: kept)
+      if (!(v1 > lim && v2 > lim) && row_in && 8 * c + 0.5f <= xmax) m |= 1u << (G::kCols * r + c);
+    }
+  }
+  return m;
 }
 
-// Builds the warp's list of staged entries (ascending) whose rows mask meets
-// the warp's rows; returns its length.
-template <int TS, int PPT>
-__device__ __forceinline__ int warp_entries(const unsigned short* s_rows, unsigned char* list,
+// Builds the warp's list of staged entries (ascending) whose blocks mask holds
+// the warp's block; returns its length.
+__device__ __forceinline__ int warp_entries(const unsigned char* s_blocks, unsigned char* list,
                                             int cnt, int lane, int warp) {
-  constexpr int kRows = (32 / TS) * PPT;  // tile rows of one warp
-  constexpr unsigned kBand = (1u << kRows) - 1u;
-  const unsigned band = kBand << (warp * kRows);
   const unsigned below = (1u << lane) - 1u;
   int n = 0;
   for (int c = 0; c < cnt; c += 32) {
     const int j = c + lane;
-    const bool hit = j < cnt && (s_rows[j] & band);
+    const bool hit = j < cnt && ((s_blocks[j] >> warp) & 1u);
     const unsigned b = __ballot_sync(kFull, hit);
     if (hit) list[n + __popc(b & below)] = (unsigned char)j;
     n += __popc(b);
@@ -243,7 +270,7 @@ __device__ __forceinline__ void fwd_tile(const CamTable& ct, const RenderConsts&
   __shared__ float4 s0[B];
   __shared__ float4 s1[B];
   __shared__ float s2[B];
-  __shared__ unsigned short s_rows[B];
+  __shared__ unsigned char s_blocks[B];
   __shared__ unsigned char s_list[NW][B];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const TileGeom<TS, PPT> tg = tile_geom<TS, PPT>(ct, tile);
@@ -281,15 +308,15 @@ __device__ __forceinline__ void fwd_tile(const CamTable& ct, const RenderConsts&
         s0[j] = make_float4(m.x, m.y, s.f11, s.f21);
         s1[j] = make_float4(s.f22, s.L2S, s.R, s.G);
         s2[j] = s.B;
-        s_rows[j] = (unsigned short)splat_rows<TS>(m.x, m.y, s.f11, s.f21, s.f22, s.L2S,
-                                                   rc.log2_alpha_min, tg.xmax, tg.rows);
+        s_blocks[j] = (unsigned char)splat_blocks<TS, PPT>(m.x, m.y, s.f11, s.f21, s.f22, s.L2S,
+                                                           rc.log2_alpha_min, tg.xmax, tg.ymax);
       }
     }
     __syncthreads();
     const int cnt = (int)min((unsigned)B, r.y - base);
-    // only the entries that may reach a pixel of this warp's rows
+    // only the entries that may reach a pixel of this warp's block
     const int n = __any_sync(kFull, live != 0u)
-                      ? warp_entries<TS, PPT>(s_rows, s_list[warp], cnt, lane, warp)
+                      ? warp_entries(s_blocks, s_list[warp], cnt, lane, warp)
                       : 0;
     for (int i = 0; i < n && live; ++i) {
       const int k = s_list[warp][i];
@@ -467,18 +494,25 @@ __device__ __forceinline__ float warp_sum9(const float v[9], int lane, int& slot
 // alpha = 0: its transmittance is kept by a select and every contribution
 // is zero, and its L stays finite (w is floored at 1e-30 inside the log).
 // The exponent is the scalar path's value exactly: RN(q^2 - base) is
-// -RN(base - q^2).  Sets gsum to the pixel sums of the 6 moments and 3
-// colour weights, which are exact zeros where neither pixel takes part
-// (alpha = 0 makes w and dd zero; every other factor is finite), so a lane
-// past its last blended entry needs no branch of its own.  Returns the
-// warp's lanes where either pixel took part (gsum is left unset when there
-// are none).
+// -RN(base - q^2).
+//
+// Colour and entropy share one recursion.  With gc = g . c_i, h = gc - gH L_i
+// and U = g . S - gH R (each in the units of R, see the top of the file):
+//   dL/dalpha_i = T_i h - U / (1 - alpha_i) = (T_i+1 h - U) / (1 - alpha_i),
+//   U += w_i h    (U starts at -gH R_N+1).
+// The signs are turned so that no packed operand needs a negation: the pixel's
+// g enters as -g and alpha as -alpha, which gives -h and -w.
+//
+// Sets gsum to the pixel sums of the 6 moments and 3 colour weights, which
+// are exact zeros where neither pixel takes part (alpha = 0 makes w and dd
+// zero; every other factor is finite), so a lane past its last blended entry
+// needs no branch of its own.  Returns the warp's lanes where either pixel
+// took part (gsum is left unset when there are none).
 __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float4 g0, const float4 g1,
                                          const float cB, float rx, float2 ry2, unsigned pos,
                                          unsigned last0, unsigned last1, float2& T2,
-                                         const float2 gr2, const float2 gg2, const float2 gb2,
-                                         const float2 gH2, float2& gS2, float2& R2,
-                                         float gsum[9]) {
+                                         const float2 ngr2, const float2 ngg2, const float2 ngb2,
+                                         const float2 gH2, float2& U2, float gsum[9]) {
   const float dx = rx - g0.x;
   const SplatColumn col = splat_column(g0.z, g0.w, g1.y, dx);
   const float2 dy = __fadd2_rn(ry2, make_float2(-g0.y, -g0.y));
@@ -490,29 +524,25 @@ __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float
   if (!who) return 0u;  // (warp-uniform) no pixel of the warp takes part
   const float ar0 = a0 ? fast_exp2(-en.x) : 0.f;
   const float ar1 = a1 ? fast_exp2(-en.y) : 0.f;
-  const float2 al = make_float2(fminf(rc.alpha_max, ar0), fminf(rc.alpha_max, ar1));
-  const float2 om = __fadd2_rn(make_float2(1.f, 1.f), make_float2(-al.x, -al.y));
+  const float2 nal = make_float2(fmaxf(-rc.alpha_max, -ar0), fmaxf(-rc.alpha_max, -ar1));
+  const float2 om = __fadd2_rn(make_float2(1.f, 1.f), nal);
   const float2 iom = make_float2(fast_rcp(om.x), fast_rcp(om.y));
   const float2 Ti = __fmul2_rn(T2, iom);
-  const float2 w = __fmul2_rn(al, Ti);
+  const float2 nw = __fmul2_rn(nal, Ti);
   const float2 L = __fadd2_rn(
-      make_float2(fast_log2(fmaxf(w.x, 1e-30f)), fast_log2(fmaxf(w.y, 1e-30f))),
+      make_float2(fast_log2(fmaxf(-nw.x, 1e-30f)), fast_log2(fmaxf(-nw.y, 1e-30f))),
       make_float2(kLog2e, kLog2e));
-  // colour part T_i gc - gS / (1 - alpha_i), entropy part gH (-L T_i + R / (1 - alpha_i))
-  const float2 gc = __ffma2_rn(gb2, make_float2(cB, cB),
-                               __ffma2_rn(gg2, make_float2(g1.w, g1.w),
-                                          __fmul2_rn(gr2, make_float2(g1.z, g1.z))));
-  const float2 sq = __fmul2_rn(gS2, iom);
-  float2 dA = __ffma2_rn(Ti, gc, make_float2(-sq.x, -sq.y));
-  const float2 ent = __ffma2_rn(make_float2(-L.x, -L.y), Ti, __fmul2_rn(R2, iom));
-  dA = __ffma2_rn(gH2, ent, dA);
-  const float2 c6 = __fmul2_rn(w, gr2), c7 = __fmul2_rn(w, gg2), c8 = __fmul2_rn(w, gb2);
-  gS2 = __ffma2_rn(w, gc, gS2);
-  R2 = __ffma2_rn(L, w, R2);
+  const float2 ngc = __ffma2_rn(ngb2, make_float2(cB, cB),
+                                __ffma2_rn(ngg2, make_float2(g1.w, g1.w),
+                                           __fmul2_rn(ngr2, make_float2(g1.z, g1.z))));
+  const float2 nh = __ffma2_rn(gH2, L, ngc);
+  const float2 ndA = __fmul2_rn(iom, __ffma2_rn(T2, nh, U2));
+  const float2 c6 = __fmul2_rn(nw, ngr2), c7 = __fmul2_rn(nw, ngg2), c8 = __fmul2_rn(nw, ngb2);
+  U2 = __ffma2_rn(nw, nh, U2);
   T2 = make_float2(a0 ? Ti.x : T2.x, a1 ? Ti.y : T2.y);
   // dd = dalpha alpha where alpha is below its clamp, then the moments
-  const float2 dd = __fmul2_rn(dA, make_float2(ar0 <= rc.alpha_max ? ar0 : 0.f,
-                                               ar1 <= rc.alpha_max ? ar1 : 0.f));
+  const float2 dd = __fmul2_rn(ndA, make_float2(ar0 <= rc.alpha_max ? nal.x : 0.f,
+                                                ar1 <= rc.alpha_max ? nal.y : 0.f));
   // the two pixels share the column offset dx: the dx-moments are dx times
   // the pixel sums of dd and dd dy
   const float2 ddy = __fmul2_rn(dd, dy);
@@ -528,6 +558,41 @@ __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float
   return who;
 }
 
+// The same for one pixel per thread (plain FP32, the same recursion).
+__device__ __forceinline__ unsigned bwd_one(const RenderConsts& rc, const float4 g0, const float4 g1,
+                                        const float cB, float rx, float ry, unsigned pos,
+                                        unsigned last, float& T, float gr, float gg, float gb,
+                                        float gH, float& U, float gsum[9]) {
+  const float dx = rx - g0.x, dy = ry - g0.y;
+  const SplatColumn col = splat_column(g0.z, g0.w, g1.y, dx);
+  float q;
+  const float e = splat_row(col, g1.x, dy, q);
+  const bool a = pos < last && !(e < rc.log2_alpha_min);
+  const unsigned who = __ballot_sync(kFull, a);
+  if (!who) return 0u;  // (warp-uniform)
+  const float ar = a ? fast_exp2(e) : 0.f;
+  const float al = fminf(rc.alpha_max, ar);
+  const float iom = fast_rcp(1.f - al);
+  const float Ti = T * iom;
+  const float w = al * Ti;
+  const float L = fast_log2(fmaxf(w, 1e-30f)) + kLog2e;
+  const float h = __fmaf_rn(-gH, L, __fmaf_rn(gb, cB, __fmaf_rn(gg, g1.w, gr * g1.z)));
+  const float dA = iom * __fmaf_rn(T, h, -U);
+  gsum[6] = w * gr;
+  gsum[7] = w * gg;
+  gsum[8] = w * gb;
+  U = __fmaf_rn(w, h, U);
+  T = a ? Ti : T;
+  const float dd = dA * (ar <= rc.alpha_max ? al : 0.f);
+  gsum[5] = dd;
+  gsum[0] = dd * dx;
+  gsum[1] = dd * dy;
+  gsum[2] = gsum[0] * dx;
+  gsum[3] = gsum[0] * dy;
+  gsum[4] = gsum[1] * dy;
+  return who;
+}
+
 template <int DT, int TS, int PPT, int B>
 __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts& rc,
                                          const BwdArgs& a, int tile) {
@@ -536,7 +601,7 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
   __shared__ float4 s1[B];
   __shared__ float s2[B];  // blue
   __shared__ unsigned s_row[B];
-  __shared__ unsigned short s_rows[B];
+  __shared__ unsigned char s_blocks[B];
   constexpr int NT = TileGeom<TS, PPT>::kThreads;
   constexpr int NW = NT / 32;
   static_assert(NW >= 1, "a tile needs at least one full warp");
@@ -570,17 +635,17 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
     mylast = max(mylast, last[q]);
   }
   // two pixels per thread: the state as FP32 pairs (packed f32x2 arithmetic)
-  float2 T2, gr2, gg2, gb2, gH2, gS2, R2;
+  float2 T2, ngr2, ngg2, ngb2, gH2, U2;
   if constexpr (PPT == 2) {
     T2 = make_float2(T[0], T[1]);
-    gr2 = make_float2(gr[0], gr[1]);
-    gg2 = make_float2(gg[0], gg[1]);
-    gb2 = make_float2(gb[0], gb[1]);
+    ngr2 = make_float2(-gr[0], -gr[1]);
+    ngg2 = make_float2(-gg[0], -gg[1]);
+    ngb2 = make_float2(-gb[0], -gb[1]);
     gH2 = make_float2(gH[0], gH[1]);
-    gS2 = make_float2(0.f, 0.f);
-    R2 = make_float2(Rent[0], Rent[1]);
+    U2 = make_float2(-gH[0] * Rent[0], -gH[1] * Rent[1]);
   }
   const float2 ry2 = make_float2(tg.ry0, tg.ry0 + 1.f);
+  float U1 = -gH[0] * Rent[0];  // (one pixel per thread)
   if (tid == 0) s_max = 0u;
   __syncthreads();
   if (mylast) atomicMax(&s_max, mylast);
@@ -599,13 +664,13 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       s1[j] = make_float4(s.f22, s.L2S, s.R, s.G);
       s2[j] = s.B;
       s_row[j] = row;
-      s_rows[j] = (unsigned short)splat_rows<TS>(m.x, m.y, s.f11, s.f21, s.f22, s.L2S,
-                                                 rc.log2_alpha_min, tg.xmax, tg.rows);
+      s_blocks[j] = (unsigned char)splat_blocks<TS, PPT>(m.x, m.y, s.f11, s.f21, s.f22, s.L2S,
+                                                         rc.log2_alpha_min, tg.xmax, tg.ymax);
     }
     __syncthreads();
-    // only the entries that may reach a pixel of this warp's rows, last first
+    // only the entries that may reach a pixel of this warp's block, last first
     const int n = __any_sync(kFull, mylast > start)
-                      ? warp_entries<TS, PPT>(s_rows, s_list[warp], cnt, lane, warp)
+                      ? warp_entries(s_blocks, s_list[warp], cnt, lane, warp)
                       : 0;
     for (int i = n - 1; i >= 0; --i) {
       const int k = s_list[warp][i];
@@ -617,14 +682,18 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       unsigned who = 0u;
       if constexpr (PPT == 2) {
         // every lane (one past its last blended entry takes no part and adds zeros)
-        who = bwd_pair(rc, s0[k], s1[k], s2[k], tg.rx, ry2, pos, last[0], last[1], T2, gr2, gg2,
-                       gb2, gH2, gS2, R2, gsum);
+        who = bwd_pair(rc, s0[k], s1[k], s2[k], tg.rx, ry2, pos, last[0], last[1], T2, ngr2, ngg2,
+                       ngb2, gH2, U2, gsum);
+        contrib = (who >> lane) & 1u;
+      } else if constexpr (PPT == 1) {
+        who = bwd_one(rc, s0[k], s1[k], s2[k], tg.rx, tg.ry0, pos, last[0], T[0], gr[0], gg[0],
+                      gb[0], gH[0], U1, gsum);
         contrib = (who >> lane) & 1u;
       } else {
 #pragma unroll
         for (int i = 0; i < 9; ++i) gsum[i] = 0.f;
       }
-      if (PPT != 2 && any_here) {
+      if (PPT > 2 && any_here) {
         const float4 g0 = s0[k];
         const float4 g1 = s1[k];
         const float cB = s2[k];
@@ -666,7 +735,7 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
           }
         }
       }
-      if constexpr (PPT != 2) who = __ballot_sync(kFull, contrib);
+      if constexpr (PPT > 2) who = __ballot_sync(kFull, contrib);
       if (who) {
         float* G = a.grad2d + 12ll * s_row[k];
         if (__popc(who) <= kDirectLanes) {
@@ -756,12 +825,27 @@ void launch_bwd_ppt(const CamTable& ct, const RenderConsts& rc, const BwdArgs& a
   launch_bwd_b<DT, TS, PPT, kMaxBatch>(ct, rc, a, ctas, st);
 }
 
+// Pixels per thread when the caller leaves the choice (the outputs do not
+// depend on it; the gradients only in the order of their sums).  Two pixels
+// share an entry's column part and halve the per-entry work, which counts as
+// long as the SMs are full.  With few tiles they are not: a tile's walk is one
+// serial chain, and 8 warps of 8x4 pixels walk shorter lists than 4 of 8x8.
+// Measured (forward / backward us, one against two pixels): 48 tiles 26.7 /
+// 33.8 against 32.2 / 43.5; 256 tiles 43.2 / 61.9 against 51.8 / 76.3; 384
+// tiles 43.8 / 63.9 against 55.6 / 76.3; 768 tiles 45.4 / 92.6 against 45.4 /
+// 72.1; 1014 tiles 54.7 / 104.9 against 46.4 / 80.4.
+constexpr int kOnePixelTilesFwd = 4 * 152, kOnePixelTilesBwd = 3 * 152;
+int pixels_per_thread(const CamTable& ct, const gs_launch* opt, int ctas, int few) {
+  if (opt && opt->pixels_per_thread) return opt->pixels_per_thread;
+  return ct.tile == 16 && ctas == 0 && ct.total_tiles <= few ? 1 : 2;
+}
+
 template <int DT>
 int launch_fwd_t(const CamTable& ct, const RenderConsts& rc, const FwdArgs& a, int ctas,
                  const gs_launch* opt, cudaStream_t st) {
   int e = record_event(opt ? opt->ev_begin : nullptr, st);
   if (e != GS_OK) return e;
-  const int ppt = (opt && opt->pixels_per_thread) ? opt->pixels_per_thread : 2;
+  const int ppt = pixels_per_thread(ct, opt, ctas, kOnePixelTilesFwd);
   const int batch = (opt && opt->batch) ? opt->batch : kMaxBatch;
   if (ct.total_tiles > 0) {
     if (ct.tile == 8) {  // 8x8 tiles: 1 or 2 px per thread (a CTA is at least one warp)
@@ -784,7 +868,7 @@ int launch_bwd_t(const CamTable& ct, const RenderConsts& rc, const BwdArgs& a, i
                  const gs_launch* opt, cudaStream_t st) {
   int e = record_event(opt ? opt->ev_begin : nullptr, st);
   if (e != GS_OK) return e;
-  const int ppt = (opt && opt->pixels_per_thread) ? opt->pixels_per_thread : 2;
+  const int ppt = pixels_per_thread(ct, opt, ctas, kOnePixelTilesBwd);
   const int batch = (opt && opt->batch) ? opt->batch : kMaxBatch;
   if (ct.total_tiles > 0) {
     if (ct.tile == 8) {

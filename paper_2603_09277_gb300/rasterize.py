@@ -78,7 +78,7 @@ class Rasterizer:
     claiming tiles from a list-length-ordered queue (the batched form);
     ordered: with one CTA per tile, launch the tiles longest list first (the
     same queue as the block order);
-    pixels_per_thread: 1, 2 or 4 (0 = the library default, 2);
+    pixels_per_thread: 1, 2 or 4 (0 = the library's choice: 2, or 1 with few tiles);
     batch: list entries staged per shared-memory batch, 128 or 256 (0 = 256).
     """
 
