@@ -6,7 +6,6 @@
 #include <string.h>
 
 #include <algorithm>
-#include <mutex>
 
 #include "gs_internal.cuh"
 
@@ -18,11 +17,8 @@ int launch_preprocess(const float* means, const float* log_scales, const float* 
                       const gs_params* prm, const gs_proj* out, cudaStream_t st);
 int launch_preprocess_bwd(const float* means, const float* log_scales, const float* quats,
                           const float* opacity_logits, const float* sh, int N, const CamTable& ct,
-                          const gs_params* prm, const unsigned* tiles_touched, const float* grad2d,
-                          float* g_means, float* g_ls, float* g_quats, float* g_opac, float* g_sh,
-                          cudaStream_t st);
-int launch_adjoint_list(const unsigned* tiles_touched, int N, int V, float* grad2d,
-                        cudaStream_t st);
+                          const gs_params* prm, float* grad2d, float* g_means, float* g_ls,
+                          float* g_quats, float* g_opac, float* g_sh, cudaStream_t st);
 int launch_grad2d_attributes(const gs_proj* proj, long long rows, const gs_params* prm,
                              const float* grad2d, float* out, cudaStream_t st);
 size_t bin_sort_workspace_size(long long n_rows, long long cap, long long total_tiles);
@@ -44,8 +40,8 @@ int launch_render_fwd(const gs_proj* proj, long long rows, const CamTable& ct,
 int launch_render_bwd(const gs_proj* proj, long long rows, const CamTable& ct,
                       const gs_params* prm, const unsigned* vals, const unsigned* ranges,
                       const float* final_T, const unsigned* last_idx, const float* dL_dimage,
-                      const float* dL_dentropy, float* grad2d, const gs_launch* opt,
-                      cudaStream_t st);
+                      const float* dL_dentropy, float* grad2d, const ZeroRegions& zero,
+                      const gs_launch* opt, cudaStream_t st);
 int bounds_status_render(unsigned* out, bool clear);
 int bounds_status_binning(unsigned* out, bool clear);
 int bounds_status_preprocess(unsigned* out, bool clear);
@@ -68,36 +64,6 @@ int invalid(const char* what) {
   return GS_ERR_INVALID_ARG;
 }
 
-// A second stream per device for work a call can run beside its own kernels.
-// The call forks it from the caller's stream with an event and joins it back
-// before the dependent kernel, so the ordering on the caller's stream is
-// unchanged and a stream capture records the side work as a parallel branch.
-struct SideStream {
-  cudaStream_t s = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-  bool tried = false, ok = false;
-};
-constexpr int kMaxDevices = 64;
-SideStream g_side[kMaxDevices];
-std::mutex g_side_mu;  // guards g_side and every fork..join sequence
-
-// The current device's side stream, or nullptr (then the call stays on one
-// stream).  It is created on first use outside a stream capture.
-SideStream* side_stream_locked(cudaStream_t st) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-  SideStream& ss = g_side[dev];
-  if (!ss.tried) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
-      return nullptr;
-    ss.tried = true;
-    ss.ok = cudaStreamCreateWithFlags(&ss.s, cudaStreamNonBlocking) == cudaSuccess &&
-            cudaEventCreateWithFlags(&ss.fork, cudaEventDisableTiming) == cudaSuccess &&
-            cudaEventCreateWithFlags(&ss.join, cudaEventDisableTiming) == cudaSuccess;
-  }
-  return ss.ok ? &ss : nullptr;
-}
 }  // namespace
 
 namespace {
@@ -598,46 +564,18 @@ int gs_render_bwd(const gs_proj* proj, int N, const gs_camera* cams, int V, cons
   if (N == 0) return GS_OK;  // no Gaussians: no gradients
   if (!opt || !opt->grad2d_zeroed)
     GS_TRY_CUDA(cudaMemsetAsync(grad2d, 0, sizeof(float) * 12 * (size_t)N * V, st));
-  // Beside the blending adjoint (bound by instruction issue, most of the
-  // memory bandwidth free), on the side stream: the list of Gaussians some
-  // view sees (in grad2d's pad floats, after its zeroing) and the zeroing of
-  // every parameter gradient.  (Zeroing only the unseen Gaussians' gradients
-  // inside the list kernel was slower where most Gaussians are unseen and
-  // no faster where all are seen.)
-  auto side_work = [&](cudaStream_t s) -> int {
-    const int r = launch_adjoint_list(proj->tiles_touched, N, V, grad2d, s);
-    if (r != GS_OK) return r;
-    GS_TRY_CUDA(cudaMemsetAsync(g_sh, 0, sizeof(float) * 3 * (size_t)prm->sh_stride * N, s));
-    GS_TRY_CUDA(cudaMemsetAsync(g_means, 0, sizeof(float) * 3 * (size_t)N, s));
-    GS_TRY_CUDA(cudaMemsetAsync(g_log_scales, 0, sizeof(float) * 3 * (size_t)N, s));
-    GS_TRY_CUDA(cudaMemsetAsync(g_quats, 0, sizeof(float) * 4 * (size_t)N, s));
-    GS_TRY_CUDA(cudaMemsetAsync(g_opacity_logits, 0, sizeof(float) * (size_t)N, s));
-    return GS_OK;
-  };
-  std::lock_guard<std::mutex> lock(g_side_mu);
-  SideStream* ss = side_stream_locked(st);
-  int rc = GS_OK;
-  if (ss) {
-    GS_TRY_CUDA(cudaEventRecord(ss->fork, st));
-    GS_TRY_CUDA(cudaStreamWaitEvent(ss->s, ss->fork, 0));
-    const int rs = side_work(ss->s);
-    // (the side branch is joined back on every path from here)
-    GS_TRY_CUDA(cudaEventRecord(ss->join, ss->s));
-    if (rs == GS_OK)
-      rc = launch_render_bwd(proj, (long long)N * V, ct, prm, sorted_vals, tile_ranges, final_T,
-                             last_idx, dL_dimage, dL_dentropy, grad2d, opt, st);
-    GS_TRY_CUDA(cudaStreamWaitEvent(st, ss->join, 0));
-    if (rs != GS_OK) return rs;
-  } else {
-    rc = side_work(st);
-    if (rc == GS_OK)
-      rc = launch_render_bwd(proj, (long long)N * V, ct, prm, sorted_vals, tile_ranges, final_T,
-                             last_idx, dL_dimage, dL_dentropy, grad2d, opt, st);
-  }
+  // the blending adjoint's CTAs also zero every parameter gradient (the
+  // projection's adjoint writes those of the Gaussians it takes)
+  const unsigned long long n = (unsigned long long)N;
+  const ZeroRegions zero{{g_sh, g_means, g_log_scales, g_quats, g_opacity_logits},
+                         {3ull * prm->sh_stride * n, 3 * n, 3 * n, 4 * n, n}};
+  const int rc = launch_render_bwd(proj, (long long)N * V, ct, prm, sorted_vals, tile_ranges,
+                                   final_T, last_idx, dL_dimage, dL_dentropy, grad2d, zero, opt,
+                                   st);
   if (rc != GS_OK) return rc;
   return launch_preprocess_bwd(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                               proj->tiles_touched, grad2d, g_means, g_log_scales, g_quats,
-                               g_opacity_logits, g_sh, st);
+                               grad2d, g_means, g_log_scales, g_quats, g_opacity_logits, g_sh,
+                               st);
 }
 
 int gs_grad2d_attributes(const gs_proj* proj, int N, int V, const gs_params* prm,

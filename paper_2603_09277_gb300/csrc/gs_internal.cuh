@@ -85,6 +85,13 @@ inline bool rect8_fits(const CamTable& ct) {
   return true;
 }
 
+// Float arrays that a kernel's CTAs zero beside their own work.
+struct ZeroRegions {
+  static constexpr int kMax = 5;
+  float* p[kMax];               // (4-byte aligned; NULL or n = 0: none)
+  unsigned long long n[kMax];   // floats
+};
+
 // Threshold constants in the forms the kernels test them.
 struct RenderConsts {
   float alpha_max;

@@ -12,8 +12,7 @@
 // coalesced across the warp; quaternions and SH rows use 16-byte loads.
 //
 // Backward: hand-derived adjoint of the same steps, one thread per Gaussian
-// that some view sees (a list built beside the blending adjoint), summing
-// over views; the covariance part runs through the Cholesky factor of the
+// that the blending adjoint touched in some view, summing over views; the covariance part runs through the Cholesky factor of the
 // 2D covariance (whitened form) and accumulates the log-scale and
 // rotation-matrix gradients over views, pushed to the quaternion once.
 #include <algorithm>
@@ -319,6 +318,8 @@ __device__ __forceinline__ float det2(float a, float b, float c, float d) {
   return __fadd_rn(f, e);
 }
 
+constexpr float kFactor = 0.8493218002880191f;  // sqrt(log2(e) / 2), the records' F = kFactor L^-1
+
 struct Projected {
   bool ok;
   float tx, ty, tz, ux, uy;
@@ -399,7 +400,7 @@ __device__ __forceinline__ void project_tail(const CamInfo& c, const Activated& 
   const float l22 = sqrtf(p.det) * i11;
   const float i22 = __frcp_rn(l22);
   const float i21 = -l21 * i11 * i22;
-  const float kc = 0.8493218002880191f;  // sqrt(log2(e) / 2)
+  const float kc = kFactor;
   p.f11 = kc * i11;
   p.f22 = kc * i22;
   p.f21 = kc * i21;
@@ -581,15 +582,24 @@ __global__ void __launch_bounds__(256, pre_ctas_per_sm<DEG>()) preprocess_kernel
 
 // ---------------------------------------------------------------------------
 // Adjoint of the projection.  grad2d rows, summed over the pixels of every
-// blended pair of the row: dd (dx, dy, dx^2, dx dy, dy^2, 1) and w (r, g, b),
-// with dd = dL/dalpha alpha where alpha is not clamped and (dx, dy) the
-// pixel centre minus the 2D mean.  Since alpha = sigma exp(-d^T K d / 2)
-// (K the conic, d = pixel - mean):
+// blended pair of the row, hold dd-moments and w (r, g, b), with dd = dL/dalpha
+// alpha where alpha is not clamped.  Since alpha = sigma exp(-d^T K d / 2) (K
+// the conic, d = (dx, dy) = pixel centre - mean):
 //   dL/dsigma = sum dd / sigma,  dL/dK = -(1/2) sum dd d d^T
 //   (so dL/da = -Sxx / 2, dL/db = -Sxy with b counted twice in d^T K d,
 //   dL/dc = -Syy / 2),  dL/dmean = K (Sx, Sy).
+// Two forms of the moments:
+//   WHITE (FP32 records): dd (p, q, p^2, pq, q^2, 1) with (p, q) = F d, the
+//   record's square-root factor F = kFactor L^-1 applied to d.  These are the
+//   whitened moments the adjoint works with, each of them a sum of terms of
+//   its own size: for an elongated Gaussian the moments of dx and dy are sums
+//   of the long direction's size whose difference is the short direction's.
+//   The adjoint writes the moments of (dx, dy) back into the rows it takes,
+//   which is what grad2d holds after the call.
+//   Otherwise (16-bit records, whose F is rounded): dd (dx, dy, dx^2, dx dy,
+//   dy^2, 1).
 // ---------------------------------------------------------------------------
-// Per-lane sums of one Gaussian's adjoint over the views the lane takes:
+// Sums of one Gaussian's adjoint over the views:
 // dL/dmean, dL/dlog-scale, dL/d(rotation matrix entries), the sum of dd
 // (-> opacity) and dL/dSH for the K coefficients in use.
 template <int DEG>
@@ -604,23 +614,6 @@ struct AdjAcc {
     gsig = 0.f;
 #pragma unroll
     for (int i = 0; i < 3 * K; ++i) gsh[i] = 0.f;
-  }
-  // sum over the L lanes of a group (butterfly, group-local mask)
-  template <int L>
-  __device__ __forceinline__ void reduce(unsigned mask) {
-#pragma unroll
-    for (int o = 1; o < L; o <<= 1) {
-#pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        gm[i] += __shfl_xor_sync(mask, gm[i], o);
-        gls[i] += __shfl_xor_sync(mask, gls[i], o);
-      }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) gRq[i] += __shfl_xor_sync(mask, gRq[i], o);
-      gsig += __shfl_xor_sync(mask, gsig, o);
-#pragma unroll
-      for (int i = 0; i < 3 * K; ++i) gsh[i] += __shfl_xor_sync(mask, gsh[i], o);
-    }
   }
 };
 
@@ -649,14 +642,13 @@ struct ShCoef {
   }
 };
 
-// SHREG: the SH gradient is summed in acc (a group of several lanes);
-// otherwise (one lane per Gaussian, degree 3: 48 sums would halve the
-// occupancy) it goes to g_sh directly: the first view that sees the
-// Gaussian stores, later ones add.
-template <int DEG, bool SHREG>
+// SHREG: the SH gradient is summed in acc; otherwise (degree 3: 48 sums would
+// halve the occupancy) it goes to g_sh directly: the first view that touched
+// the Gaussian stores, later ones add.
+template <int DEG, bool SHREG, bool WHITE>
 __device__ __forceinline__ void adjoint_view(
     int g, int v, const Activated& a, const float* __restrict__ sh, int N, const CamTable& ct,
-    float dilation, const ShPtr& shp, const float* __restrict__ grad2d,
+    float dilation, const ShPtr& shp, float* __restrict__ grad2d,
     AdjAcc<SHREG ? DEG : 0>& acc, bool first_view, bool vec_out, float* __restrict__ g_sh,
     const ShCoef<DEG>& shc) {
   constexpr int sh_deg = DEG;
@@ -666,17 +658,44 @@ __device__ __forceinline__ void adjoint_view(
   float* gRq = acc.gRq;
   float& gsig = acc.gsig;
     long long row = (long long)v * N + g;
-    const float4* G4 = reinterpret_cast<const float4*>(grad2d + row * 12);
-    float4 G0 = G4[0], G1 = G4[1], G2 = G4[2];
-    // G0 = (Sx, Sy, Sxx, Sxy), G1 = (Syy, S1, r, g), G2 = (b, pad, pad, pad)
+    float4* G4 = reinterpret_cast<float4*>(grad2d + row * 12);
+    const float4 G0 = G4[0], G1 = G4[1];
+    const float Gb = grad2d[row * 12 + 8];
+    // G0 = (Sx, Sy, Sxx, Sxy), G1 = (Syy, S1, r, g), then b (or of p, q)
     const CamInfo& c = ct.c[v];
     // (degree 3 keeps the exact projection: the FP32 head with its fallback
     // spills there, 31 -> 33 us on a 1M-Gaussian view)
     Projected p = DEG < 3 ? project_adjoint(c, a, dilation) : project(c, a, depth_of(c, a.mean), dilation);
 
     gsig += G1.y;  // sum dd; dL/dlogit = (sum dd / sigma) sigma (1 - sigma)
-    const float gmx = p.ca * G0.x + p.cb * G0.y;  // dL/dmean2d = K (Sx, Sy)
-    const float gmy = p.cb * G0.x + p.cc * G0.y;
+    // the projection's Cholesky factor L of Sigma' + dilation I
+    const float l21 = p.l21, i11 = p.i11, i22 = p.i22;
+    const float i21 = -l21 * i11 * i22;
+    float gmx, gmy;         // dL/dmean2d = K (Sx, Sy)
+    float G00, G01, G11;    // L^-1 dL/dK L^-T
+    if constexpr (WHITE) {
+      // z = L^-1 d = (p, q) / kFactor
+      constexpr float k1 = 1.f / kFactor, k2 = k1 * k1;
+      const float z0 = k1 * G0.x, z1 = k1 * G0.y;
+      const float z00 = k2 * G0.z, z01 = k2 * G0.w, z11 = k2 * G1.x;
+      gmx = i11 * z0 + i21 * z1;  // L^-T z
+      gmy = i22 * z1;
+      G00 = -0.5f * z00;
+      G01 = -0.5f * z01;
+      G11 = -0.5f * z11;
+      // the moments of d = L z
+      const float l11 = p.A * i11, l22 = __frcp_rn(i22);
+      const float sxx = l11 * z00, sxy = l21 * z00 + l22 * z01;
+      G4[0] = make_float4(l11 * z0, l21 * z0 + l22 * z1, l11 * sxx, l11 * sxy);
+      grad2d[row * 12 + 4] = l21 * sxy + l22 * (l21 * z01 + l22 * z11);
+    } else {
+      gmx = p.ca * G0.x + p.cb * G0.y;
+      gmy = p.cb * G0.x + p.cc * G0.y;
+      const float ga = -0.5f * G0.z, gbh = -0.5f * G0.w, gc = -0.5f * G1.x;
+      G00 = i11 * i11 * ga;
+      G01 = i11 * (i21 * ga + i22 * gbh);
+      G11 = i21 * i21 * ga + 2.f * i21 * i22 * gbh + i22 * i22 * gc;
+    }
 
     // --- colour -> SH coefficients and view direction
     float vx = a.mean[0] - c.cp[0], vy = a.mean[1] - c.cp[1], vz = a.mean[2] - c.cp[2];
@@ -687,7 +706,7 @@ __device__ __forceinline__ void adjoint_view(
     float raw[3] = {0.5f, 0.5f, 0.5f};
     shc.each(sh, g, shp, [&](int e, float v) { raw[e % 3] += Y[e / 3] * v; });
     float grgb[3] = {raw[0] < 0.f ? 0.f : G1.z, raw[1] < 0.f ? 0.f : G1.w,
-                     raw[2] < 0.f ? 0.f : G2.x};
+                     raw[2] < 0.f ? 0.f : Gb};
     float cdot[16] = {};  // SH[k] . grgb
     shc.each(sh, g, shp,
              [&](int e, float v) { cdot[e / 3] = __fmaf_rn(v, grgb[e % 3], cdot[e / 3]); });
@@ -744,9 +763,6 @@ __device__ __forceinline__ void adjoint_view(
     // Every factor is scaled by L^-1, so the condition number of Sigma' is
     // not squared as it would be through dL/dSigma' = -K Gk K.
     const float* T = p.T;
-    // the projection's Cholesky factor of Sigma' + dilation I
-    const float l21 = p.l21, i11 = p.i11, i22 = p.i22;
-    const float i21 = -l21 * i11 * i22;
     float Th[6];
     for (int j = 0; j < 3; ++j) {
       Th[j] = T[j] * i11;
@@ -757,10 +773,6 @@ __device__ __forceinline__ void adjoint_view(
       Z[j] = a.s[j] * (Th[0] * a.Rq[j] + Th[1] * a.Rq[3 + j] + Th[2] * a.Rq[6 + j]);
       Z[3 + j] = a.s[j] * (Th[3] * a.Rq[j] + Th[4] * a.Rq[3 + j] + Th[5] * a.Rq[6 + j]);
     }
-    const float ga = -0.5f * G0.z, gbh = -0.5f * G0.w, gc = -0.5f * G1.x;
-    const float G00 = i11 * i11 * ga;
-    const float G01 = i11 * (i21 * ga + i22 * gbh);
-    const float G11 = i21 * i21 * ga + 2.f * i21 * i22 * gbh + i22 * i22 * gc;
     float GZ[6];
     for (int j = 0; j < 3; ++j) {
       GZ[j] = G00 * Z[j] + G01 * Z[3 + j];
@@ -814,16 +826,15 @@ __device__ __forceinline__ void adjoint_view(
     gm[2] += c.R[2] * gtx + c.R[5] * gty + c.R[8] * gtz;
   }
 
-// Writes Gaussian g's gradients from the group's sums: lane `sub` == 0 the
-// per-Gaussian ones, the K SH coefficients in use split over the group's L
-// lanes as 16-byte stores where aligned, up to the end of the 32-byte sector
+// Writes Gaussian g's gradients from the sums over its views; the K SH
+// coefficients in use as 16-byte stores where aligned, up to the end of the 32-byte sector
 // holding the last of them (a partly written sector is filled from DRAM
 // first); the coefficients past that keep the zeros of the caller's zeroing
 // (with 16 coefficients stored per Gaussian and degree 0 in use, rewriting
 // them was 15/16 of this kernel's SH writes).
-template <int DEG, int L, bool SHREG>
+template <int DEG, bool SHREG>
 __device__ __forceinline__ void adjoint_finish(
-    int g, int sub, const Activated& a, const AdjAcc<DEG>& acc, const ShPtr& shp, bool vec_out,
+    int g, const Activated& a, const AdjAcc<DEG>& acc, const ShPtr& shp, bool vec_out,
     float* __restrict__ g_means, float* __restrict__ g_ls, float* __restrict__ g_quats,
     float* __restrict__ g_opac, float* __restrict__ g_sh) {
   constexpr int K = AdjAcc<DEG>::K;
@@ -833,7 +844,7 @@ __device__ __forceinline__ void adjoint_finish(
   } else if (vec_out) {
 #pragma unroll
     for (int i = 0; i < 12; ++i) {
-      if (i % L == sub && 4 * i < kSectorFloats && 4 * i < shp.gs) {
+      if (4 * i < kSectorFloats && 4 * i < shp.gs) {
         float o[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) o[j] = 4 * i + j < 3 * K ? acc.gsh[4 * i + j] : 0.f;
@@ -843,9 +854,8 @@ __device__ __forceinline__ void adjoint_finish(
   } else {
 #pragma unroll
     for (int e = 0; e < 48; ++e)
-      if (e % L == sub && e < 3 * K) g_sh[sh_index(shp, g, e)] = acc.gsh[e];
+      if (e < 3 * K) g_sh[sh_index(shp, g, e)] = acc.gsh[e];
   }
-  if (sub != 0) return;
   const float* gm = acc.gm;
   const float* gls = acc.gls;
   const float* gRq = acc.gRq;
@@ -874,163 +884,129 @@ __device__ __forceinline__ void adjoint_finish(
   reinterpret_cast<float4*>(g_quats)[g] = gq;
 }
 
-// Adjoint of one listed Gaussian by a group of L lanes (L = the views rounded
-// up to a power of two, at most 8): lane `sub` takes views sub, sub + L, ...
-// that see the Gaussian, the group sums its lanes' parts with shuffles and
-// writes the gradients.  Every gradient starts at zero (the caller zeroes
-// them), so the Gaussians no view sees keep zeros.
-template <int DEG, int L>
-__device__ __forceinline__ void adjoint_group(
-    int g, int sub, unsigned mask, const float* __restrict__ means,
-    const float* __restrict__ log_scales, const float* __restrict__ quats,
-    const float* __restrict__ opacity_logits, const float* __restrict__ sh, int N,
-    const CamTable& ct, float dilation, const ShPtr& shp,
-    const unsigned* __restrict__ tiles_touched, const float* __restrict__ grad2d,
-    float* __restrict__ g_means, float* __restrict__ g_ls, float* __restrict__ g_quats,
-    float* __restrict__ g_opac, float* __restrict__ g_sh) {
+// The rows the blending adjoint staged (a superset of those it added to) are
+// marked in a bitmap: bit row % 32 of the third pad float (float 10) of
+// grad2d's row row / 32, zeroed with grad2d.
+__device__ __forceinline__ unsigned touched_word(const float* grad2d, long long word) {
+  return __ldg(reinterpret_cast<const unsigned*>(grad2d) + 12 * word + 10);
+}
+
+// Adjoint of Gaussian g: sums its parts over the views whose blending touched
+// it and writes the gradients.  Every gradient starts at zero (the caller
+// zeroes them), so the Gaussians no pixel met keep zeros.
+template <int DEG, bool WHITE>
+__device__ __forceinline__ void adjoint_gaussian(
+    int g, const float* __restrict__ means, const float* __restrict__ log_scales,
+    const float* __restrict__ quats, const float* __restrict__ opacity_logits,
+    const float* __restrict__ sh, int N, const CamTable& ct, float dilation, const ShPtr& shp,
+    float* __restrict__ grad2d, float* __restrict__ g_means, float* __restrict__ g_ls,
+    float* __restrict__ g_quats, float* __restrict__ g_opac, float* __restrict__ g_sh) {
   const bool vec_out = shp.vec && (reinterpret_cast<uintptr_t>(g_sh) & 15) == 0;
   const Activated a = activate(means, log_scales, quats, opacity_logits, g);
-  constexpr bool SHREG = L > 1 || DEG < 3;
+  constexpr bool SHREG = DEG < 3;
   AdjAcc<SHREG ? DEG : 0> acc;
   acc.zero();
-  // the views (of this lane's share) that see the Gaussian, as a mask: the
-  // loads are issued together instead of one memory latency per view ahead
-  // of its moment row's
+  // the views that touched the Gaussian as a mask: the loads are issued
+  // together instead of one memory latency per view ahead of its moment row's
   unsigned long long seen = 0ull;
 #pragma unroll 8
-  for (int v = sub; v < ct.V; v += L)
-    seen |= (unsigned long long)(tiles_touched[(long long)v * N + g] != 0u) << v;
+  for (int v = 0; v < ct.V; ++v) {
+    const long long row = (long long)v * N + g;
+    seen |= (unsigned long long)((touched_word(grad2d, row >> 5) >> (row & 31)) & 1u) << v;
+  }
   ShCoef<DEG> shc;
   shc.load(sh, g, shp);
   bool first = true;
   while (seen) {
     const int v = __ffsll((long long)seen) - 1;
     seen &= seen - 1ull;
-    adjoint_view<DEG, SHREG>(g, v, a, sh, N, ct, dilation, shp, grad2d, acc, first, vec_out,
-                             g_sh, shc);
+    adjoint_view<DEG, SHREG, WHITE>(g, v, a, sh, N, ct, dilation, shp, grad2d, acc, first,
+                                    vec_out, g_sh, shc);
     first = false;
   }
-  acc.template reduce<L>(mask);
-  adjoint_finish<SHREG ? DEG : 0, L, SHREG>(g, sub, a, acc, shp, vec_out, g_means, g_ls,
-                                            g_quats, g_opac, g_sh);
+  adjoint_finish<SHREG ? DEG : 0, SHREG>(g, a, acc, shp, vec_out, g_means, g_ls, g_quats, g_opac,
+                                         g_sh);
 }
 
-// The adjoint runs over a list of the Gaussians some view sees, kept in the
-// pad floats of grad2d (the blending adjoint writes floats 0..8 of a row):
-// entry k is float 9 of row k and the count is float 11 of row 0, all as
-// unsigned; grad2d is zeroed before.  A CTA ranks its visible threads by
-// warp ballots and reserves their slots with one atomic (one per CTA keeps
-// the shared counter from serialising), so the list is in no particular
-// order (each entry is independent).  A Gaussian's views are tested in order
-// up to the first that sees it.
-constexpr int kListThreads = 256;
-__global__ void __launch_bounds__(kListThreads) adjoint_list_kernel(
-    const unsigned* __restrict__ tiles_touched, int N, int V, float* __restrict__ grad2d) {
-  __shared__ unsigned s_cnt[kListThreads / 32];
-  __shared__ unsigned s_base;
-  unsigned* g2 = reinterpret_cast<unsigned*>(grad2d);
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (long long base = (long long)blockIdx.x * kListThreads; base < N;
-       base += (long long)gridDim.x * kListThreads) {
-    const long long g = base + threadIdx.x;
-    bool vis = false;
-    if (g < N)
-      for (int v = 0; v < V && !vis; ++v) vis = tiles_touched[(long long)v * N + g] != 0u;
-    const unsigned b = __ballot_sync(0xffffffffu, vis);
-    if (lane == 0) s_cnt[w] = __popc(b);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned run = 0u;
-      for (int k = 0; k < kListThreads / 32; ++k) {
-        const unsigned c = s_cnt[k];
-        s_cnt[k] = run;
-        run += c;
-      }
-      s_base = run ? atomicAdd(g2 + 11, run) : 0u;
-    }
-    __syncthreads();
-    if (vis) g2[12ll * (s_base + s_cnt[w] + __popc(b & ((1u << lane) - 1u))) + 9] = (unsigned)g;
-    __syncthreads();  // s_cnt and s_base are rewritten by the next round
-  }
-}
-
-// The adjoint over the listed Gaussians: a resident grid, one group of L
-// lanes per Gaussian and iteration (a group's lanes share the Gaussian, so
-// they leave the loop together; shuffles use the group's lanes only).
+// The adjoint over the touched Gaussians.  A CTA takes `chunk` consecutive
+// Gaussians: it merges the views' bitmap words of its range in shared memory,
+// compacts the touched ones, and its threads take one each.  On dense scenes
+// most visible rows lie behind the pixels' last blended entries: reading the
+// moment rows and parameters of every visible Gaussian was most of this
+// kernel (8 views of 3M Gaussians, where the blending meets about a tenth of
+// the 24 M visible rows).  Compacting by chunk instead of into one list keeps
+// the parameter reads and gradient writes of neighbours together and needs no
+// launch of its own.
 constexpr int kAdjThreads = 128;
-// CTAs per SM the register budget allows: 2 where a group sums 48 SH
-// gradients in registers, 3 with 27, else 4 (at most 128 registers)
+constexpr int kAdjChunk = 2048;  // most Gaussians of a CTA
+// CTAs per SM the register budget allows
 #ifndef GS_ADJ_CTAS
-#define GS_ADJ_CTAS 5  // CTAs per SM of the single-lane adjoint (measured: 4 -> 0.725 ms, 5 -> 0.689, 6 -> 0.723 on 8 views of 3M)
+#define GS_ADJ_CTAS 5  // (measured on 8 views of 3M: 4 -> 0.725 ms, 5 -> 0.689, 6 -> 0.723)
 #endif
-template <int DEG, int L>
-constexpr int adj_ctas_per_sm() { return (DEG == 3 && L > 1) ? 2 : (DEG == 2 ? 3 : GS_ADJ_CTAS); }
+template <int DEG>
+constexpr int adj_ctas_per_sm() { return DEG == 2 ? 3 : GS_ADJ_CTAS; }
 
-template <int DEG, int L>
-__global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG, L>()) preprocess_bwd_kernel(
+template <int DEG, bool WHITE>
+__global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preprocess_bwd_kernel(
     const float* __restrict__ means, const float* __restrict__ log_scales,
     const float* __restrict__ quats, const float* __restrict__ opacity_logits,
     const float* __restrict__ sh, int N, const CamTable ct, float dilation, const ShPtr shp,
-    const unsigned* __restrict__ tiles_touched, const float* __restrict__ grad2d,
-    float* __restrict__ g_means, float* __restrict__ g_ls, float* __restrict__ g_quats,
-    float* __restrict__ g_opac, float* __restrict__ g_sh) {
-  const unsigned* g2 = reinterpret_cast<const unsigned*>(grad2d);
-  const unsigned n = g2[11];
-  const int lane = threadIdx.x & 31;
-  const int sub = lane % L;
-  const unsigned mask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u)) << (lane - sub);
-  const unsigned groups = gridDim.x * (kAdjThreads / L);
-  for (unsigned i = (blockIdx.x * kAdjThreads + threadIdx.x) / L; i < n; i += groups) {
-    if (!GS_IN_BOUNDS(i, N, 302)) break;  // the list holds at most N Gaussians
-    const unsigned g = g2[12ll * i + 9];
+    int chunk, float* __restrict__ grad2d, float* __restrict__ g_means, float* __restrict__ g_ls,
+    float* __restrict__ g_quats, float* __restrict__ g_opac, float* __restrict__ g_sh) {
+  __shared__ unsigned s_any[kAdjChunk / 32];
+  __shared__ unsigned short s_idx[kAdjChunk];
+  __shared__ unsigned s_n;
+  const int tid = threadIdx.x;
+  const long long g0 = (long long)blockIdx.x * chunk;
+  const int n = (int)min((long long)chunk, N - g0), words = (n + 31) / 32;
+  for (int i = tid; i < words; i += kAdjThreads) s_any[i] = 0u;
+  if (tid == 0) s_n = 0u;
+  __syncthreads();
+  const long long rows = (long long)ct.V * N;
+#pragma unroll 4
+  for (int i = tid; i < ct.V * words; i += kAdjThreads) {
+    const int v = i / words, w = i - v * words;
+    const long long r0 = (long long)v * N + g0 + 32 * w;  // the word's first row
+    const unsigned lo = touched_word(grad2d, r0 >> 5);
+    const unsigned hi = (r0 | 31) + 1 < rows ? touched_word(grad2d, (r0 >> 5) + 1) : 0u;
+    unsigned m = __funnelshift_r(lo, hi, (unsigned)(r0 & 31));
+    if (n - 32 * w < 32) m &= (1u << (n - 32 * w)) - 1u;  // (rows of the next view)
+    if (m) atomicOr(&s_any[w], m);
+  }
+  __syncthreads();
+  for (int w = tid; w < words; w += kAdjThreads) {
+    unsigned m = s_any[w];
+    if (!m) continue;
+    unsigned at = atomicAdd(&s_n, (unsigned)__popc(m));
+    for (; m; m &= m - 1u) s_idx[at++] = (unsigned short)(32 * w + __ffs((int)m) - 1);
+  }
+  __syncthreads();
+  const int cnt = (int)s_n;
+  for (int i = tid; i < cnt; i += kAdjThreads) {
+    const long long g = g0 + s_idx[i];
     if (!GS_IN_BOUNDS(g, N, 301)) continue;
-    adjoint_group<DEG, L>((int)g, sub, mask, means, log_scales, quats,
-                          opacity_logits, sh, N, ct, dilation, shp, tiles_touched, grad2d,
-                          g_means, g_ls, g_quats, g_opac, g_sh);
+    adjoint_gaussian<DEG, WHITE>((int)g, means, log_scales, quats, opacity_logits, sh, N, ct,
+                                 dilation, shp, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
   }
 }
 
-template <int DEG, int L>
+template <int DEG>
 void launch_adjoint(const float* means, const float* log_scales, const float* quats,
                     const float* opacity_logits, const float* sh, int N, const CamTable& ct,
-                    const gs_params* prm, const unsigned* tiles_touched, const float* grad2d,
-                    float* g_means, float* g_ls, float* g_quats, float* g_opac, float* g_sh,
-                    cudaStream_t st) {
-  // a resident grid: enough groups for every listed Gaussian at most
-  const long long want = ((long long)N * L + kAdjThreads - 1) / kAdjThreads;
-  const int grid = (int)std::min<long long>(152ll * adj_ctas_per_sm<DEG, L>() * 2, want);
-  preprocess_bwd_kernel<DEG, L><<<grid, kAdjThreads, 0, st>>>(
-      means, log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
-      tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
-}
-
-// Largest group of lanes per Gaussian.  1 (one thread walks all of a
-// Gaussian's views) is the form the timings chose: on 8 views of 3M
-// Gaussians 0.78 ms against 1.39 ms for groups of 8 lanes, whose redundant
-// activation and shuffle reduction cost more than their parallelism gains.
-#ifndef GS_ADJ_MAX_LANES
-#define GS_ADJ_MAX_LANES 1
-#endif
-
-template <int DEG>
-void launch_adjoint_deg(const float* means, const float* log_scales, const float* quats,
-                        const float* opacity_logits, const float* sh, int N, const CamTable& ct,
-                        const gs_params* prm, const unsigned* tiles_touched, const float* grad2d,
-                        float* g_means, float* g_ls, float* g_quats, float* g_opac, float* g_sh,
-                        cudaStream_t st) {
-  // lanes per Gaussian: the views rounded up to a power of two, at most 8
-  if (ct.V <= 1 || GS_ADJ_MAX_LANES == 1)
-    launch_adjoint<DEG, 1>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                           tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-  else if (ct.V <= 2 || GS_ADJ_MAX_LANES == 2)
-    launch_adjoint<DEG, 2>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                           tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-  else if (ct.V <= 4 || GS_ADJ_MAX_LANES == 4)
-    launch_adjoint<DEG, 4>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                           tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
+                    const gs_params* prm, float* grad2d, float* g_means, float* g_ls,
+                    float* g_quats, float* g_opac, float* g_sh, cudaStream_t st) {
+  // a chunk per resident CTA, in whole warps' words, at most kAdjChunk
+  const long long per = ((long long)N + 152 * GS_ADJ_CTAS - 1) / (152 * GS_ADJ_CTAS);
+  const int chunk = (int)std::min<long long>(kAdjChunk, (per + kAdjThreads - 1) / kAdjThreads * kAdjThreads);
+  const unsigned grid = (unsigned)(((long long)N + chunk - 1) / chunk);
+  if (prm->attr_dtype == GS_ATTR_F32)
+    preprocess_bwd_kernel<DEG, true><<<grid, kAdjThreads, 0, st>>>(
+        means, log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
+        chunk, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
   else
-    launch_adjoint<DEG, 8>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                           tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
+    preprocess_bwd_kernel<DEG, false><<<grid, kAdjThreads, 0, st>>>(
+        means, log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
+        chunk, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
 }
 
 // The 2D gradients of Suppl. C per row from the moment rows of the blending
@@ -1154,42 +1130,28 @@ int launch_preprocess(const float* means, const float* log_scales, const float* 
 
 int launch_preprocess_bwd(const float* means, const float* log_scales, const float* quats,
                           const float* opacity_logits, const float* sh, int N, const CamTable& ct,
-                          const gs_params* prm, const unsigned* tiles_touched, const float* grad2d,
-                          float* g_means, float* g_ls, float* g_quats, float* g_opac, float* g_sh,
-                          cudaStream_t st) {
+                          const gs_params* prm, float* grad2d, float* g_means, float* g_ls,
+                          float* g_quats, float* g_opac, float* g_sh, cudaStream_t st) {
   if (N == 0) return GS_OK;
   {
     const int e = stage_event(GS_STAGE_ADJOINT, false, st);
     if (e != GS_OK) return e;
   }
+#define GS_ADJ_LAUNCH(D)                                                                     \
+  launch_adjoint<D>(means, log_scales, quats, opacity_logits, sh, N, ct, prm, grad2d, g_means, \
+                    g_ls, g_quats, g_opac, g_sh, st)
   switch (prm->sh_degree) {
-    case 0: launch_adjoint_deg<0>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                                  tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-      break;
-    case 1: launch_adjoint_deg<1>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                                  tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-      break;
-    case 2: launch_adjoint_deg<2>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                                  tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-      break;
-    default: launch_adjoint_deg<3>(means, log_scales, quats, opacity_logits, sh, N, ct, prm,
-                                   tiles_touched, grad2d, g_means, g_ls, g_quats, g_opac, g_sh, st);
-      break;
+    case 0: GS_ADJ_LAUNCH(0); break;
+    case 1: GS_ADJ_LAUNCH(1); break;
+    case 2: GS_ADJ_LAUNCH(2); break;
+    default: GS_ADJ_LAUNCH(3); break;
   }
+#undef GS_ADJ_LAUNCH
   count_launches(1);
   {
     const int e = stage_event(GS_STAGE_ADJOINT, true, st);
     if (e != GS_OK) return e;
   }
-  return check_launch();
-}
-
-int launch_adjoint_list(const unsigned* tiles_touched, int N, int V, float* grad2d,
-                        cudaStream_t st) {
-  if (N == 0) return GS_OK;
-  const int grid = (int)std::min<long long>(152ll * 8, ((long long)N + kListThreads - 1) / kListThreads);
-  adjoint_list_kernel<<<grid, kListThreads, 0, st>>>(tiles_touched, N, V, grad2d);
-  count_launches(1);
   return check_launch();
 }
 

@@ -28,8 +28,10 @@
 //   the pixel centre minus the 2D mean: dsigma = dd / sigma,
 //   dconic = dd (-dx^2/2, -dx dy, -dy^2/2), dmean = dd conic (dx, dy).
 //   Every one of these is linear in the moments dd (1, dx, dy, dx^2, dx dy,
-//   dy^2), so the kernel sums the moments and the projection's adjoint
-//   applies 1 / sigma, the conic and the signs once per Gaussian.
+//   dy^2), so the kernel sums the moments (FP32 records: those of (p, q) =
+//   F (dx, dy), from which the projection's adjoint makes these) and the
+//   projection's adjoint applies 1 / sigma, the conic and the signs once per
+//   Gaussian.
 // The thread sums the 9 per-Gaussian values (6 moments, 3 colour weights)
 // over its pixels.  When at most kDirectLanes lanes of the warp contribute,
 // each of them adds its values to grad2d with three vector atomics;
@@ -440,11 +442,40 @@ struct BwdArgs {
   const unsigned* last_idx;
   const float* dL_dimage;
   const float* dL_dentropy;
-  float* grad2d;  // [rows][12]: sums dd (dx, dy, dx^2, dx dy, dy^2, 1), w (r, g, b), pad
+  float* grad2d;  // [rows][12]: sums dd (u, t, u^2, u t, t^2, 1), w (r, g, b), pad, with
+                  // (u, t) = F d for FP32 records and d otherwise
   const unsigned* order;
   unsigned* counter;
   unsigned long long rows, pixels;  // extents of the record and per-pixel arrays
+  ZeroRegions zero;                 // zeroed by the kernel's CTAs
 };
+
+// A CTA's stripes of the regions (16-byte stores; the first CTA also takes the
+// ends off 16-byte boundaries).  The backward's CTAs zero the parameter
+// gradients this way after their tiles: the stores drain while other CTAs
+// blend, which is bound by instruction issue, and no memsets (five, on a
+// second stream forked and joined by events) stand beside the kernel.
+__device__ __forceinline__ void zero_regions(const ZeroRegions& z) {
+#pragma unroll 1
+  for (int r = 0; r < ZeroRegions::kMax; ++r) {
+    float* p = z.p[r];
+    const unsigned long long n = z.n[r];
+    if (!p || n == 0) continue;
+    const unsigned long long head =
+        min(n, (unsigned long long)((0u - (unsigned)(reinterpret_cast<uintptr_t>(p) >> 2)) & 3u));
+    const unsigned long long n16 = (n - head) / 4;
+    const unsigned long long per = (n16 + gridDim.x - 1) / gridDim.x;
+    const unsigned long long b = (unsigned long long)blockIdx.x * per, e = min(n16, b + per);
+    uint4* q = reinterpret_cast<uint4*>(p + head);
+    for (unsigned long long i = b + threadIdx.x; i < e; i += blockDim.x)
+      __stcs(q + i, make_uint4(0u, 0u, 0u, 0u));
+    if (blockIdx.x == 0) {
+      if (threadIdx.x < head) p[threadIdx.x] = 0.f;
+      const unsigned long long t0 = head + 4 * n16;
+      if (t0 + threadIdx.x < n) p[t0 + threadIdx.x] = 0.f;  // (at most 3)
+    }
+  }
+}
 
 // Split-transpose warp sum of v[0..8]: at each butterfly level a lane keeps
 // one part of its values and sends the other, so 5 + 3 + 2 + 1 + 1 shuffles
@@ -508,6 +539,7 @@ __device__ __forceinline__ float warp_sum9(const float v[9], int lane, int& slot
 // zero; every other factor is finite), so a lane past its last blended entry
 // needs no branch of its own.  Returns the warp's lanes where either pixel
 // took part (gsum is left unset when there are none).
+template <bool WHITE>
 __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float4 g0, const float4 g1,
                                          const float cB, float rx, float2 ry2, unsigned pos,
                                          unsigned last0, unsigned last1, float2& T2,
@@ -543,15 +575,17 @@ __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float
   // dd = dalpha alpha where alpha is below its clamp, then the moments
   const float2 dd = __fmul2_rn(ndA, make_float2(ar0 <= rc.alpha_max ? nal.x : 0.f,
                                                 ar1 <= rc.alpha_max ? nal.y : 0.f));
-  // the two pixels share the column offset dx: the dx-moments are dx times
-  // the pixel sums of dd and dd dy
-  const float2 ddy = __fmul2_rn(dd, dy);
+  // the two pixels share their column, and with it p (or dx): those moments
+  // are p times the pixel sums of dd and dd q
+  const float u = WHITE ? col.p : dx;
+  const float2 t = WHITE ? qv : dy;
+  const float2 ddt = __fmul2_rn(dd, t);
   gsum[5] = dd.x + dd.y;
-  gsum[1] = ddy.x + ddy.y;
-  gsum[0] = dx * gsum[5];
-  gsum[2] = dx * gsum[0];
-  gsum[3] = dx * gsum[1];
-  gsum[4] = __fmaf_rn(ddy.x, dy.x, ddy.y * dy.y);
+  gsum[1] = ddt.x + ddt.y;
+  gsum[0] = u * gsum[5];
+  gsum[2] = u * gsum[0];
+  gsum[3] = u * gsum[1];
+  gsum[4] = __fmaf_rn(ddt.x, t.x, ddt.y * t.y);
   gsum[6] = c6.x + c6.y;
   gsum[7] = c7.x + c7.y;
   gsum[8] = c8.x + c8.y;
@@ -559,6 +593,7 @@ __device__ __forceinline__ unsigned bwd_pair(const RenderConsts& rc, const float
 }
 
 // The same for one pixel per thread (plain FP32, the same recursion).
+template <bool WHITE>
 __device__ __forceinline__ unsigned bwd_one(const RenderConsts& rc, const float4 g0, const float4 g1,
                                         const float cB, float rx, float ry, unsigned pos,
                                         unsigned last, float& T, float gr, float gg, float gb,
@@ -584,12 +619,13 @@ __device__ __forceinline__ unsigned bwd_one(const RenderConsts& rc, const float4
   U = __fmaf_rn(w, h, U);
   T = a ? Ti : T;
   const float dd = dA * (ar <= rc.alpha_max ? al : 0.f);
+  const float u = WHITE ? col.p : dx, t = WHITE ? q : dy;
   gsum[5] = dd;
-  gsum[0] = dd * dx;
-  gsum[1] = dd * dy;
-  gsum[2] = gsum[0] * dx;
-  gsum[3] = gsum[0] * dy;
-  gsum[4] = gsum[1] * dy;
+  gsum[0] = dd * u;
+  gsum[1] = dd * t;
+  gsum[2] = gsum[0] * u;
+  gsum[3] = gsum[0] * t;
+  gsum[4] = gsum[1] * t;
   return who;
 }
 
@@ -597,6 +633,9 @@ template <int DT, int TS, int PPT, int B>
 __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts& rc,
                                          const BwdArgs& a, int tile) {
   static_assert(B % 32 == 0 && B <= kMaxBatch, "batch: a multiple of 32, at most 256");
+  // the moments of (p, q) = F d where the records hold F in FP32, else of d
+  // (the projection's adjoint takes the same forms)
+  constexpr bool WHITE = DT == GS_ATTR_F32;
   __shared__ float4 s0[B];
   __shared__ float4 s1[B];
   __shared__ float s2[B];  // blue
@@ -664,6 +703,11 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       s1[j] = make_float4(s.f22, s.L2S, s.R, s.G);
       s2[j] = s.B;
       s_row[j] = row;
+      {  // marks the row for the projection's adjoint (see touched_word there)
+        unsigned* word = reinterpret_cast<unsigned*>(a.grad2d) + 12ll * (row >> 5) + 10;
+        const unsigned bit = 1u << (row & 31);
+        if (!(__ldcg(word) & bit)) atomicOr(word, bit);
+      }
       s_blocks[j] = (unsigned char)splat_blocks<TS, PPT>(m.x, m.y, s.f11, s.f21, s.f22, s.L2S,
                                                          rc.log2_alpha_min, tg.xmax, tg.ymax);
     }
@@ -682,11 +726,11 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       unsigned who = 0u;
       if constexpr (PPT == 2) {
         // every lane (one past its last blended entry takes no part and adds zeros)
-        who = bwd_pair(rc, s0[k], s1[k], s2[k], tg.rx, ry2, pos, last[0], last[1], T2, ngr2, ngg2,
+        who = bwd_pair<WHITE>(rc, s0[k], s1[k], s2[k], tg.rx, ry2, pos, last[0], last[1], T2, ngr2, ngg2,
                        ngb2, gH2, U2, gsum);
         contrib = (who >> lane) & 1u;
       } else if constexpr (PPT == 1) {
-        who = bwd_one(rc, s0[k], s1[k], s2[k], tg.rx, tg.ry0, pos, last[0], T[0], gr[0], gg[0],
+        who = bwd_one<WHITE>(rc, s0[k], s1[k], s2[k], tg.rx, tg.ry0, pos, last[0], T[0], gr[0], gg[0],
                       gb[0], gH[0], U1, gsum);
         contrib = (who >> lane) & 1u;
       } else {
@@ -725,12 +769,13 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
           T[q] = Ti;
           if (araw <= rc.alpha_max) {
             const float dd = dA * araw;
-            const float ddx = dd * dx, ddy = dd * dy;
-            gsum[0] += ddx;
-            gsum[1] += ddy;
-            gsum[2] = __fmaf_rn(ddx, dx, gsum[2]);
-            gsum[3] = __fmaf_rn(ddx, dy, gsum[3]);
-            gsum[4] = __fmaf_rn(ddy, dy, gsum[4]);
+            const float u = WHITE ? col.p : dx, t = WHITE ? qq : dy;
+            const float ddu = dd * u, ddt = dd * t;
+            gsum[0] += ddu;
+            gsum[1] += ddt;
+            gsum[2] = __fmaf_rn(ddu, u, gsum[2]);
+            gsum[3] = __fmaf_rn(ddu, t, gsum[3]);
+            gsum[4] = __fmaf_rn(ddt, t, gsum[4]);
             gsum[5] += dd;
           }
         }
@@ -779,6 +824,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, (TS == 16 && PPT != 4) ? 4 * PP
     const int t = blockIdx.x;
     bwd_tile<DT, TS, PPT, B>(ct, rc, a, a.order ? (int)a.order[t] : t);
   }
+  zero_regions(a.zero);
 }
 
 int record_event(void* ev, cudaStream_t st) {
@@ -938,9 +984,10 @@ int launch_render_fwd(const gs_proj* proj, long long rows, const CamTable& ct,
 int launch_render_bwd(const gs_proj* proj, long long rows, const CamTable& ct,
                       const gs_params* prm, const unsigned* vals, const unsigned* ranges,
                       const float* final_T, const unsigned* last_idx, const float* dL_dimage,
-                      const float* dL_dentropy, float* grad2d, const gs_launch* opt,
-                      cudaStream_t st) {
+                      const float* dL_dentropy, float* grad2d, const ZeroRegions& zero,
+                      const gs_launch* opt, cudaStream_t st) {
   BwdArgs a;
+  a.zero = zero;
   a.recs = proj->records;
   a.vals = vals;
   a.ranges = reinterpret_cast<const uint2*>(ranges);

@@ -55,9 +55,8 @@ def capture_step(fn, device="cuda"):
     host memory and the loss read-back included -- in a CUDA graph on a side
     stream and returns the graph; graph.replay() reruns the step with the
     buffers' current contents.  Run the step once eagerly first (the pair
-    buffers are sized there, and the library's second stream is created
-    outside a capture); list construction inside the graph keeps the pair
-    count on the device (bin_sort(sync=False)): after a replay, a nonzero
+    buffers are sized there); list construction inside the graph keeps the
+    pair count on the device (bin_sort(sync=False)): after a replay, a nonzero
     status_dev means the pair buffers overflowed."""
     g = torch.cuda.CUDAGraph()
     s = torch.cuda.Stream(device=device)
