@@ -33,8 +33,7 @@
 //   projection's adjoint applies 1 / sigma, the conic and the signs once per
 //   Gaussian.
 // The thread sums the 9 per-Gaussian values (6 moments, 3 colour weights)
-// over its pixels.  When at most kDirectLanes lanes of the warp contribute,
-// each of them adds its values to grad2d with three vector atomics;
+// over its pixels.  When few lanes of the warp contribute, each of them adds its values to grad2d with three vector atomics;
 // otherwise the warp sums them with a split-transpose shuffle reduction (12
 // shuffles leave one of the 9 totals in each of 9 lane pairs) and 9 lanes
 // add them with one atomic instruction.  (All 32 lanes adding to one address
@@ -57,7 +56,16 @@ namespace {
 // kernels, 256 or (F32 records, 16-pixel tiles) 128; at most 256 (a batch
 // position is one byte in the per-warp entry lists).
 constexpr int kMaxBatch = 256;
-constexpr int kDirectLanes = 24;  // up to this many contributing lanes add directly
+// Up to this many contributing lanes add directly; above, a warp reduction.  At
+// two pixels per thread 16 to 24 are the fastest (977 us on 8 views of 3M
+// Gaussians, 996 at 12, 1010 at 8), but every add into a large Gaussian's row
+// rounds: at 24 the colour and opacity gradients of a 1M-Gaussian view are up
+// to twice as far from their 64-bit values as at 12.  One pixel per thread runs
+// on few tiles, where the adds are few.
+template <int PPT>
+struct DirectLanes {
+  static constexpr int value = PPT == 1 ? 24 : 12;
+};
 constexpr unsigned kFull = 0xffffffffu;
 // A row coordinate this far from every mean makes the exponent -inf (f22 > 0),
 // so a finished or outside pixel never passes the alpha_min test again.
@@ -783,7 +791,7 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       if constexpr (PPT > 2) who = __ballot_sync(kFull, contrib);
       if (who) {
         float* G = a.grad2d + 12ll * s_row[k];
-        if (__popc(who) <= kDirectLanes) {
+        if (__popc(who) <= DirectLanes<PPT>::value) {
           // few contributing lanes: each adds its own values (three vector
           // atomics) instead of the 12-shuffle warp reduction
           if (contrib) {

@@ -3,25 +3,34 @@
 // the image, C1 = 0.01^2, C2 = 0.03^2, SSIM = mean over the view's pixels and
 // channels (the 3DGS reading; the paper does not define the term).
 //
-// Forward, one CTA per 16x16 block of output pixels of one view: the block and
-// its 5-pixel halo of image and target (all three channels) are staged in
-// shared memory.  The window moments are taken about a constant per block and
-// channel (the staged value at the block centre, c): with d = s - c (padding
-// samples s = 0), mu = c + E[d] and sigma^2 = E[d^2] - E[d]^2 hold exactly
-// for any constant, and around a value of the block two large FP32 sums do
-// not cancel in smooth regions.  Because c is constant over the block, the
-// 11x11 window sums are separable: a horizontal pass over the 26 staged rows
-// and a vertical pass per output pixel.  Per pixel and channel the forward
-// saves (mu_x, mu_y, dS/dmu_x, dS/dsigma_x^2, dS/dsigma_xy) (planar, one plane
-// per quantity) and adds lambda (1 - S) / (3 M_v V) to the loss partials.
+// Forward, one CTA per 32x32 block of output pixels of one view, one channel
+// after the other: the block and its 5-pixel halo of image and target are
+// staged in shared memory as pairs (x, y).  The window moments are taken about
+// a constant per block and channel (the staged value at the block centre, c):
+// with d = s - c (padding samples s = 0), mu = c + E[d] and sigma^2 = E[d^2] -
+// E[d]^2 hold exactly for any constant, and around a value of the block two
+// large FP32 sums do not cancel in smooth regions.  Because c is constant over
+// the block, the 11x11 window sums are separable: a horizontal pass over the 42
+// staged rows and a vertical pass per output pixel.  Per pixel and channel the
+// forward saves (mu_x, mu_y, dS/dmu_x, dS/dsigma_x^2, dS/dsigma_xy) (planar, one
+// plane per quantity) and adds lambda (1 - S) / (3 M_v V) to the loss partials.
 //
 // Backward, same blocking:
-//   dL/dx(p) -= lambda / (3 M_v V) sum_q G(q - p) [dS/dmu_x(q)
-//               + 2 (x(p) - mu_x(q)) dS/dsigma_x^2(q) + (y(p) - mu_y(q)) dS/dsigma_xy(q)]
-// over the window centres q inside the image (dsigma_x^2(q)/dx(p) =
-// 2 G(q-p)(x(p) - mu_x(q)) because the window weights sum to 1); with the
-// block constant c the bracket splits into five separable correlations:
-// G*a + 2 (x(p) - c) G*b - 2 G*((mu_x - c) b) + (y(p) - c') G*e - G*((mu_y - c') e).
+//   dL/dx(p) -= lambda / (3 M_v V) sum_q G(q - p) [a(q)
+//               + 2 (x(p) - mu_x(q)) b(q) + (y(p) - mu_y(q)) e(q)]
+// over the window centres q inside the image, with a = dS/dmu_x, b =
+// dS/dsigma_x^2, e = dS/dsigma_xy (dsigma_x^2(q)/dx(p) = 2 G(q-p)(x(p) -
+// mu_x(q)) because the window weights sum to 1).  With the block constants c, c'
+// of image and target the bracket splits into three separable correlations:
+//   G*(a - 2 (mu_x - c) b - (mu_y - c') e) + 2 (x(p) - c) G*b + (y(p) - c') G*e.
+//
+// What bounds them: instruction issue (the window sums; about 60 FP32
+// operations per pixel, channel and moment).  Blocks of 32 instead of 16 pixels
+// cut the halo rows of the horizontal pass from 1.6 to 1.3 per output row, one
+// channel at a time keeps the shared memory of a CTA at 42 KB (5 CTAs per SM;
+// three channels of 16x16 blocks took 67 KB in the backward, 33 % issue active),
+// packed FP32 pairs halve the instructions of paired quantities, and the
+// backward runs three correlations where it ran five.
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -30,9 +39,11 @@ namespace gs {
 namespace {
 
 constexpr int kSsimR = 5;                   // window radius
-constexpr int kSsimB = 16;                  // output block side
-constexpr int kSsimS = kSsimB + 2 * kSsimR; // staged side (26)
-constexpr int kSsimThreads = kSsimB * kSsimB;
+constexpr int kSsimTaps = 2 * kSsimR + 1;
+constexpr int kSsimB = 32;                  // output block side
+constexpr int kSsimS = kSsimB + 2 * kSsimR; // staged side (42)
+constexpr int kSsimP = 44;                  // staged row pitch (16-byte rows of 4 samples)
+constexpr int kSsimThreads = 256;
 constexpr float kC1 = 0.01f * 0.01f;
 constexpr float kC2 = 0.03f * 0.03f;
 
@@ -42,7 +53,7 @@ struct SsimViews {
   int W[GS_MAX_VIEWS], H[GS_MAX_VIEWS], BX[GS_MAX_VIEWS];
   int block_off[GS_MAX_VIEWS + 1];
   float scale[GS_MAX_VIEWS];  // lambda / (3 M_v V)
-  float win[2 * kSsimR + 1];  // normalised 1D Gaussian, sigma 1.5
+  float2 win[kSsimTaps];      // normalised 1D Gaussian, sigma 1.5, each weight twice
 };
 
 __device__ __forceinline__ int view_of_block(const SsimViews& sv, int b) {
@@ -52,16 +63,14 @@ __device__ __forceinline__ int view_of_block(const SsimViews& sv, int b) {
 }
 
 // Both passes of the separable window are register-blocked: a thread takes
-// kRun consecutive outputs along the pass direction, loads the kRun + 10
-// samples they share from shared memory once, and sums each output's 11 taps
-// in tap order (the same arithmetic per output as a tap-by-tap loop).  All
-// three channels are passed together.
-constexpr int kRun = 4;                          // outputs per thread and pass
-constexpr int kSpan = kRun + 2 * kSsimR;         // samples per run (14)
-constexpr int kHItems = 3 * kSsimS * (kSsimB / kRun);  // horizontal runs (312)
-constexpr int kVItems = 3 * kSsimB * (kSsimB / kRun);  // vertical runs (192)
-static_assert(kSsimB % kRun == 0, "runs tile the block");
-static_assert(kVItems <= kSsimThreads, "one vertical run per thread");
+// kRun consecutive outputs along the pass direction and reads the kRun + 10
+// samples they share from shared memory once; each output's 11 taps are summed
+// in tap order.
+constexpr int kRun = 4;                              // outputs per thread and pass
+constexpr int kSpan = kRun + 2 * kSsimR;             // samples per run (14)
+constexpr int kHItems = kSsimS * (kSsimB / kRun);    // horizontal runs (336)
+static_assert(kSsimB * (kSsimB / kRun) == kSsimThreads, "one vertical run per thread");
+static_assert(kSsimB == 32, "a warp is a row of the block in the vertical pass");
 
 // Exclusive per-block partial of sum (1 - S) (FP32 within the thread and the
 // warp: every term is >= 0; FP64 across the warps).
@@ -78,97 +87,112 @@ __device__ __forceinline__ void block_partial(float acc, double scale, double* o
   }
 }
 
-__global__ void __launch_bounds__(kSsimThreads) ssim_fwd_kernel(
+// The block of CTA b: its view, origin, extents and first pixel.
+struct SsimBlock {
+  int v, W, H, bx, by;
+  long long base;
+};
+__device__ __forceinline__ SsimBlock ssim_block(const SsimViews& sv, int b) {
+  SsimBlock k;
+  k.v = view_of_block(sv, b);
+  const int lb = b - sv.block_off[k.v];
+  k.W = sv.W[k.v];
+  k.H = sv.H[k.v];
+  k.bx = (lb % sv.BX[k.v]) * kSsimB;
+  k.by = (lb / sv.BX[k.v]) * kSsimB;
+  k.base = sv.pix_off[k.v];
+  return k;
+}
+
+__global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     float* __restrict__ maps /* 15 planes of P */, long long P, double* __restrict__ partials) {
-  __shared__ float sx[3][kSsimS][kSsimS];
-  __shared__ float sy[3][kSsimS][kSsimS];
-  __shared__ __align__(16) float sh[3][5][kSsimS][kSsimB];  // horizontal sums
-  const int b = blockIdx.x;
-  const int v = view_of_block(sv, b);
-  const int lb = b - sv.block_off[v];
-  const int W = sv.W[v], H = sv.H[v];
-  const int bx = (lb % sv.BX[v]) * kSsimB, by = (lb / sv.BX[v]) * kSsimB;
-  const long long base = sv.pix_off[v];
-  for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
-    const int yy = by - kSsimR + i / kSsimS, xx = bx - kSsimR + i % kSsimS;
-    const bool in = xx >= 0 && xx < W && yy >= 0 && yy < H;
-    const long long p = base + (long long)yy * W + xx;
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      sx[ch][i / kSsimS][i % kSsimS] = in ? image[3 * p + ch] : 0.f;
-      sy[ch][i / kSsimS][i % kSsimS] = in ? target[3 * p + ch] : 0.f;
-    }
-  }
-  __syncthreads();
-  // horizontal: run (ch, staged row r, columns x0 .. x0 + kRun - 1)
-  for (int it = threadIdx.x; it < kHItems; it += kSsimThreads) {
-    const int g = it % (kSsimB / kRun), r = (it / (kSsimB / kRun)) % kSsimS;
-    const int ch = it / (kSsimS * (kSsimB / kRun));
-    const int x0 = g * kRun;
-    const float cx = sx[ch][kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
-    const float cy = sy[ch][kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
-    float d[kSpan], e[kSpan];
-#pragma unroll
-    for (int j = 0; j < kSpan; ++j) {
-      d[j] = sx[ch][r][x0 + j] - cx;
-      e[j] = sy[ch][r][x0 + j] - cy;
-    }
-    float m[kRun], n[kRun], dd[kRun], ee[kRun], de[kRun];
-#pragma unroll
-    for (int o = 0; o < kRun; ++o) m[o] = n[o] = dd[o] = ee[o] = de[o] = 0.f;
-#pragma unroll
-    for (int i = 0; i < 2 * kSsimR + 1; ++i) {
-      const float w = sv.win[i];
-#pragma unroll
-      for (int o = 0; o < kRun; ++o) {
-        const float wd = w * d[o + i], we = w * e[o + i];
-        m[o] += wd;
-        n[o] += we;
-        dd[o] = __fmaf_rn(wd, d[o + i], dd[o]);
-        ee[o] = __fmaf_rn(we, e[o + i], ee[o]);
-        de[o] = __fmaf_rn(wd, e[o + i], de[o]);
-      }
-    }
-    *reinterpret_cast<float4*>(&sh[ch][0][r][x0]) = make_float4(m[0], m[1], m[2], m[3]);
-    *reinterpret_cast<float4*>(&sh[ch][1][r][x0]) = make_float4(n[0], n[1], n[2], n[3]);
-    *reinterpret_cast<float4*>(&sh[ch][2][r][x0]) = make_float4(dd[0], dd[1], dd[2], dd[3]);
-    *reinterpret_cast<float4*>(&sh[ch][3][r][x0]) = make_float4(ee[0], ee[1], ee[2], ee[3]);
-    *reinterpret_cast<float4*>(&sh[ch][4][r][x0]) = make_float4(de[0], de[1], de[2], de[3]);
-  }
-  __syncthreads();
-  // vertical: run (ch, column c, output rows y0 .. y0 + kRun - 1)
+  __shared__ __align__(16) float2 s_xy[kSsimS][kSsimP];
+  __shared__ __align__(16) float2 s_m[kSsimS][kSsimB];   // horizontal sums of (x, y)
+  __shared__ __align__(16) float2 s_q[kSsimS][kSsimB];   // of (x^2, y^2)
+  __shared__ __align__(16) float s_x[kSsimS][kSsimB];    // of x y
+  const SsimBlock k = ssim_block(sv, blockIdx.x);
+  const int col = threadIdx.x & 31, y0 = (threadIdx.x >> 5) * kRun;
   float acc = 0.f;
-  if (threadIdx.x < kVItems) {
-    const int c = threadIdx.x % kSsimB, q = (threadIdx.x / kSsimB) % (kSsimB / kRun);
-    const int ch = threadIdx.x / (kSsimB * (kSsimB / kRun));
-    const int y0 = q * kRun;
-    const float cx = sx[ch][kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
-    const float cy = sy[ch][kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
-    float mom[5][kRun];
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      float col[kSpan];
-#pragma unroll
-      for (int j = 0; j < kSpan; ++j) col[j] = sh[ch][k][y0 + j][c];
+#pragma unroll 1
+  for (int ch = 0; ch < 3; ++ch) {
+    for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
+      const int r = i / kSsimS, c = i - r * kSsimS;
+      const int yy = k.by - kSsimR + r, xx = k.bx - kSsimR + c;
+      const bool in = xx >= 0 && xx < k.W && yy >= 0 && yy < k.H;
+      const long long p = 3 * (k.base + (long long)yy * k.W + xx) + ch;
+      s_xy[r][c] = in ? make_float2(image[p], target[p]) : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const float2 cc = s_xy[kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
+    const float2 ncc = make_float2(-cc.x, -cc.y);
+    // horizontal: run (staged row r, columns x0 .. x0 + kRun - 1)
+    for (int it = threadIdx.x; it < kHItems; it += kSsimThreads) {
+      const int r = it / (kSsimB / kRun), x0 = (it % (kSsimB / kRun)) * kRun;
+      float2 m[kRun], q[kRun];
+      float x[kRun];
 #pragma unroll
       for (int o = 0; o < kRun; ++o) {
-        float t = 0.f;
-#pragma unroll
-        for (int j = 0; j < 2 * kSsimR + 1; ++j) t = __fmaf_rn(sv.win[j], col[o + j], t);
-        mom[k][o] = t;
+        m[o] = q[o] = make_float2(0.f, 0.f);
+        x[o] = 0.f;
       }
+#pragma unroll
+      for (int j = 0; j < kSpan; j += 2) {
+        const float4 t = *reinterpret_cast<const float4*>(&s_xy[r][x0 + j]);
+        const float2 d[2] = {__fadd2_rn(make_float2(t.x, t.y), ncc),
+                             __fadd2_rn(make_float2(t.z, t.w), ncc)};
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int o = 0; o < kRun; ++o) {
+            const int tap = j + h - o;
+            if (tap < 0 || tap >= kSsimTaps) continue;
+            const float2 w = __fmul2_rn(sv.win[tap], d[h]);
+            m[o] = __fadd2_rn(m[o], w);
+            q[o] = __ffma2_rn(w, d[h], q[o]);
+            x[o] = __fmaf_rn(w.x, d[h].y, x[o]);
+          }
+      }
+      float4* pm = reinterpret_cast<float4*>(&s_m[r][x0]);
+      float4* pq = reinterpret_cast<float4*>(&s_q[r][x0]);
+      pm[0] = make_float4(m[0].x, m[0].y, m[1].x, m[1].y);
+      pm[1] = make_float4(m[2].x, m[2].y, m[3].x, m[3].y);
+      pq[0] = make_float4(q[0].x, q[0].y, q[1].x, q[1].y);
+      pq[1] = make_float4(q[2].x, q[2].y, q[3].x, q[3].y);
+      *reinterpret_cast<float4*>(&s_x[r][x0]) = make_float4(x[0], x[1], x[2], x[3]);
     }
-    const int px = bx + c;
+    __syncthreads();
+    // vertical: column col, output rows y0 .. y0 + kRun - 1
+    float2 m[kRun], q[kRun];
+    float x[kRun];
 #pragma unroll
     for (int o = 0; o < kRun; ++o) {
-      const int py = by + y0 + o;
-      if (px < W && py < H) {
-        const long long p = base + (long long)py * W + px;
-        const float m1 = mom[0][o], n1 = mom[1][o];
-        const float mx = cx + m1, my = cy + n1;
-        const float sxx = __fmaf_rn(-m1, m1, mom[2][o]), syy = __fmaf_rn(-n1, n1, mom[3][o]);
-        const float sxy = __fmaf_rn(-m1, n1, mom[4][o]);
+      m[o] = q[o] = make_float2(0.f, 0.f);
+      x[o] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < kSpan; ++j) {
+      const float2 tm = s_m[y0 + j][col], tq = s_q[y0 + j][col];
+      const float tx = s_x[y0 + j][col];
+#pragma unroll
+      for (int o = 0; o < kRun; ++o) {
+        const int tap = j - o;
+        if (tap < 0 || tap >= kSsimTaps) continue;
+        m[o] = __ffma2_rn(sv.win[tap], tm, m[o]);
+        q[o] = __ffma2_rn(sv.win[tap], tq, q[o]);
+        x[o] = __fmaf_rn(sv.win[tap].x, tx, x[o]);
+      }
+    }
+    const int px = k.bx + col;
+#pragma unroll
+    for (int o = 0; o < kRun; ++o) {
+      const int py = k.by + y0 + o;
+      if (px < k.W && py < k.H) {
+        const long long p = k.base + (long long)py * k.W + px;
+        const float m1 = m[o].x, n1 = m[o].y;
+        const float mx = cc.x + m1, my = cc.y + n1;
+        const float sxx = __fmaf_rn(-m1, m1, q[o].x), syy = __fmaf_rn(-n1, n1, q[o].y);
+        const float sxy = __fmaf_rn(-m1, n1, x[o]);
         const float A1 = 2.f * mx * my + kC1, A2 = 2.f * sxy + kC2;
         const float B1 = mx * mx + my * my + kC1, B2 = sxx + syy + kC2;
         const float D = B1 * B2;
@@ -182,105 +206,102 @@ __global__ void __launch_bounds__(kSsimThreads) ssim_fwd_kernel(
         mp[4 * P] = 2.f * A1 / D;                              // dS/dsigma_xy
       }
     }
+    __syncthreads();  // (the staged channel is overwritten)
   }
-  block_partial(acc, (double)sv.scale[v], partials + b);
+  block_partial(acc, (double)sv.scale[k.v], partials + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kSsimThreads) ssim_bwd_kernel(
+__global__ void __launch_bounds__(kSsimThreads, 4) ssim_bwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     const float* __restrict__ maps, long long P, float* __restrict__ dimg) {
-  __shared__ float sm[3][5][kSsimS][kSsimS + 1];             // staged map terms
-  __shared__ __align__(16) float sh[3][5][kSsimS][kSsimB];  // horizontal sums
-  __shared__ float s_c[3][2];
-  const int b = blockIdx.x;
-  const int v = view_of_block(sv, b);
-  const int lb = b - sv.block_off[v];
-  const int W = sv.W[v], H = sv.H[v];
-  const int bx = (lb % sv.BX[v]) * kSsimB, by = (lb / sv.BX[v]) * kSsimB;
-  const long long base = sv.pix_off[v];
-  // block constants: the image and target at the block's first pixel
-  const long long p0 = base + (long long)by * W + bx;
-  if (threadIdx.x < 3) {
-    s_c[threadIdx.x][0] = image[3 * p0 + threadIdx.x];
-    s_c[threadIdx.x][1] = target[3 * p0 + threadIdx.x];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
-    const int yy = by - kSsimR + i / kSsimS, xx = bx - kSsimR + i % kSsimS;
-    const bool in = xx >= 0 && xx < W && yy >= 0 && yy < H;  // window centres in the image
-    const long long q = base + (long long)yy * W + xx;
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) {
-      const float* mp = maps + (long long)(5 * ch) * P;
-      float a = 0.f, bb = 0.f, e = 0.f, pm = 0.f, qm = 0.f;
-      if (in) {
-        const float mx = mp[q], my = mp[P + q];
-        a = mp[2 * P + q];
-        bb = mp[3 * P + q];
+  __shared__ __align__(16) float2 s_ab[kSsimS][kSsimP];  // (a - 2 (mu_x - c) b - (mu_y - c') e, b)
+  __shared__ __align__(16) float s_e[kSsimS][kSsimP];
+  __shared__ __align__(16) float2 s_hab[kSsimS][kSsimB];  // horizontal sums
+  __shared__ __align__(16) float s_he[kSsimS][kSsimB];
+  const SsimBlock k = ssim_block(sv, blockIdx.x);
+  const int col = threadIdx.x & 31, y0 = (threadIdx.x >> 5) * kRun;
+  const long long p0 = 3 * (k.base + (long long)k.by * k.W + k.bx);
+#pragma unroll 1
+  for (int ch = 0; ch < 3; ++ch) {
+    // block constants: the image and target at the block's first pixel
+    const float cx = image[p0 + ch], cy = target[p0 + ch];
+    const float* __restrict__ mp = maps + (long long)(5 * ch) * P;
+    for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
+      const int r = i / kSsimS, c = i - r * kSsimS;
+      const int yy = k.by - kSsimR + r, xx = k.bx - kSsimR + c;
+      float a = 0.f, b = 0.f, e = 0.f;
+      if (xx >= 0 && xx < k.W && yy >= 0 && yy < k.H) {  // window centres in the image
+        const long long q = k.base + (long long)yy * k.W + xx;
+        const float mx = mp[q] - cx, my = mp[P + q] - cy;
+        b = mp[3 * P + q];
         e = mp[4 * P + q];
-        pm = (mx - s_c[ch][0]) * bb;
-        qm = (my - s_c[ch][1]) * e;
+        a = __fmaf_rn(-2.f * mx, b, __fmaf_rn(-my, e, mp[2 * P + q]));
       }
-      sm[ch][0][i / kSsimS][i % kSsimS] = a;
-      sm[ch][1][i / kSsimS][i % kSsimS] = bb;
-      sm[ch][2][i / kSsimS][i % kSsimS] = e;
-      sm[ch][3][i / kSsimS][i % kSsimS] = pm;
-      sm[ch][4][i / kSsimS][i % kSsimS] = qm;
+      s_ab[r][c] = make_float2(a, b);
+      s_e[r][c] = e;
     }
-  }
-  __syncthreads();
-  for (int it = threadIdx.x; it < kHItems; it += kSsimThreads) {
-    const int g = it % (kSsimB / kRun), r = (it / (kSsimB / kRun)) % kSsimS;
-    const int ch = it / (kSsimS * (kSsimB / kRun));
-    const int x0 = g * kRun;
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      float row[kSpan];
-#pragma unroll
-      for (int j = 0; j < kSpan; ++j) row[j] = sm[ch][k][r][x0 + j];
-      float h[kRun];
+    __syncthreads();
+    for (int it = threadIdx.x; it < kHItems; it += kSsimThreads) {
+      const int r = it / (kSsimB / kRun), x0 = (it % (kSsimB / kRun)) * kRun;
+      float2 h[kRun];
+      float g[kRun];
 #pragma unroll
       for (int o = 0; o < kRun; ++o) {
-        float t = 0.f;
-#pragma unroll
-        for (int i = 0; i < 2 * kSsimR + 1; ++i) t = __fmaf_rn(sv.win[i], row[o + i], t);
-        h[o] = t;
+        h[o] = make_float2(0.f, 0.f);
+        g[o] = 0.f;
       }
-      *reinterpret_cast<float4*>(&sh[ch][k][r][x0]) = make_float4(h[0], h[1], h[2], h[3]);
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < kVItems) {
-    const int c = threadIdx.x % kSsimB, q = (threadIdx.x / kSsimB) % (kSsimB / kRun);
-    const int ch = threadIdx.x / (kSsimB * (kSsimB / kRun));
-    const int y0 = q * kRun;
-    float gsum[5][kRun];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
-      float col[kSpan];
+      for (int j = 0; j < kSpan; j += 2) {
+        const float4 t = *reinterpret_cast<const float4*>(&s_ab[r][x0 + j]);
+        const float2 u = *reinterpret_cast<const float2*>(&s_e[r][x0 + j]);
+        const float2 d[2] = {make_float2(t.x, t.y), make_float2(t.z, t.w)};
+        const float f[2] = {u.x, u.y};
 #pragma unroll
-      for (int j = 0; j < kSpan; ++j) col[j] = sh[ch][k][y0 + j][c];
+        for (int i = 0; i < 2; ++i)
 #pragma unroll
-      for (int o = 0; o < kRun; ++o) {
-        float t = 0.f;
-#pragma unroll
-        for (int j = 0; j < 2 * kSsimR + 1; ++j) t = __fmaf_rn(sv.win[j], col[o + j], t);
-        gsum[k][o] = t;
+          for (int o = 0; o < kRun; ++o) {
+            const int tap = j + i - o;
+            if (tap < 0 || tap >= kSsimTaps) continue;
+            h[o] = __ffma2_rn(sv.win[tap], d[i], h[o]);
+            g[o] = __fmaf_rn(sv.win[tap].x, f[i], g[o]);
+          }
       }
+      float4* ph = reinterpret_cast<float4*>(&s_hab[r][x0]);
+      ph[0] = make_float4(h[0].x, h[0].y, h[1].x, h[1].y);
+      ph[1] = make_float4(h[2].x, h[2].y, h[3].x, h[3].y);
+      *reinterpret_cast<float4*>(&s_he[r][x0]) = make_float4(g[0], g[1], g[2], g[3]);
     }
-    const float cx = s_c[ch][0], cy = s_c[ch][1];
-    const int px = bx + c;
+    __syncthreads();
+    float2 h[kRun];
+    float g[kRun];
 #pragma unroll
     for (int o = 0; o < kRun; ++o) {
-      const int py = by + y0 + o;
-      if (px < W && py < H) {
-        const long long p = base + (long long)py * W + px;
-        const float xp = image[3 * p + ch], yp = target[3 * p + ch];
-        const float grad = gsum[0][o] + 2.f * ((xp - cx) * gsum[1][o] - gsum[3][o]) +
-                           (yp - cy) * gsum[2][o] - gsum[4][o];
-        dimg[3 * p + ch] -= sv.scale[v] * grad;
+      h[o] = make_float2(0.f, 0.f);
+      g[o] = 0.f;
+    }
+#pragma unroll
+    for (int j = 0; j < kSpan; ++j) {
+      const float2 t = s_hab[y0 + j][col];
+      const float u = s_he[y0 + j][col];
+#pragma unroll
+      for (int o = 0; o < kRun; ++o) {
+        const int tap = j - o;
+        if (tap < 0 || tap >= kSsimTaps) continue;
+        h[o] = __ffma2_rn(sv.win[tap], t, h[o]);
+        g[o] = __fmaf_rn(sv.win[tap].x, u, g[o]);
       }
     }
+    const int px = k.bx + col;
+#pragma unroll
+    for (int o = 0; o < kRun; ++o) {
+      const int py = k.by + y0 + o;
+      if (px < k.W && py < k.H) {
+        const long long p = 3 * (k.base + (long long)py * k.W + px) + ch;
+        const float grad = h[o].x + 2.f * (image[p] - cx) * h[o].y + (target[p] - cy) * g[o];
+        dimg[p] -= sv.scale[k.v] * grad;
+      }
+    }
+    __syncthreads();  // (the staged channel is overwritten)
   }
 }
 
@@ -308,7 +329,8 @@ int launch_ssim(const float* image, const float* target, const CamTable& ct, flo
       g[k + kSsimR] = exp(-(double)(k * k) / (2.0 * 1.5 * 1.5));
       sum += g[k + kSsimR];
     }
-    for (int k = 0; k < 2 * kSsimR + 1; ++k) sv.win[k] = (float)(g[k] / sum);
+    for (int k = 0; k < kSsimTaps; ++k)
+      sv.win[k] = make_float2((float)(g[k] / sum), (float)(g[k] / sum));
   }
   sv.V = ct.V;
   sv.block_off[0] = 0;
