@@ -176,6 +176,17 @@ struct CountsOut {
   int* status;
 };
 
+// The totals q (super-tile items) and pp (pairs) into the counts (one thread).
+__device__ __forceinline__ void counts_check(const CountsOut& o, long long q, long long pp) {
+  const bool over = pp > o.capacity;
+  *o.Q = q;
+  *o.P = pp;
+  *o.num_pairs_dev = pp;
+  *o.status = over ? GS_ERR_CAPACITY : GS_OK;
+  *o.p_eff = over ? 0 : pp;  // on overflow every later stage sees zero pairs
+  *o.q_eff = over ? 0 : q;   // (Q <= P: a super-pair holds at least one pair)
+}
+
 __device__ __forceinline__ void scan_counts_check_dev(const CountsOut& o, int nblocks);
 
 __global__ void __launch_bounds__(kScanThreads) scan_counts_check_kernel(const CountsOut o,
@@ -184,23 +195,9 @@ __global__ void __launch_bounds__(kScanThreads) scan_counts_check_kernel(const C
 }
 
 __device__ __forceinline__ void scan_counts_check_dev(const CountsOut& o, int nblocks) {
-  unsigned long long* sums_q = o.sums_q;
-  unsigned long long* sums_p = o.sums_p;
-  const long long capacity = o.capacity;
-  long long *Q = o.Q, *P = o.P, *q_eff = o.q_eff, *p_eff = o.p_eff;
-  long long* num_pairs_dev = o.num_pairs_dev;
-  int* status = o.status;
-  const long long q = scan_blocks_dev(sums_q, nblocks);
-  const long long pp = scan_blocks_dev(sums_p, nblocks);
-  if (threadIdx.x == 0) {
-    const bool over = pp > capacity;
-    *Q = q;
-    *P = pp;
-    *num_pairs_dev = pp;
-    *status = over ? GS_ERR_CAPACITY : GS_OK;
-    *p_eff = over ? 0 : pp;  // on overflow every later stage sees zero pairs
-    *q_eff = over ? 0 : q;   // (Q <= P: a super-pair holds at least one pair)
-  }
+  const long long q = scan_blocks_dev(o.sums_q, nblocks);
+  const long long pp = scan_blocks_dev(o.sums_p, nblocks);
+  if (threadIdx.x == 0) counts_check(o, q, pp);
 }
 
 
@@ -266,13 +263,13 @@ __device__ __forceinline__ int4 unpack_rect8(unsigned p) {
 __device__ __forceinline__ int radix_result(const unsigned* range, int bits);
 
 // The depth-sorted rows: the buffer the sort left them in follows from the
-// device-side key range (the number of passes it ran).
+// device-side key range (the number of passes it ran); buf0 without a range.
 struct SortedRows {
   const unsigned* buf0;
   const unsigned* buf1;
   const unsigned* range;
   __device__ __forceinline__ const unsigned* get() const {
-    return radix_result(range, 32) ? buf1 : buf0;
+    return range && radix_result(range, 32) ? buf1 : buf0;
   }
 };
 
@@ -751,6 +748,422 @@ __global__ void __launch_bounds__(kRadixThreads, GS_RADIX_CTAS) radix_downsweep_
 // Buffer index (0 or 1) holding the sorted result.
 __device__ __forceinline__ int radix_result(const unsigned* range, int bits) {
   return radix_plan(range, bits).passes & 1;
+}
+
+// ----------------------------------------------------------------------------
+// Steps 1 to 3 in one cooperative launch, for up to kCoopRows rows: compaction
+// of the visible rows, the depth sort and the depth-ordered gather with its
+// counts, with a grid barrier between dependent phases.  As separate kernels
+// they are 13 launches of 4 to 10 us each whatever the rows, most of it
+// launching, filling and draining the chip and re-reading arguments: 10k rows
+// took about 75 us, 1M rows of which 70k are visible about 110 us.  Here the
+// counts a phase needs from all CTAs are summed by each CTA for itself, and a
+// pass's scatter also counts the next pass's digits (one reduction per item
+// into the chunk that will own it), so a pass is one phase.  Above kCoopRows the
+// passes are long enough for the separate kernels, whose three CTAs per SM hide
+// more latency.
+//
+// Every CTA is resident (cooperative launch).  The barrier's wait is bounded:
+// when it runs out, the CTA reports GS_ERR_TIMEOUT and leaves, the others run
+// out in turn, and the later kernels find zero counts.
+// ----------------------------------------------------------------------------
+constexpr int kCoopThreads = 512;
+constexpr int kCoopWarps = kCoopThreads / 32;
+constexpr int kCoopTile = kCoopThreads * kRadixIpt;  // 4096 items
+constexpr int kCoopShift = 12;                       // log2(kCoopTile)
+constexpr int kCoopGrid = 152;                       // most CTAs (one per SM)
+constexpr long long kCoopRows = 2ll << 20;
+static_assert(kCoopTile == 1 << kCoopShift, "chunks are whole tiles");
+
+struct CoopArgs {
+  RadixRows rows;
+  unsigned* k[2];
+  unsigned* v[2];
+  unsigned* hist;   // [passes][grid][256] digit counts of every chunk (zeroed here)
+  unsigned* cnt;    // [grid] visible rows per CTA
+  unsigned* range;  // [~smallest, largest] visible key (zero)
+  unsigned* bar;    // barrier arrivals (zero)
+  const int* rect;
+  const unsigned* rect8;
+  int N;
+  uint2* rect_sorted;
+  unsigned long long* arrive;  // (zero)
+  CountsOut co;
+};
+
+struct CoopShared {
+  unsigned key[kCoopTile], val[kCoopTile];
+  unsigned wc[kCoopWarps][kRadixBins + 1];  // per-warp digit counters (+ dummy)
+  unsigned pre[kCoopWarps][kRadixBins];     // per-warp start within the digit's run
+  unsigned off[kRadixBins];                 // tile-local start per digit
+  unsigned gl[kRadixBins];                  // global minus tile-local start per digit
+  unsigned part[2][kRadixBins];
+  unsigned ws[kCoopWarps], ws2[kCoopWarps];
+  unsigned long long wt[2][9];
+  int ok, last;
+};
+
+// Grid barrier number `phase` (1, 2, ...).  False when the wait ran out.
+__device__ __forceinline__ bool coop_barrier(const CoopArgs& a, CoopShared& s, unsigned phase) {
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const unsigned want = phase * gridDim.x;
+    atomicAdd(a.bar, 1u);
+    int ok = 0;
+    for (int i = 0; i < (1 << 21) && !ok; ++i) {  // (about a second)
+      unsigned x;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(a.bar) : "memory");
+      ok = x >= want;
+    }
+    if (!ok) {
+      *a.co.status = GS_ERR_TIMEOUT;
+      *a.co.num_pairs_dev = 0;
+      *a.co.P = -1;  // (for the host's read of the count)
+    }
+    s.ok = ok;
+  }
+  __syncthreads();
+  return s.ok != 0;
+}
+
+// Inclusive warp scan (32-bit).
+__device__ __forceinline__ unsigned warp_scan32(unsigned x) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  return x;
+}
+
+__global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopArgs a,
+                                                                     const CamTable ct) {
+  extern __shared__ __align__(16) unsigned char coop_smem[];
+  CoopShared& s = *reinterpret_cast<CoopShared*>(coop_smem);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const unsigned lt = (1u << lane) - 1u;
+  const int G = gridDim.x, cta = blockIdx.x;
+  const long long n_rows = a.rows.n;
+  // A. visible rows of the CTA's chunk (a contiguous part per warp) and the
+  //    visible rows' key range; the digit counts are cleared
+  const long long sub = ((n_rows + (long long)G * kCoopWarps - 1) / ((long long)G * kCoopWarps) + 31) / 32 * 32;
+  const long long r0 = ((long long)cta * kCoopWarps + w) * sub, r1 = min(n_rows, r0 + sub);
+  unsigned mine = 0u, kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll 4
+  for (long long b = r0; b < r1; b += 32) {
+    const long long j = b + lane;
+    const bool in = j < r1 && a.rows.tiles_touched[j] > 0u;
+    const unsigned k = in ? __float_as_uint(a.rows.depth[j]) : 0u;
+    mine += __popc(__ballot_sync(0xffffffffu, in));
+    if (in) {
+      kmin = min(kmin, k);
+      kmax = max(kmax, k);
+    }
+  }
+  for (int i = tid; i < kRadixMaxPasses * kRadixBins; i += kCoopThreads)
+    a.hist[(long long)cta * (kRadixMaxPasses * kRadixBins) + i] = 0u;
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) {
+    s.ws[w] = mine;
+    if (kmin <= kmax) {
+      atomicMax(a.range, ~kmin);
+      atomicMax(a.range + 1, kmax);
+    }
+  }
+  __syncthreads();
+  unsigned woff = 0u, total = 0u;  // the warp's start in the CTA, the CTA's rows
+#pragma unroll
+  for (int i = 0; i < kCoopWarps; ++i) {
+    woff += i < w ? s.ws[i] : 0u;
+    total += s.ws[i];
+  }
+  if (tid == 0) a.cnt[cta] = total;
+  unsigned phase = 1u;
+  if (!coop_barrier(a, s, phase++)) return;
+  // B. ordered compaction, with the first pass's digit counts
+  unsigned before = 0u, all = 0u;
+  if (tid < G) {
+    const unsigned c = __ldcg(a.cnt + tid);
+    all = c;
+    before = tid < cta ? c : 0u;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if (lane == 0) {
+    s.ws[w] = before;
+    s.ws2[w] = all;
+  }
+  __syncthreads();
+  before = all = 0u;
+#pragma unroll
+  for (int i = 0; i < kCoopWarps; ++i) {
+    before += s.ws[i];
+    all += s.ws2[i];
+  }
+  const unsigned n = all;
+  if (cta == 0 && tid == 0) *a.rows.n_vis = (long long)n;
+  const unsigned lo = ~__ldcg(a.range), hi = __ldcg(a.range + 1);
+  const unsigned base = n ? lo : 0u;
+  const int bits = n && hi > lo ? 32 - __clz(hi - lo) : 0;
+  const RadixPlan pl = radix_plan_bits(base, bits);
+  const unsigned dmask = (1u << pl.dbits) - 1u;  // (dbits 0: no pass)
+  // chunks of whole tiles, a power of two of them: chunk = position >> shift
+  int shift = kCoopShift;
+  while (((unsigned long long)G << shift) < n) ++shift;
+  auto count = [&](int pass, unsigned pos, unsigned k) {
+    atomicAdd(a.hist + ((long long)pass * G + (pos >> shift)) * kRadixBins +
+                  (((k - base) >> (pass * pl.dbits)) & dmask), 1u);
+  };
+  int buf = pl.passes & 1;  // (the result lands in buffer 0)
+  {
+    unsigned at = before + woff;
+    unsigned* __restrict__ ko = a.k[buf];
+    unsigned* __restrict__ vo = a.v[buf];
+#pragma unroll 2
+    for (long long b = r0; b < r1; b += 32) {
+      const long long j = b + lane;
+      const bool in = j < r1 && a.rows.tiles_touched[j] > 0u;
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (in) {
+        const unsigned k = __float_as_uint(a.rows.depth[j]), pos = at + __popc(m & lt);
+        if (pl.passes) {
+          ko[pos] = k;
+          count(0, pos, k);
+        }
+        vo[pos] = (unsigned)j;
+      }
+      at += __popc(m);
+    }
+  }
+  if (!coop_barrier(a, s, phase++)) return;
+  // C. stable passes over the digits, as radix_downsweep_kernel
+  const int chunks = (int)((n + (1u << shift) - 1u) >> shift);
+  for (int pass = 0; pass < pl.passes; ++pass, buf ^= 1) {
+    if (cta < chunks) {
+      // digit starts: the digits below over all chunks, then the chunks before
+      const int dd = tid & (kRadixBins - 1), half = tid >> kRadixMaxBits;
+      const unsigned* __restrict__ h = a.hist + (long long)pass * G * kRadixBins + dd;
+      unsigned hb = 0u, ha = 0u;
+#pragma unroll 8
+      for (int c = half; c < chunks; c += 2) {
+        const unsigned x = __ldcg(h + c * kRadixBins);
+        ha += x;
+        hb += c < cta ? x : 0u;
+      }
+      if (half) {
+        s.part[0][dd] = hb;
+        s.part[1][dd] = ha;
+      }
+      for (int i = tid; i < kCoopWarps * (kRadixBins + 1); i += kCoopThreads) (&s.wc[0][0])[i] = 0u;
+      __syncthreads();
+      unsigned gbase = 0u;
+      if (!half) {
+        hb += s.part[0][dd];
+        ha += s.part[1][dd];
+        gbase = warp_scan32(ha);
+        if (lane == 31) s.ws[w] = gbase;
+      }
+      __syncthreads();
+      if (!half) {
+        unsigned wo = 0u;
+        for (int i = 0; i < kRadixBins / 32; ++i) wo += i < w ? s.ws[i] : 0u;
+        gbase += wo - ha + hb;
+      }
+      const unsigned* __restrict__ ki = a.k[buf];
+      const unsigned* __restrict__ vi = a.v[buf];
+      unsigned* __restrict__ ko = a.k[buf ^ 1];
+      unsigned* __restrict__ vo = a.v[buf ^ 1];
+      const unsigned c0 = (unsigned)cta << shift, c1 = min(n, c0 + (1u << shift));
+      const int dshift = pass * pl.dbits;
+      const bool more = pass + 1 < pl.passes;
+      for (unsigned t0 = c0; t0 < c1; t0 += kCoopTile) {
+        unsigned k[kRadixIpt], v[kRadixIpt], dg[kRadixIpt], loc[kRadixIpt];
+        const unsigned p0 = t0 + w * (32 * kRadixIpt) + lane;
+#pragma unroll
+        for (int i = 0; i < kRadixIpt; ++i) {
+          const bool in = p0 + 32 * i < c1;
+          k[i] = in ? __ldcg(ki + p0 + 32 * i) : 0u;
+          v[i] = in ? __ldcg(vi + p0 + 32 * i) : 0u;
+          dg[i] = in ? ((k[i] - base) >> dshift) & dmask : (unsigned)kRadixBins;
+        }
+#pragma unroll
+        for (int i = 0; i < kRadixIpt; ++i) {
+          const bool valid = dg[i] < (unsigned)kRadixBins;
+          const unsigned vm = __ballot_sync(0xffffffffu, valid);
+          unsigned peers = valid ? vm : ~vm;
+#pragma unroll
+          for (int b = 0; b < kRadixMaxBits; ++b) {
+            const bool bit = (dg[i] >> b) & 1u;
+            const unsigned m = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? m : ~m;
+          }
+          const unsigned rank = __popc(peers & lt);
+          const unsigned old = s.wc[w][dg[i]];
+          __syncwarp();
+          if (rank == 0) s.wc[w][dg[i]] = old + __popc(peers);
+          __syncwarp();
+          loc[i] = old + rank;
+        }
+        __syncthreads();
+        unsigned run = 0u, inc = 0u;
+        if (tid < kRadixBins) {
+#pragma unroll
+          for (int ww = 0; ww < kCoopWarps; ++ww) {
+            const unsigned c = s.wc[ww][tid];
+            s.pre[ww][tid] = run;
+            s.wc[ww][tid] = 0u;
+            run += c;
+          }
+          inc = warp_scan32(run);
+          if (lane == 31) s.ws2[w] = inc;
+        }
+        __syncthreads();
+        if (tid < kRadixBins) {
+          unsigned wo = 0u;
+#pragma unroll
+          for (int ww = 0; ww < kRadixBins / 32 - 1; ++ww) wo += ww < w ? s.ws2[ww] : 0u;
+          const unsigned off = wo + inc - run;
+          s.off[tid] = off;
+          s.gl[tid] = gbase - off;
+          gbase += run;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kRadixIpt; ++i) {
+          if (dg[i] < (unsigned)kRadixBins) {
+            const unsigned lp = s.off[dg[i]] + s.pre[w][dg[i]] + loc[i];
+            s.key[lp] = k[i];
+            s.val[lp] = v[i];
+          }
+        }
+        __syncthreads();
+        const unsigned nt = min(c1 - t0, (unsigned)kCoopTile);
+        for (unsigned i = tid; i < nt; i += kCoopThreads) {
+          const unsigned kk = s.key[i];
+          const unsigned pos = s.gl[((kk - base) >> dshift) & dmask] + i;
+          if (!GS_IN_BOUNDS(pos, n, 202)) continue;
+          if (more) {
+            ko[pos] = kk;
+            count(pass + 1, pos, kk);
+          }
+          vo[pos] = s.val[i];
+        }
+      }
+    }
+    if (!coop_barrier(a, s, phase++)) return;
+  }
+  // D. the rects in depth order and the counts per block of 1,024 rows (the
+  //    blocks rows_expand_kernel takes); the last CTA scans them
+  const unsigned* __restrict__ rows = a.v[0];
+  const int nb = (int)((n + kScanTile - 1) / kScanTile);
+  for (int b = cta; b < nb; b += G) {
+    unsigned long long q = 0ull, pp = 0ull;
+    unsigned row[2];
+    int4 rr[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const unsigned at = (unsigned)b * kScanTile + i * kCoopThreads + tid;
+      row[i] = at < n ? __ldcg(rows + at) : 0xffffffffu;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      rr[i] = make_int4(0, 0, 0, 0);
+      if (row[i] != 0xffffffffu && GS_IN_BOUNDS(row[i], n_rows, 205))
+        rr[i] = a.rect8 ? unpack_rect8(a.rect8[row[i]]) : view_rect(a.rect, row[i], a.N, ct);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const unsigned at = (unsigned)b * kScanTile + i * kCoopThreads + tid;
+      if (at < n) {
+        a.rect_sorted[at] = pack_rect(rr[i]);
+        q += st_count(rr[i]);
+        pp += (unsigned long long)((rr[i].z - rr[i].x) * (rr[i].w - rr[i].y));
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      q += __shfl_xor_sync(0xffffffffu, q, o);
+      pp += __shfl_xor_sync(0xffffffffu, pp, o);
+    }
+    unsigned long long* red = reinterpret_cast<unsigned long long*>(s.key);
+    __syncthreads();
+    if (lane == 0) {
+      red[w] = q;
+      red[kCoopWarps + w] = pp;
+    }
+    __syncthreads();
+    if (tid < 2) {
+      unsigned long long t = 0ull;
+      for (int i = 0; i < kCoopWarps; ++i) t += red[tid * kCoopWarps + i];
+      (tid ? a.co.sums_p : a.co.sums_q)[b] = t;
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s.last = atomicAdd(a.arrive, 1ull) == (unsigned long long)G - 1ull;
+  __syncthreads();
+  if (!s.last) return;
+  __threadfence();
+  // warps 0-7 scan the super-tile counts, 8-15 the pair counts: each warp a
+  // contiguous part of the blocks
+  const int which = w >> 3, wi = w & 7;
+  unsigned long long* sums = which ? a.co.sums_p : a.co.sums_q;
+  const int per = (nb + 7) / 8, b0 = min(nb, wi * per), b1 = min(nb, b0 + per);
+  unsigned long long tot = 0ull;
+#pragma unroll 4
+  for (int i = b0 + lane; i < b1; i += 32) tot += __ldcg(sums + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+  if (lane == 0) s.wt[which][wi] = tot;
+  __syncthreads();
+  unsigned long long carry = 0ull, grand = 0ull;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    carry += i < wi ? s.wt[which][i] : 0ull;
+    grand += s.wt[which][i];
+  }
+  for (int b = b0; b < b1; b += 32) {  // (warp-uniform)
+    const int i = b + lane;
+    const unsigned long long x = i < b1 ? __ldcg(sums + i) : 0ull;
+    const unsigned long long incl = warp_incl_scan(x);
+    if (i < b1) sums[i] = carry + incl - x;
+    carry += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (tid == 0) {
+    unsigned long long pp = 0ull;
+    for (int i = 0; i < 8; ++i) pp += s.wt[1][i];
+    counts_check(a.co, (long long)grand, (long long)pp);
+  }
+}
+
+cudaError_t allow_coop_smem() {
+  return cudaFuncSetAttribute(depth_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(CoopShared));
+}
+
+// Most CTAs of depth_sort_kernel for a cooperative launch on the current device
+// (0: not available there); cached per device.
+int coop_grid() {
+  static std::atomic<int> cache[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  const int c = cache[dev].load(std::memory_order_relaxed);
+  if (c) return c > 0 ? c : 0;
+  int per_sm = 0, sms = 0, coop = 0;
+  int v = -1;
+  if (allow_coop_smem() == cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, depth_sort_kernel, kCoopThreads,
+                                                    sizeof(CoopShared)) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+      per_sm > 0 && sms > 0)
+    v = std::min(kCoopGrid, sms);
+  cudaGetLastError();
+  cache[dev].store(v, std::memory_order_relaxed);
+  return v > 0 ? v : 0;
 }
 
 // ----------------------------------------------------------------------------
@@ -1476,6 +1889,9 @@ constexpr int kRadixGrid = 4 * 152;  // largest radix grid (4 CTAs per SM of a G
 // Radix histograms: [256][grid] per-CTA digit counts and their scan, then the
 // 256 digit totals.
 constexpr size_t radix_hist_bytes() { return 4ull * kRadixBins * (kRadixGrid + 1); }
+// (depth_sort_kernel: a table of [kCoopGrid][256] per pass, then a count per CTA)
+static_assert((size_t)kRadixMaxPasses * kCoopGrid * kRadixBins + kCoopGrid <= radix_hist_bytes() / 4,
+              "the sort's counts fit the histogram buffer");
 
 // CTAs of radix_downsweep_kernel resident on the current device at once
 // (cached per device).
@@ -1504,7 +1920,7 @@ inline long long scan_blocks(long long n) { return (n + kScanTile - 1) / kScanTi
 // ceil(len / kSeg) <= Q / kSeg + super-tiles, and Q <= P <= cap.
 inline long long max_segments(long long cap, long long tiles) { return cap / kSeg + tiles + 2; }
 
-constexpr int kCounters = 14;  // 8 counts, 3 arrival counters, spare, the depth-key range
+constexpr int kCounters = 14;  // 8 counts, 3 arrival counters, the grid barrier, the depth-key range
 
 Workspace carve(void* base, long long n_rows, long long cap, long long tiles) {
   Workspace w;
@@ -1615,7 +2031,8 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
                      status_dev};
   // the visible rows' depth-bit range (complement of the smallest, largest)
   unsigned* range = reinterpret_cast<unsigned*>(w.counters + 12);
-  const SortedRows rows_sorted{w.rv[0], w.rv[1], range};
+  const int coop = n_rows <= kCoopRows ? coop_grid() : 0;
+  const SortedRows rows_sorted{w.rv[0], w.rv[1], coop ? nullptr : range};
   // scan blocks of 1,024 rows (4 per thread) keep many CTAs in flight when
   // few rows are visible; on large row counts 4,096-row blocks (16 per
   // thread) are faster
@@ -1624,7 +2041,33 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
   const bool small = n_rows <= (4ll << 20);
   const int items = small ? 4 : 16;
   const long long nb = (n_rows + kScanThreads * items - 1) / (kScanThreads * items);
-  if (n_rows > 0) {
+  if (n_rows > 0 && coop) {
+    // 1-3. in one launch
+    CoopArgs a;
+    a.rows = RadixRows{proj->depth, proj->tiles_touched, n_rows, n_vis};
+    for (int i = 0; i < 2; ++i) {
+      a.k[i] = w.rk[i];
+      a.v[i] = w.rv[i];
+    }
+    a.hist = w.hist;
+    a.cnt = w.hist + (size_t)kRadixMaxPasses * kCoopGrid * kRadixBins;
+    a.range = range;
+    a.bar = reinterpret_cast<unsigned*>(w.counters + 11);
+    a.rect = proj->rect;
+    a.rect8 = rect8;
+    a.N = N;
+    a.rect_sorted = w.rect_sorted;
+    a.arrive = arrive + 1;
+    a.co = co;
+    CamTable cams = ct;
+    void* args[] = {&a, &cams};
+    // a CTA per 1,024 rows, at most one per SM: fewer CTAs meet at a barrier sooner
+    const int ctas = (int)std::min<long long>(coop, (n_rows + 1023) / 1024);
+    GS_TRY_CUDA(allow_coop_smem());
+    GS_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(depth_sort_kernel), dim3(ctas),
+                                            dim3(kCoopThreads), args, sizeof(CoopShared), st));
+    count_launches(1);
+  } else if (n_rows > 0) {
     // 1-2. stable depth sort of the visible rows (ties keep row order = id
     //    order) on the significant bits of their depth range; the first pass
     //    reads the rows (depth bits, visible when tiles_touched > 0), drops
@@ -1652,6 +2095,11 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     long long p_host = 0;
     GS_TRY_CUDA(cudaMemcpyAsync(&p_host, P, sizeof(long long), cudaMemcpyDeviceToHost, st));
     GS_TRY_CUDA(cudaStreamSynchronize(st));
+    if (p_host < 0) {
+      *num_pairs_host = 0;
+      GS_TRY_CUDA(cudaMemsetAsync(ranges, 0, 2 * sizeof(unsigned) * (size_t)T, st));
+      return GS_ERR_TIMEOUT;
+    }
     *num_pairs_host = p_host;
     if (p_host > cap) {
       GS_TRY_CUDA(cudaMemsetAsync(ranges, 0, 2 * sizeof(unsigned) * (size_t)T, st));

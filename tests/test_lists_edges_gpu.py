@@ -83,3 +83,29 @@ def test_lists_of_ragged_views(N, sizes, big):
 
 def test_lists_of_a_view_too_wide_for_packed_descriptors():
     _check([(16 * 8003 + 5, 40)], 3000, 5, 30)
+
+
+@pytest.mark.parametrize("lo,hi", [(1.0, 1.0), (1.0, 1.00001), (0.9, 1.1), (0.25, 3e4)])
+@pytest.mark.parametrize("N", [1, 1000, 4095, 4097, 152 * 4096, 152 * 4096 + 1, 1 << 21,
+                               (1 << 21) + 1])
+def test_depth_order_on_both_sides_of_the_one_launch_sort(N, lo, hi):
+    """One tile, so that its list is the visible rows by (depth, row): up to 2^21
+    rows the sort runs in one launch, above in separate passes; depth ranges of 0
+    to 4 digits."""
+    from paper_2603_09277_gb300 import scenes
+    from paper_2603_09277_gb300.rasterize import Rasterizer
+    g = torch.Generator(device="cuda").manual_seed(N)
+    r = Rasterizer([scenes.camera(16, 16, 16)], scenes.params(), N, pair_capacity=N)
+    u = torch.rand(N, generator=g, device="cuda", dtype=torch.float64)
+    depth = (lo * (hi / lo) ** u).float()
+    vis = torch.rand(N, generator=g, device="cuda") < 0.7
+    r.depth.copy_(depth)
+    r.tiles_touched.copy_(vis.int())
+    r.rect8.copy_(torch.where(vis, 1 << 16 | 1 << 24, 0))
+    rows = torch.nonzero(vis)[:, 0]
+    want = rows[torch.argsort(depth[rows], stable=True)]
+    for sync in (True, False):
+        r.sorted_vals.fill_(-1)
+        r.bin_sort(sync=sync)
+        assert int(r.num_pairs_dev) == rows.numel() and int(r.status_dev) == 0
+        assert torch.equal(r.sorted_vals[:rows.numel()].long(), want)
