@@ -773,6 +773,14 @@ constexpr int kCoopTile = kCoopThreads * kRadixIpt;  // 4096 items
 constexpr int kCoopShift = 12;                       // log2(kCoopTile)
 constexpr int kCoopGrid = 152;                       // most CTAs (one per SM)
 constexpr long long kCoopRows = 2ll << 20;
+// Row groups of 32 of a warp: at most kCoopRows over the warps of the whole
+// grid (smaller grids take fewer rows: a CTA per 1,024 rows).
+constexpr int kCoopGroups = (int)((kCoopRows / (kCoopGrid * kCoopWarps) + 31) / 32 + 1);
+// Up to this many rows the grid is one cluster of up to 8 CTAs.
+constexpr int kCoopCluster = 8;
+constexpr long long kClusterRows = (long long)kCoopCluster * kCoopTile;
+static_assert(kClusterRows / (kCoopCluster * kCoopWarps) <= 32 * kCoopGroups,
+              "a warp's rows of the cluster form fit");
 static_assert(kCoopTile == 1 << kCoopShift, "chunks are whole tiles");
 
 struct CoopArgs {
@@ -799,32 +807,44 @@ struct CoopShared {
   unsigned gl[kRadixBins];                  // global minus tile-local start per digit
   unsigned part[2][kRadixBins];
   unsigned ws[kCoopWarps], ws2[kCoopWarps];
+  unsigned vis[kCoopWarps][kCoopGroups];    // visible lanes of the warp's rows
   unsigned long long wt[2][9];
   int ok, last;
 };
 
-// Grid barrier number `phase` (1, 2, ...).  False when the wait ran out.
+// Barrier number `phase` (1, 2, ...) over the grid.  CLUSTER: the grid is one
+// cluster, whose hardware barrier takes a fraction of the time.  Otherwise
+// through an arrival counter: false when the wait ran out.
+template <bool CLUSTER>
 __device__ __forceinline__ bool coop_barrier(const CoopArgs& a, CoopShared& s, unsigned phase) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned want = phase * gridDim.x;
-    atomicAdd(a.bar, 1u);
-    int ok = 0;
-    for (int i = 0; i < (1 << 21) && !ok; ++i) {  // (about a second)
-      unsigned x;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(a.bar) : "memory");
-      ok = x >= want;
+  if constexpr (CLUSTER) {
+    asm volatile(
+        "barrier.cluster.arrive.release.aligned;\n\t"
+        "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    return true;
+  } else {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const unsigned want = phase * gridDim.x;
+      __threadfence();  // (after the block barrier: covers the whole CTA's writes)
+      atomicAdd(a.bar, 1u);
+      int ok = 0;
+      for (int i = 0; i < (1 << 21) && !ok; ++i) {  // (about a second)
+        unsigned x;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(a.bar) : "memory");
+        ok = x >= want;
+      }
+      if (!ok) {
+        *a.co.status = GS_ERR_TIMEOUT;
+        *a.co.num_pairs_dev = 0;
+        *a.co.P = -1;  // (for the host's read of the count)
+      }
+      __threadfence();
+      s.ok = ok;
     }
-    if (!ok) {
-      *a.co.status = GS_ERR_TIMEOUT;
-      *a.co.num_pairs_dev = 0;
-      *a.co.P = -1;  // (for the host's read of the count)
-    }
-    s.ok = ok;
+    __syncthreads();
+    return s.ok != 0;
   }
-  __syncthreads();
-  return s.ok != 0;
 }
 
 // Inclusive warp scan (32-bit).
@@ -838,6 +858,7 @@ __device__ __forceinline__ unsigned warp_scan32(unsigned x) {
   return x;
 }
 
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopArgs a,
                                                                      const CamTable ct) {
   extern __shared__ __align__(16) unsigned char coop_smem[];
@@ -850,14 +871,17 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
   //    visible rows' key range; the digit counts are cleared
   const long long sub = ((n_rows + (long long)G * kCoopWarps - 1) / ((long long)G * kCoopWarps) + 31) / 32 * 32;
   const long long r0 = ((long long)cta * kCoopWarps + w) * sub, r1 = min(n_rows, r0 + sub);
+  const int groups = (int)((max(r1 - r0, 0ll) + 31) / 32);
   unsigned mine = 0u, kmin = 0xffffffffu, kmax = 0u;
-#pragma unroll 4
-  for (long long b = r0; b < r1; b += 32) {
-    const long long j = b + lane;
-    const bool in = j < r1 && a.rows.tiles_touched[j] > 0u;
-    const unsigned k = in ? __float_as_uint(a.rows.depth[j]) : 0u;
-    mine += __popc(__ballot_sync(0xffffffffu, in));
-    if (in) {
+#pragma unroll 8
+  for (int i = 0; i < groups; ++i) {
+    const long long j = r0 + 32 * i + lane;
+    const unsigned t = j < r1 ? a.rows.tiles_touched[j] : 0u;
+    const unsigned k = j < r1 ? __float_as_uint(a.rows.depth[j]) : 0u;
+    const unsigned m = __ballot_sync(0xffffffffu, t > 0u);
+    if (lane == 0) s.vis[w][i] = m;
+    mine += __popc(m);
+    if (t > 0u) {
       kmin = min(kmin, k);
       kmax = max(kmax, k);
     }
@@ -882,7 +906,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
   }
   if (tid == 0) a.cnt[cta] = total;
   unsigned phase = 1u;
-  if (!coop_barrier(a, s, phase++)) return;
+  if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
   // B. ordered compaction, with the first pass's digit counts
   unsigned before = 0u, all = 0u;
   if (tid < G) {
@@ -922,12 +946,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
     unsigned at = before + woff;
     unsigned* __restrict__ ko = a.k[buf];
     unsigned* __restrict__ vo = a.v[buf];
-#pragma unroll 2
-    for (long long b = r0; b < r1; b += 32) {
-      const long long j = b + lane;
-      const bool in = j < r1 && a.rows.tiles_touched[j] > 0u;
-      const unsigned m = __ballot_sync(0xffffffffu, in);
-      if (in) {
+#pragma unroll 8
+    for (int i = 0; i < groups; ++i) {
+      const long long j = r0 + 32 * i + lane;
+      const unsigned m = s.vis[w][i];
+      if ((m >> lane) & 1u) {
         const unsigned k = __float_as_uint(a.rows.depth[j]), pos = at + __popc(m & lt);
         if (pl.passes) {
           ko[pos] = k;
@@ -938,11 +961,25 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
       at += __popc(m);
     }
   }
-  if (!coop_barrier(a, s, phase++)) return;
+  if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
   // C. stable passes over the digits, as radix_downsweep_kernel
   const int chunks = (int)((n + (1u << shift) - 1u) >> shift);
   for (int pass = 0; pass < pl.passes; ++pass, buf ^= 1) {
     if (cta < chunks) {
+      const unsigned* __restrict__ ki = a.k[buf];
+      const unsigned* __restrict__ vi = a.v[buf];
+      const unsigned c0 = (unsigned)cta << shift, c1 = min(n, c0 + (1u << shift));
+      // (a tile's items are requested while the one before is ranked)
+      unsigned nk[kRadixIpt], nv[kRadixIpt];
+      auto request = [&](unsigned t0) {
+#pragma unroll
+        for (int i = 0; i < kRadixIpt; ++i) {
+          const unsigned p = t0 + w * (32 * kRadixIpt) + lane + 32 * i;
+          nk[i] = p < c1 ? __ldcg(ki + p) : 0u;
+          nv[i] = p < c1 ? __ldcg(vi + p) : 0u;
+        }
+      };
+      request(c0);
       // digit starts: the digits below over all chunks, then the chunks before
       const int dd = tid & (kRadixBins - 1), half = tid >> kRadixMaxBits;
       const unsigned* __restrict__ h = a.hist + (long long)pass * G * kRadixBins + dd;
@@ -972,11 +1009,8 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
         for (int i = 0; i < kRadixBins / 32; ++i) wo += i < w ? s.ws[i] : 0u;
         gbase += wo - ha + hb;
       }
-      const unsigned* __restrict__ ki = a.k[buf];
-      const unsigned* __restrict__ vi = a.v[buf];
       unsigned* __restrict__ ko = a.k[buf ^ 1];
       unsigned* __restrict__ vo = a.v[buf ^ 1];
-      const unsigned c0 = (unsigned)cta << shift, c1 = min(n, c0 + (1u << shift));
       const int dshift = pass * pl.dbits;
       const bool more = pass + 1 < pl.passes;
       for (unsigned t0 = c0; t0 < c1; t0 += kCoopTile) {
@@ -984,11 +1018,11 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
         const unsigned p0 = t0 + w * (32 * kRadixIpt) + lane;
 #pragma unroll
         for (int i = 0; i < kRadixIpt; ++i) {
-          const bool in = p0 + 32 * i < c1;
-          k[i] = in ? __ldcg(ki + p0 + 32 * i) : 0u;
-          v[i] = in ? __ldcg(vi + p0 + 32 * i) : 0u;
-          dg[i] = in ? ((k[i] - base) >> dshift) & dmask : (unsigned)kRadixBins;
+          k[i] = nk[i];
+          v[i] = nv[i];
+          dg[i] = p0 + 32 * i < c1 ? ((k[i] - base) >> dshift) & dmask : (unsigned)kRadixBins;
         }
+        if (t0 + kCoopTile < c1) request(t0 + kCoopTile);
 #pragma unroll
         for (int i = 0; i < kRadixIpt; ++i) {
           const bool valid = dg[i] < (unsigned)kRadixBins;
@@ -1053,7 +1087,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
         }
       }
     }
-    if (!coop_barrier(a, s, phase++)) return;
+    if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
   }
   // D. the rects in depth order and the counts per block of 1,024 rows (the
   //    blocks rows_expand_kernel takes); the last CTA scans them
@@ -1139,13 +1173,14 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
   }
 }
 
+template <bool CLUSTER>
 cudaError_t allow_coop_smem() {
-  return cudaFuncSetAttribute(depth_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(CoopShared));
+  return cudaFuncSetAttribute(depth_sort_kernel<CLUSTER>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CoopShared));
 }
 
 // Most CTAs of depth_sort_kernel for a cooperative launch on the current device
-// (0: not available there); cached per device.
+// (0: not available there, e.g. on part of a GPU); cached per device.
 int coop_grid() {
   static std::atomic<int> cache[64];
   int dev = 0;
@@ -1154,13 +1189,14 @@ int coop_grid() {
   if (c) return c > 0 ? c : 0;
   int per_sm = 0, sms = 0, coop = 0;
   int v = -1;
-  if (allow_coop_smem() == cudaSuccess &&
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, depth_sort_kernel, kCoopThreads,
-                                                    sizeof(CoopShared)) == cudaSuccess &&
+  if (allow_coop_smem<false>() == cudaSuccess &&
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, depth_sort_kernel<false>,
+                                                    kCoopThreads, sizeof(CoopShared)) ==
+          cudaSuccess &&
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-      per_sm > 0 && sms > 0)
-    v = std::min(kCoopGrid, sms);
+      per_sm > 0 && sms >= kCoopGrid)
+    v = kCoopGrid;
   cudaGetLastError();
   cache[dev].store(v, std::memory_order_relaxed);
   return v > 0 ? v : 0;
@@ -2062,10 +2098,31 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     CamTable cams = ct;
     void* args[] = {&a, &cams};
     // a CTA per 1,024 rows, at most one per SM: fewer CTAs meet at a barrier sooner
-    const int ctas = (int)std::min<long long>(coop, (n_rows + 1023) / 1024);
-    GS_TRY_CUDA(allow_coop_smem());
-    GS_TRY_CUDA(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(depth_sort_kernel), dim3(ctas),
-                                            dim3(kCoopThreads), args, sizeof(CoopShared), st));
+    int ctas = (int)std::min<long long>(coop, (n_rows + 1023) / 1024);
+    if (n_rows <= kClusterRows) {
+      int c = 1;  // (cluster sizes are powers of two)
+      while (c < kCoopCluster && c < ctas) c *= 2;
+      ctas = c;
+      GS_TRY_CUDA(allow_coop_smem<true>());
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(ctas);
+      cfg.blockDim = dim3(kCoopThreads);
+      cfg.dynamicSmemBytes = sizeof(CoopShared);
+      cfg.stream = st;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = ctas;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      cfg.attrs = at;
+      cfg.numAttrs = 1;
+      GS_TRY_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(depth_sort_kernel<true>),
+                                      args));
+    } else {
+      GS_TRY_CUDA(allow_coop_smem<false>());
+      GS_TRY_CUDA(cudaLaunchCooperativeKernel(
+          reinterpret_cast<const void*>(depth_sort_kernel<false>), dim3(ctas), dim3(kCoopThreads),
+          args, sizeof(CoopShared), st));
+    }
     count_launches(1);
   } else if (n_rows > 0) {
     // 1-2. stable depth sort of the visible rows (ties keep row order = id
