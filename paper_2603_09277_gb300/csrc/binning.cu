@@ -104,16 +104,18 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long x) {
 // A CTA's arrival at the end of a kernel whose last CTA goes on to a step
 // over every CTA's results (a scan of the block sums, say), in place of a
 // separate single-CTA launch.  Each CTA makes its results visible
-// (__threadfence) before it counts itself, so the CTA that counts last sees
+// (a fence by one thread behind a block barrier) before it counts itself, so the CTA that counts last sees
 // all of them; it reads them through L2 (__ldcg).  No CTA waits for another.
 // The counter is zeroed with the pipeline's counters before the launch.
 // Returns true in every thread of the last CTA.
 __device__ __forceinline__ bool last_block_arrives(unsigned long long* counter,
                                                    unsigned long long expected) {
   __shared__ int s_last;
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(counter, 1ull) == expected - 1ull ? 1 : 0;
+  if (threadIdx.x == 0) {
+    __threadfence();  // (after the block barrier: covers the whole CTA's results)
+    s_last = atomicAdd(counter, 1ull) == expected - 1ull ? 1 : 0;
+  }
   __syncthreads();
   const bool last = s_last != 0;
   if (last) __threadfence();
@@ -771,6 +773,7 @@ constexpr int kCoopThreads = 512;
 constexpr int kCoopWarps = kCoopThreads / 32;
 constexpr int kCoopTile = kCoopThreads * kRadixIpt;  // 4096 items
 constexpr int kCoopShift = 12;                       // log2(kCoopTile)
+constexpr int kCoopBlock = kScanThreads;             // rows per block of the expansion
 constexpr int kCoopGrid = 152;                       // most CTAs (one per SM)
 constexpr long long kCoopRows = 2ll << 20;
 // Row groups of 32 of a warp: at most kCoopRows over the warps of the whole
@@ -809,7 +812,7 @@ struct CoopShared {
   unsigned ws[kCoopWarps], ws2[kCoopWarps];
   unsigned vis[kCoopWarps][kCoopGroups];    // visible lanes of the warp's rows
   unsigned long long wt[2][9];
-  int ok, last;
+  int ok;
 };
 
 // Barrier number `phase` (1, 2, ...) over the grid.  CLUSTER: the grid is one
@@ -1089,28 +1092,30 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
     }
     if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
   }
-  // D. the rects in depth order and the counts per block of 1,024 rows (the
-  //    blocks rows_expand_kernel takes); the last CTA scans them
+  // D. the rects in depth order and the counts per block of 256 rows (the
+  //    blocks rows_expand_kernel<1> takes), a warp per block and 8 rows per
+  //    lane; the last CTA scans them
   const unsigned* __restrict__ rows = a.v[0];
-  const int nb = (int)((n + kScanTile - 1) / kScanTile);
-  for (int b = cta; b < nb; b += G) {
+  const int nb = (int)((n + kCoopBlock - 1) / kCoopBlock);
+  for (int b = cta + G * w; b < nb; b += G * kCoopWarps) {
     unsigned long long q = 0ull, pp = 0ull;
-    unsigned row[2];
-    int4 rr[2];
+    constexpr int kPer = kCoopBlock / 32;
+    unsigned row[kPer];
+    int4 rr[kPer];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const unsigned at = (unsigned)b * kScanTile + i * kCoopThreads + tid;
+    for (int i = 0; i < kPer; ++i) {
+      const unsigned at = (unsigned)b * kCoopBlock + 32 * i + lane;
       row[i] = at < n ? __ldcg(rows + at) : 0xffffffffu;
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kPer; ++i) {
       rr[i] = make_int4(0, 0, 0, 0);
       if (row[i] != 0xffffffffu && GS_IN_BOUNDS(row[i], n_rows, 205))
         rr[i] = a.rect8 ? unpack_rect8(a.rect8[row[i]]) : view_rect(a.rect, row[i], a.N, ct);
     }
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const unsigned at = (unsigned)b * kScanTile + i * kCoopThreads + tid;
+    for (int i = 0; i < kPer; ++i) {
+      const unsigned at = (unsigned)b * kCoopBlock + 32 * i + lane;
       if (at < n) {
         a.rect_sorted[at] = pack_rect(rr[i]);
         q += st_count(rr[i]);
@@ -1122,25 +1127,12 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
       q += __shfl_xor_sync(0xffffffffu, q, o);
       pp += __shfl_xor_sync(0xffffffffu, pp, o);
     }
-    unsigned long long* red = reinterpret_cast<unsigned long long*>(s.key);
-    __syncthreads();
     if (lane == 0) {
-      red[w] = q;
-      red[kCoopWarps + w] = pp;
-    }
-    __syncthreads();
-    if (tid < 2) {
-      unsigned long long t = 0ull;
-      for (int i = 0; i < kCoopWarps; ++i) t += red[tid * kCoopWarps + i];
-      (tid ? a.co.sums_p : a.co.sums_q)[b] = t;
+      a.co.sums_q[b] = q;
+      a.co.sums_p[b] = pp;
     }
   }
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s.last = atomicAdd(a.arrive, 1ull) == (unsigned long long)G - 1ull;
-  __syncthreads();
-  if (!s.last) return;
-  __threadfence();
+  if (!last_block_arrives(a.arrive, (unsigned long long)G)) return;
   // warps 0-7 scan the super-tile counts, 8-15 the pair counts: each warp a
   // contiguous part of the blocks
   const int which = w >> 3, wi = w & 7;
@@ -1435,52 +1427,17 @@ __device__ __forceinline__ Segment load_segment(const Segment* __restrict__ segs
 // Segments of every super-tile: seg_first[s] (exclusive scan of
 // ceil(len_s / kSeg)), seg_first[S] = total, segs[g] and (when not NULL)
 // seg_st[g] = super-tile of g.
-// One CTA of 1024 threads.
-__global__ void __launch_bounds__(1024) st_segments_kernel(uint2* __restrict__ st_ranges,
-                                                           int S, const unsigned* __restrict__ totals,
-                                                           const long long* __restrict__ q_eff,
-                                                           unsigned* __restrict__ seg_first,
-                                                           Segment* __restrict__ segs,
-                                                           unsigned* __restrict__ seg_st,
-                                                           const CamTable ct,
-                                                           long long* __restrict__ n_seg) {
+// One CTA of 1024 threads; for more than 256 super-tiles (up to that many
+// st_count_kernel forms the segments itself).
+__global__ void __launch_bounds__(1024) st_segments_kernel(
+    const uint2* __restrict__ st_ranges, int S, unsigned* __restrict__ seg_first,
+    Segment* __restrict__ segs, unsigned* __restrict__ seg_st, const CamTable ct,
+    long long* __restrict__ n_seg) {
   __shared__ unsigned s_w[32];
   __shared__ unsigned s_carry;
   __shared__ Segment s_seg[1024];    // the super-tile's whole range, tile and shape
   __shared__ unsigned s_first[1024];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  if (totals) {
-    // one radix pass sorted the items by super-tile (S <= 512): the per-digit
-    // totals are the per-super-tile counts, and their exclusive scan the starts
-    // (S <= 256: the first 8 warps, one block-level scan)
-    const unsigned tot = tid < S ? totals[tid] : 0u;
-    unsigned incl = tot;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += y;
-    }
-    if (lane == 31) s_w[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-      const unsigned x = s_w[lane];
-      unsigned xi = x;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, xi, o);
-        if (lane >= o) xi += y;
-      }
-      s_w[lane] = xi - x;
-    }
-    __syncthreads();
-    if (tid < S) {
-      const unsigned run = s_w[w] + incl - tot;
-      st_ranges[tid] = make_uint2(tot ? run : 0u, tot ? run + tot : 0u);
-    }
-  } else if (S == 1 && tid == 0) {  // no sort: one super-tile holds every item
-    const unsigned q = (unsigned)*q_eff;
-    st_ranges[0] = make_uint2(0u, q);
-  }
   if (tid == 0) s_carry = 0u;
   __syncthreads();
   for (int base = 0; base < S; base += 1024) {
@@ -1571,23 +1528,91 @@ __device__ __forceinline__ void mma_count(float d[4], unsigned a0, unsigned a2, 
       : "r"(a0), "r"(0u), "r"(a2), "r"(b0), "r"(b1));
 }
 
+// With `totals` (the items were sorted by super-tile in at most one pass: S <=
+// 256) every CTA forms the segments itself from the super-tiles' item counts,
+// two scans of 256 values, and writes the table entries of the segments it
+// takes, instead of a launch of st_segments_kernel before.
+__device__ __forceinline__ unsigned block_scan256(unsigned x, unsigned* s_w) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned inc = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) s_w[w] = inc;
+  __syncthreads();
+  unsigned wo = 0u;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) wo += i < w ? s_w[i] : 0u;
+  __syncthreads();
+  return wo + inc - x;
+}
+
 __global__ void __launch_bounds__(256) st_count_kernel(
     const unsigned* __restrict__ sp_keys, const unsigned* __restrict__ sp_rows,
-    const Segment* __restrict__ segs, const unsigned* __restrict__ seg_st,
-    const long long* __restrict__ n_seg, int packed, const int* __restrict__ rect, int N,
-    const CamTable ct, unsigned* __restrict__ desc, unsigned* __restrict__ hist) {
+    Segment* __restrict__ segs, const unsigned* __restrict__ seg_st,
+    long long* __restrict__ n_seg, int packed, const int* __restrict__ rect, int N,
+    const CamTable ct, unsigned* __restrict__ desc, unsigned* __restrict__ hist,
+    const unsigned* __restrict__ totals, const long long* __restrict__ q_eff, int S,
+    unsigned* __restrict__ seg_first) {
   __shared__ unsigned s_cnt[8][64];
   constexpr int kPer = kSeg / 8;  // items of a warp
   __shared__ __align__(16) unsigned short s_desc[8][kPer];
+  __shared__ unsigned s_start[256], s_first[257];  // (totals) items, segments before a super-tile
+  __shared__ unsigned s_w[8];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int t = lane & 3, q = lane >> 2;  // the lane's four items of 16; its tile row and column
   const int sr = 14 - q, sc = 6 - q;      // moves its bits to bit 14 (a rotation by -1 for column 7)
-  const long long G = *n_seg;
+  long long G;
+  const bool own = totals || S == 1;  // the segments are formed here
+  if (own) {
+    const unsigned items = tid < S ? (S == 1 ? (unsigned)*q_eff : totals[tid]) : 0u;
+    const unsigned start = block_scan256(items, s_w);
+    const unsigned first = block_scan256((items + kSeg - 1) / kSeg, s_w);
+    s_start[tid] = start;
+    s_first[tid] = first;
+    if (tid == 255) s_first[256] = first + (items + kSeg - 1) / kSeg;
+    __syncthreads();
+    G = s_first[256];
+    if (blockIdx.x == 0) {
+      if (tid < S) seg_first[tid] = first;
+      if (tid == 0) {
+        seg_first[S] = (unsigned)G;
+        *n_seg = G;
+      }
+    }
+  } else {
+    G = *n_seg;
+  }
   for (long long g = blockIdx.x; g < G; g += gridDim.x) {
-    const Segment si = load_segment(segs, g);
+    Segment si;
+    int s = 0;
+    if (own) {
+      // the last super-tile whose segments start at or before g (those without
+      // segments share their start with the next)
+      int hi = S - 1;
+      while (s < hi) {
+        const int mid = (s + hi + 1) >> 1;
+        if (s_first[mid] <= (unsigned)g) s = mid;
+        else hi = mid - 1;
+      }
+      const unsigned end = s + 1 < 256 ? s_start[s + 1] : (unsigned)*q_eff;
+      si.b = s_start[s] + ((unsigned)g - s_first[s]) * (unsigned)kSeg;
+      si.e = min(s + 1 < S ? end : (unsigned)*q_eff, si.b + (unsigned)kSeg);
+      const CamInfo& c = ct.c[view_of_st(ct, s)];
+      const int sl = s - c.st_off;
+      const int ox = (sl % c.STX) * kSuperTile, oy = (sl / c.STX) * kSuperTile;
+      si.tile = c.tile_off + oy * c.TX + ox;
+      si.shape = (unsigned)c.TX | (unsigned)min(kSuperTile, c.TX - ox) << 16 |
+                 (unsigned)min(kSuperTile, c.TY - oy) << 20;
+      if (tid == 0) segs[g] = si;
+    } else {
+      si = load_segment(segs, g);
+      if (!packed) s = (int)seg_st[g];
+    }
     int ox = 0, oy = 0;
     if (!packed) {
-      const int s = (int)seg_st[g];
       const CamInfo& c = ct.c[view_of_st(ct, s)];
       ox = ((s - c.st_off) % c.STX) * kSuperTile;
       oy = ((s - c.st_off) / c.STX) * kSuperTile;
@@ -1967,7 +1992,9 @@ Workspace carve(void* base, long long n_rows, long long cap, long long tiles) {
     off += align256(bytes);
     return r;
   };
-  const long long nb = scan_blocks(n_rows > cap ? n_rows : cap) + 1;
+  // (blocks of 256 rows up to kCoopRows, of 1,024 or 4,096 above)
+  const long long nb = std::max(scan_blocks(n_rows > cap ? n_rows : cap),
+                                (std::min(n_rows, kCoopRows) + kCoopBlock - 1) / kCoopBlock) + 1;
   const long long ms = max_segments(cap, tiles);
   w.block_sums = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * nb));
   w.block_sums2 = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * nb));
@@ -2075,7 +2102,7 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
   // the projection's 8-bit packed rects (views of at most 255 tiles per side)
   const unsigned* rect8 = rect8_fits(ct) ? proj->rect8 : nullptr;
   const bool small = n_rows <= (4ll << 20);
-  const int items = small ? 4 : 16;
+  const int items = coop ? 1 : small ? 4 : 16;
   const long long nb = (n_rows + kScanThreads * items - 1) / (kScanThreads * items);
   if (n_rows > 0 && coop) {
     // 1-3. in one launch
@@ -2199,7 +2226,11 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
                        reinterpret_cast<uintptr_t>(sk[0]) % 16 == 0) ? 1 : 0;
     unsigned* h = hist0 ? w.hist : nullptr;
     const unsigned hmask = (1u << radix_plan_bits(0u, sbits).d0) - 1u;
-    if (small)
+    if (coop)
+      rows_expand_kernel<1><<<(unsigned)nb, kScanThreads, 0, st>>>(
+          rows_sorted, w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N),
+          ct, sk[0], sv[0], vec16, packed, h, sgrid, hmask);
+    else if (small)
       rows_expand_kernel<4><<<(unsigned)nb, kScanThreads, 0, st>>>(
           rows_sorted, w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N),
           ct, sk[0], sv[0], vec16, packed, h, sgrid, hmask);
@@ -2227,12 +2258,16 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
                                       w.st_ranges);
     count_launches(1);
   }
-  st_segments_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<uint2*>(w.st_ranges), S, st_totals,
-                                         q_eff, w.seg_first, w.segs,
-                                         packed ? nullptr : w.seg_st, ct, n_seg);
+  if (spasses > 1) {  // (else st_count_kernel forms the segments)
+    st_segments_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<const uint2*>(w.st_ranges), S,
+                                           w.seg_first, w.segs, packed ? nullptr : w.seg_st, ct,
+                                           n_seg);
+    count_launches(1);
+  }
   const unsigned gs = (unsigned)std::min<long long>(max_segments(q_bound, S), 152ll * 8);
   st_count_kernel<<<gs, 256, 0, st>>>(sp_keys, sp_rows, w.segs, w.seg_st, n_seg, packed,
-                                      proj->rect, N, ct, desc, w.seg_hist);
+                                      proj->rect, N, ct, desc, w.seg_hist, st_totals, q_eff, S,
+                                      w.seg_first);
   st_scan_kernel<<<(unsigned)S, 1024, 0, st>>>(w.seg_first, ct,
                                                reinterpret_cast<uint4*>(w.seg_hist), w.tile_cnt,
                                                arrive + 2, w.tile_start, ranges);
@@ -2254,7 +2289,7 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     const int e = stage_event(GS_STAGE_EXPANSION, true, st);
     if (e != GS_OK) return e;
   }
-  count_launches(4);
+  count_launches(3);
   return check_launch();
 }
 
