@@ -1561,6 +1561,8 @@ __global__ void __launch_bounds__(256) st_count_kernel(
   __shared__ __align__(16) unsigned short s_desc[8][kPer];
   __shared__ unsigned s_start[256], s_first[257];  // (totals) items, segments before a super-tile
   __shared__ unsigned s_w[8];
+  __shared__ __align__(16) Segment s_seg[256];  // (totals) the CTA's segments
+  __shared__ unsigned char s_st[256];           // and their super-tiles
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int t = lane & 3, q = lane >> 2;  // the lane's four items of 16; its tile row and column
   const int sr = 14 - q, sc = 6 - q;      // moves its bits to bit 14 (a rotation by -1 for column 7)
@@ -1585,32 +1587,37 @@ __global__ void __launch_bounds__(256) st_count_kernel(
   } else {
     G = *n_seg;
   }
-  for (long long g = blockIdx.x; g < G; g += gridDim.x) {
-    Segment si;
-    int s = 0;
-    if (own) {
-      // the last super-tile whose segments start at or before g (those without
-      // segments share their start with the next)
-      int hi = S - 1;
-      while (s < hi) {
-        const int mid = (s + hi + 1) >> 1;
-        if (s_first[mid] <= (unsigned)g) s = mid;
-        else hi = mid - 1;
+  for (long long g = blockIdx.x, it = 0; g < G; g += gridDim.x, ++it) {
+    if (own && (it & 255) == 0) {
+      // the CTA's next 256 segments, one per thread
+      const long long gt = g + (long long)tid * gridDim.x;
+      __syncthreads();
+      if (gt < G) {
+        // the last super-tile whose segments start at or before gt (those
+        // without segments share their start with the next)
+        int s = 0;
+        for (int hi = S - 1; s < hi;) {
+          const int mid = (s + hi + 1) >> 1;
+          if (s_first[mid] <= (unsigned)gt) s = mid;
+          else hi = mid - 1;
+        }
+        Segment si;
+        si.b = s_start[s] + ((unsigned)gt - s_first[s]) * (unsigned)kSeg;
+        si.e = min(s + 1 < S ? s_start[s + 1] : (unsigned)*q_eff, si.b + (unsigned)kSeg);
+        const CamInfo& c = ct.c[view_of_st(ct, s)];
+        const int sl = s - c.st_off;
+        const int ox = (sl % c.STX) * kSuperTile, oy = (sl / c.STX) * kSuperTile;
+        si.tile = c.tile_off + oy * c.TX + ox;
+        si.shape = (unsigned)c.TX | (unsigned)min(kSuperTile, c.TX - ox) << 16 |
+                   (unsigned)min(kSuperTile, c.TY - oy) << 20;
+        s_seg[tid] = si;
+        s_st[tid] = (unsigned char)s;
+        segs[gt] = si;
       }
-      const unsigned end = s + 1 < 256 ? s_start[s + 1] : (unsigned)*q_eff;
-      si.b = s_start[s] + ((unsigned)g - s_first[s]) * (unsigned)kSeg;
-      si.e = min(s + 1 < S ? end : (unsigned)*q_eff, si.b + (unsigned)kSeg);
-      const CamInfo& c = ct.c[view_of_st(ct, s)];
-      const int sl = s - c.st_off;
-      const int ox = (sl % c.STX) * kSuperTile, oy = (sl / c.STX) * kSuperTile;
-      si.tile = c.tile_off + oy * c.TX + ox;
-      si.shape = (unsigned)c.TX | (unsigned)min(kSuperTile, c.TX - ox) << 16 |
-                 (unsigned)min(kSuperTile, c.TY - oy) << 20;
-      if (tid == 0) segs[g] = si;
-    } else {
-      si = load_segment(segs, g);
-      if (!packed) s = (int)seg_st[g];
+      __syncthreads();
     }
+    const Segment si = own ? s_seg[it & 255] : load_segment(segs, g);
+    const int s = packed ? 0 : own ? (int)s_st[it & 255] : (int)seg_st[g];
     int ox = 0, oy = 0;
     if (!packed) {
       const CamInfo& c = ct.c[view_of_st(ct, s)];

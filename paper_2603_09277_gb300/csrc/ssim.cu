@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
   block_partial(acc, (double)sv.scale[k.v], partials + blockIdx.x);
 }
 
-__global__ void __launch_bounds__(kSsimThreads, 4) ssim_bwd_kernel(
+__global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     const float* __restrict__ maps, long long P, float* __restrict__ dimg) {
   __shared__ __align__(16) float2 s_ab[kSsimS][kSsimP];  // (a - 2 (mu_x - c) b - (mu_y - c') e, b)
