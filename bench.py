@@ -60,13 +60,14 @@ L2_BYTES = 129 * 1024 * 1024
 #   forward:  10 per evaluated pair (pixel offset 2, base-2 exponent 8)
 #             +14 per blended pair (exp, clamp, 1-alpha, T(1-alpha), w,
 #                 colour 3 FMA, log, entropy FMA)
-#   backward: 10 per evaluated pair, +56 per blended pair (transmittance
-#             recovery 8, colour part of dL/dalpha 14, entropy part 7, colour
-#             gradient 3, S and R updates 9, dd and the six moments
-#             dd (1, dx, dy, dx^2, dx dy, dy^2) summed 12, colour sums 3; the
-#             conic, 1/sigma and the signs are applied once per Gaussian)
+#   backward: 10 per evaluated pair, +40 per blended pair (transmittance
+#             recovery 8, g . c 5, log w 2, the common factor of the colour and
+#             entropy parts 2, dL/dalpha 3, the running sum g . S - gH R 2,
+#             colour gradient 3, dd and the six moments dd (1, p, q, p^2, p q,
+#             q^2) summed 12, colour sums 3; the conic, 1/sigma and the signs
+#             are applied once per Gaussian)
 FWD_EVAL, FWD_BLEND = 10, 14
-BWD_EVAL, BWD_BLEND = 10, 56
+BWD_EVAL, BWD_BLEND = 10, 40
 
 
 def log(*a):
@@ -309,6 +310,17 @@ def run_reference(args):
 # ---------------------------------------------------------------------------
 # GPU arm
 # ---------------------------------------------------------------------------
+def reached_rows(r):
+    """Rows the latest backward's blending reached and the Gaussians reached in
+    some view, from the bitmap in grad2d's pad floats (bit row % 32 of float 10
+    of row row // 32)."""
+    import numpy as np
+    import torch
+    words = r.grad2d[:(r.rows + 31) // 32, 10].contiguous().view(torch.int32).cpu().numpy()
+    bits = np.unpackbits(words.view(np.uint8), bitorder="little")[:r.rows].reshape(r.V, r.N)
+    return int(bits.sum()), int(bits.any(0).sum())
+
+
 def traffic_from_profiles(kernel, config):
     """DRAM bytes per launch of `kernel` on workload `config` from the
     committed ncu summary (profiles/traffic.json: a list of entries, one per
@@ -879,6 +891,7 @@ def main():
     vis_rows = (r.tiles_touched[:r.rows] > 0)
     n_rows_vis = int(vis_rows.sum().item())
     n_gauss_vis = int(vis_rows.view(r.V, r.N).any(0).sum().item())
+    n_rows_t, n_gauss_t = reached_rows(r)
     Kc = (int(prm.get("sh_degree", 0)) + 1) ** 2
     n_g = int(scene["means"].shape[0])
     rec_b = gs.gs_record_bytes(r.prm_c.attr_dtype)
@@ -899,9 +912,9 @@ def main():
                               n_rows_vis * rec_b),
         # the super-tile items (packed key, row) read, every pair written once
         "st_emit_kernel": ("hbm", Q * 8 + P * 4),
-        # the moment row of every visible row; parameters read and gradients
-        # written of every seen Gaussian
-        "preprocess_bwd_kernel": ("hbm", n_rows_vis * 48 + n_gauss_vis * (44 + 12 * Kc) * 2),
+        # the moment row of every row the blending reached; parameters read and
+        # gradients written of every Gaussian reached in some view
+        "preprocess_bwd_kernel": ("hbm", n_rows_t * 48 + n_gauss_t * (44 + 12 * Kc) * 2),
     }
     kname = max(kernel_ms, key=kernel_ms.get)
     kms = kernel_ms[kname]
