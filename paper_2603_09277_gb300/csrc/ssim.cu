@@ -6,16 +6,19 @@
 // Forward, one CTA per 32x32 block of output pixels of one view, one channel
 // after the other: the block and its 5-pixel halo of image and target are
 // staged in shared memory as pairs (x, y).  The window moments are taken about
-// a constant per block and channel (the staged value at the block centre, c):
-// with d = s - c (padding samples s = 0), mu = c + E[d] and sigma^2 = E[d^2] -
-// E[d]^2 hold exactly for any constant, and around a value of the block two
-// large FP32 sums do not cancel in smooth regions.  Because c is constant over
-// the block, the 11x11 window sums are separable: a horizontal pass over the 42
-// staged rows and a vertical pass per output pixel.  Per pixel and channel the
-// forward saves (mu_x, mu_y, dS/dmu_x, dS/dsigma_x^2, dS/dsigma_xy) (planar, one
-// plane per quantity) and adds lambda (1 - S) / (3 M_v V) to the loss partials.
+// a constant per 16x16 quarter of the block and channel (the staged value at the
+// quarter's centre, c): with d = s - c (padding samples s = 0), mu = c + E[d] and
+// sigma^2 = E[d^2] - E[d]^2 hold exactly for any constant, and around a value of
+// the quarter two large FP32 sums do not cancel in smooth regions.  Because c is
+// constant over a quarter, the 11x11 window sums are separable: a horizontal pass
+// over the 26 staged rows of each row of quarters and a vertical pass per output
+// pixel.  Per pixel and channel the forward saves (mu_x, mu_y, dS/dmu_x,
+// dS/dsigma_x^2, dS/dsigma_xy) (planar, one plane per quantity) and adds
+// lambda (1 - S) / (3 M_v V) to the loss partials: a warp sums, in FP32, the 16
+// columns and 8 rows of one quarter that it holds, everything above in FP64, so
+// the loss does not depend on how blocks and channels are dealt to CTAs.
 //
-// Backward, same blocking:
+// Backward, blocks of 32x32 with one constant per block and channel:
 //   dL/dx(p) -= lambda / (3 M_v V) sum_q G(q - p) [a(q)
 //               + 2 (x(p) - mu_x(q)) b(q) + (y(p) - mu_y(q)) e(q)]
 // over the window centres q inside the image, with a = dS/dmu_x, b =
@@ -26,11 +29,15 @@
 //
 // What bounds them: instruction issue (the window sums; about 60 FP32
 // operations per pixel, channel and moment).  Blocks of 32 instead of 16 pixels
-// cut the halo rows of the horizontal pass from 1.6 to 1.3 per output row, one
-// channel at a time keeps the shared memory of a CTA at 42 KB (5 CTAs per SM;
-// three channels of 16x16 blocks took 67 KB in the backward, 33 % issue active),
-// packed FP32 pairs halve the instructions of paired quantities, and the
-// backward runs three correlations where it ran five.
+// cut the halo rows of the backward's horizontal pass from 1.6 to 1.3 per output
+// row and what both stage from 2.6 to 1.7 samples per pixel, one channel at a
+// time keeps the shared memory of a CTA at 38 to 48 KB (4 to 5 CTAs per SM; three
+// channels of 16x16 blocks took 67 KB in the backward, 33 % issue active), packed
+// FP32 pairs halve the instructions of paired quantities, and the backward runs
+// three correlations where it ran five.  The whole loss on two 1237x822 views: 204
+// us against 315 with 16x16 blocks of three channels, 1920x1080: 202 against 317.
+// (One constant per 32x32 block in the forward too is 3 % faster, but its moments
+// about a farther constant move the loss of a small image by 1e-8.)
 #include <cmath>
 
 #include "gs_internal.cuh"
@@ -43,7 +50,10 @@ constexpr int kSsimTaps = 2 * kSsimR + 1;
 constexpr int kSsimB = 32;                  // output block side
 constexpr int kSsimS = kSsimB + 2 * kSsimR; // staged side (42)
 constexpr int kSsimP = 44;                  // staged row pitch (16-byte rows of 4 samples)
+constexpr int kQ = 16;                      // side of the forward's quarters
+constexpr int kQS = kQ + 2 * kSsimR;        // staged rows of a quarter (26)
 constexpr int kSsimThreads = 256;
+constexpr int kSsimSplitBlocks = 2 * 4 * 152;  // see ssim_parts
 constexpr float kC1 = 0.01f * 0.01f;
 constexpr float kC2 = 0.03f * 0.03f;
 
@@ -68,23 +78,18 @@ __device__ __forceinline__ int view_of_block(const SsimViews& sv, int b) {
 // in tap order.
 constexpr int kRun = 4;                              // outputs per thread and pass
 constexpr int kSpan = kRun + 2 * kSsimR;             // samples per run (14)
-constexpr int kHItems = kSsimS * (kSsimB / kRun);    // horizontal runs (336)
+constexpr int kHItems = kSsimS * (kSsimB / kRun);    // the backward's horizontal runs (336)
+constexpr int kQItems = 2 * kQS * (kSsimB / kRun);   // the forward's (416)
+constexpr int kXP = 36;                              // pitch of s_x: two rows of 16 columns
+                                                     // four rows apart, no bank conflict
 static_assert(kSsimB * (kSsimB / kRun) == kSsimThreads, "one vertical run per thread");
 static_assert(kSsimB == 32, "a warp is a row of the block in the vertical pass");
 
-// Exclusive per-block partial of sum (1 - S) (FP32 within the thread and the
-// warp: every term is >= 0; FP64 across the warps).
-__device__ __forceinline__ void block_partial(float acc, double scale, double* out) {
-  __shared__ double s_red[kSsimThreads / 32];
+// Sum of a warp's FP32 terms (every term is >= 0).
+__device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = (double)acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int k = 0; k < kSsimThreads / 32; ++k) t += s_red[k];
-    *out = t * scale;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
 // The block of CTA b: its view, origin, extents and first pixel.
@@ -104,18 +109,32 @@ __device__ __forceinline__ SsimBlock ssim_block(const SsimViews& sv, int b) {
   return k;
 }
 
+// The channels of a CTA: all three, or one where the grid has three CTAs per
+// block (launch_ssim says when).
+struct ChannelRange {
+  int first, end;
+};
+__device__ __forceinline__ ChannelRange channels_of(unsigned parts, unsigned part) {
+  return parts == 1 ? ChannelRange{0, 3} : ChannelRange{(int)part, (int)part + 1};
+}
+
 __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     float* __restrict__ maps /* 15 planes of P */, long long P, double* __restrict__ partials) {
   __shared__ __align__(16) float2 s_xy[kSsimS][kSsimP];
-  __shared__ __align__(16) float2 s_m[kSsimS][kSsimB];   // horizontal sums of (x, y)
-  __shared__ __align__(16) float2 s_q[kSsimS][kSsimB];   // of (x^2, y^2)
-  __shared__ __align__(16) float s_x[kSsimS][kSsimB];    // of x y
+  __shared__ __align__(16) float2 s_m[2 * kQS][kSsimB];  // horizontal sums of (x, y)
+  __shared__ __align__(16) float2 s_q[2 * kQS][kSsimB];  // of (x^2, y^2)
+  __shared__ __align__(16) float s_x[2 * kQS][kXP];      // of x y
+  __shared__ double s_sum[kSsimThreads / 32];
   const SsimBlock k = ssim_block(sv, blockIdx.x);
-  const int col = threadIdx.x & 31, y0 = (threadIdx.x >> 5) * kRun;
-  float acc = 0.f;
+  // a warp's outputs: 16 columns and two runs of 4 rows of quarter (qx, qy)
+  const int warp = threadIdx.x >> 5, qx = (warp >> 1) & 1, qy = warp >> 2;
+  const int col = qx * kQ + (threadIdx.x & 15);
+  const int y0 = (2 * (warp & 1) + ((threadIdx.x >> 4) & 1)) * kRun;  // in the quarter
+  const ChannelRange cr = channels_of(gridDim.y, blockIdx.y);
+  double sum = 0.0;
 #pragma unroll 1
-  for (int ch = 0; ch < 3; ++ch) {
+  for (int ch = cr.first; ch < cr.end; ++ch) {
     for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
       const int r = i / kSsimS, c = i - r * kSsimS;
       const int yy = k.by - kSsimR + r, xx = k.bx - kSsimR + c;
@@ -124,11 +143,13 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
       s_xy[r][c] = in ? make_float2(image[p], target[p]) : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    const float2 cc = s_xy[kSsimR + kSsimB / 2][kSsimR + kSsimB / 2];
-    const float2 ncc = make_float2(-cc.x, -cc.y);
-    // horizontal: run (staged row r, columns x0 .. x0 + kRun - 1)
-    for (int it = threadIdx.x; it < kHItems; it += kSsimThreads) {
+    // horizontal: run (row r of the row of quarters hq, columns x0 .. x0 + kRun - 1)
+    for (int it = threadIdx.x; it < kQItems; it += kSsimThreads) {
       const int r = it / (kSsimB / kRun), x0 = (it % (kSsimB / kRun)) * kRun;
+      const int hq = r >= kQS ? 1 : 0, sr = r - hq * (kQS - kQ);  // (its staged row)
+      const float2 c =
+          s_xy[kSsimR + hq * kQ + kQ / 2][kSsimR + (x0 & kQ) + kQ / 2];
+      const float2 ncc = make_float2(-c.x, -c.y);
       float2 m[kRun], q[kRun];
       float x[kRun];
 #pragma unroll
@@ -138,7 +159,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
       }
 #pragma unroll
       for (int j = 0; j < kSpan; j += 2) {
-        const float4 t = *reinterpret_cast<const float4*>(&s_xy[r][x0 + j]);
+        const float4 t = *reinterpret_cast<const float4*>(&s_xy[sr][x0 + j]);
         const float2 d[2] = {__fadd2_rn(make_float2(t.x, t.y), ncc),
                              __fadd2_rn(make_float2(t.z, t.w), ncc)};
 #pragma unroll
@@ -162,7 +183,10 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
       *reinterpret_cast<float4*>(&s_x[r][x0]) = make_float4(x[0], x[1], x[2], x[3]);
     }
     __syncthreads();
-    // vertical: column col, output rows y0 .. y0 + kRun - 1
+    // vertical: column col, output rows y0 .. y0 + kRun - 1 of the quarter
+    const float2 cc = s_xy[kSsimR + qy * kQ + kQ / 2][kSsimR + qx * kQ + kQ / 2];
+    const int r0 = qy * kQS + y0;
+    float acc = 0.f;
     float2 m[kRun], q[kRun];
     float x[kRun];
 #pragma unroll
@@ -172,8 +196,8 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
     }
 #pragma unroll
     for (int j = 0; j < kSpan; ++j) {
-      const float2 tm = s_m[y0 + j][col], tq = s_q[y0 + j][col];
-      const float tx = s_x[y0 + j][col];
+      const float2 tm = s_m[r0 + j][col], tq = s_q[r0 + j][col];
+      const float tx = s_x[r0 + j][col];
 #pragma unroll
       for (int o = 0; o < kRun; ++o) {
         const int tap = j - o;
@@ -186,7 +210,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
     const int px = k.bx + col;
 #pragma unroll
     for (int o = 0; o < kRun; ++o) {
-      const int py = k.by + y0 + o;
+      const int py = k.by + qy * kQ + y0 + o;
       if (px < k.W && py < k.H) {
         const long long p = k.base + (long long)py * k.W + px;
         const float m1 = m[o].x, n1 = m[o].y;
@@ -206,9 +230,16 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
         mp[4 * P] = 2.f * A1 / D;                              // dS/dsigma_xy
       }
     }
+    sum += (double)warp_sum(acc);
     __syncthreads();  // (the staged channel is overwritten)
   }
-  block_partial(acc, (double)sv.scale[k.v], partials + blockIdx.x);
+  if ((threadIdx.x & 31) == 0) s_sum[warp] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < kSsimThreads / 32; ++w) t += s_sum[w];
+    partials[blockIdx.x + gridDim.x * blockIdx.y] = t * (double)sv.scale[k.v];
+  }
 }
 
 __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
@@ -221,8 +252,9 @@ __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
   const SsimBlock k = ssim_block(sv, blockIdx.x);
   const int col = threadIdx.x & 31, y0 = (threadIdx.x >> 5) * kRun;
   const long long p0 = 3 * (k.base + (long long)k.by * k.W + k.bx);
+  const ChannelRange cr = channels_of(gridDim.y, blockIdx.y);
 #pragma unroll 1
-  for (int ch = 0; ch < 3; ++ch) {
+  for (int ch = cr.first; ch < cr.end; ++ch) {
     // block constants: the image and target at the block's first pixel
     const float cx = image[p0 + ch], cy = target[p0 + ch];
     const float* __restrict__ mp = maps + (long long)(5 * ch) * P;
@@ -311,14 +343,24 @@ size_t ssim_workspace_bytes(long long total_pixels) {
   return sizeof(float) * 15 * (size_t)total_pixels;
 }
 
+namespace {
+// CTAs per block of pixels: three, one per channel, up to two waves of 4 CTAs on
+// 152 SMs; beyond, one CTA for all three, which reads a pixel's channels from the
+// same lines.  Measured (whole loss, three CTAs against one): 8 blocks 16.3
+// against 32.8 us, 70 blocks 20.8 against 37.6, 260 blocks 36.8 against 45.3,
+// 1,014 blocks 105.8 against 111.8, 2,028 blocks 218 against 205.
+int ssim_parts(long long blocks) { return blocks <= kSsimSplitBlocks ? 3 : 1; }
+}  // namespace
+
+// The partials that launch_ssim writes.
 int ssim_blocks(const CamTable& ct) {
   long long n = 0;
   for (int v = 0; v < ct.V; ++v)
     n += (long long)((ct.c[v].W + kSsimB - 1) / kSsimB) * ((ct.c[v].H + kSsimB - 1) / kSsimB);
-  return (int)n;
+  return (int)n * ssim_parts(n);
 }
 
-// Adds lambda (1 - SSIM_v) / V per view to the partials (one per block) and
+// Adds lambda (1 - SSIM_v) / V per view to the partials (ssim_blocks of them) and
 // the term's gradient to dimg; maps is ssim_workspace_bytes(P) of scratch.
 int launch_ssim(const float* image, const float* target, const CamTable& ct, float lambda,
                 float* maps, double* partials, float* dimg, cudaStream_t st) {
@@ -346,8 +388,9 @@ int launch_ssim(const float* image, const float* target, const CamTable& ct, flo
   const int nb = sv.block_off[ct.V];
   if (nb == 0) return GS_OK;
   const long long P = ct.c[ct.V - 1].pix_off + (long long)ct.c[ct.V - 1].W * ct.c[ct.V - 1].H;
-  ssim_fwd_kernel<<<nb, kSsimThreads, 0, st>>>(image, target, sv, maps, P, partials);
-  ssim_bwd_kernel<<<nb, kSsimThreads, 0, st>>>(image, target, sv, maps, P, dimg);
+  const dim3 grid(nb, ssim_parts(nb));
+  ssim_fwd_kernel<<<grid, kSsimThreads, 0, st>>>(image, target, sv, maps, P, partials);
+  ssim_bwd_kernel<<<grid, kSsimThreads, 0, st>>>(image, target, sv, maps, P, dimg);
   count_launches(2);
   return check_launch();
 }
