@@ -240,7 +240,11 @@ int gs_preprocess(const float* means, const float* log_scales, const float* quat
  *   (nothing beyond the count is then written).  If NULL (the form for CUDA
  *   graph capture) nothing is synchronised; on overflow the device writes
  *   *status_dev = GS_ERR_CAPACITY, keeps P in *num_pairs_dev, empties every
- *   range, and the caller regrows and reruns. */
+ *   range, and the caller regrows and reruns.
+ * Up to 2^21 rows part of the work is one cooperative launch whose blocks meet
+ * at grid barriers; should a barrier's bounded wait (about a second) run out,
+ * the call reports GS_ERR_TIMEOUT (in *status_dev, and as its return value with
+ * num_pairs_host), with no pairs. */
 int gs_bin_sort(const gs_proj* proj, int N, const gs_camera* cams_host, int V, int tile_size,
                 void* workspace, size_t workspace_bytes, long long pair_capacity,
                 unsigned* sorted_vals, unsigned long long* sorted_keys, unsigned* tile_ranges,

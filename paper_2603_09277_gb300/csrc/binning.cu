@@ -1171,14 +1171,14 @@ cudaError_t allow_coop_smem() {
                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CoopShared));
 }
 
-// Most CTAs of depth_sort_kernel for a cooperative launch on the current device
-// (0: not available there, e.g. on part of a GPU); cached per device.
-int coop_grid() {
+// Whether the current device can hold depth_sort_kernel's largest grid at once
+// (not a part of a GPU with fewer SMs); cached per device.
+bool coop_available() {
   static std::atomic<int> cache[64];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
   const int c = cache[dev].load(std::memory_order_relaxed);
-  if (c) return c > 0 ? c : 0;
+  if (c) return c > 0;
   int per_sm = 0, sms = 0, coop = 0;
   int v = -1;
   if (allow_coop_smem<false>() == cudaSuccess &&
@@ -1188,10 +1188,10 @@ int coop_grid() {
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
       cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
       per_sm > 0 && sms >= kCoopGrid)
-    v = kCoopGrid;
+    v = 1;
   cudaGetLastError();
   cache[dev].store(v, std::memory_order_relaxed);
-  return v > 0 ? v : 0;
+  return v > 0;
 }
 
 // ----------------------------------------------------------------------------
@@ -2065,6 +2065,42 @@ void radix_sort(unsigned* k[2], unsigned* v[2], const long long* n_dev, long lon
   }
 }
 
+// Steps 1 to 3 in one launch (depth_sort_kernel).  An error of the launch itself
+// that says the grid cannot be resident at once (a part of the GPU, say) is
+// reported as cudaErrorCooperativeLaunchTooLarge: the caller then takes the
+// separate kernels.
+cudaError_t launch_depth_sort(const CoopArgs& args_in, const CamTable& ct, cudaStream_t st) {
+  CoopArgs a = args_in;
+  CamTable cams = ct;
+  void* args[] = {&a, &cams};
+  // a CTA per 1,024 rows, at most one per SM: fewer CTAs meet at a barrier sooner
+  int ctas = (int)std::min<long long>(kCoopGrid, (a.rows.n + 1023) / 1024);
+  cudaError_t e;
+  if (a.rows.n <= kClusterRows) {
+    int c = 1;  // (cluster sizes are powers of two)
+    while (c < kCoopCluster && c < ctas) c *= 2;
+    if ((e = allow_coop_smem<true>()) != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(kCoopThreads);
+    cfg.dynamicSmemBytes = sizeof(CoopShared);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = c;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(depth_sort_kernel<true>), args);
+  } else {
+    if ((e = allow_coop_smem<false>()) != cudaSuccess) return e;
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(depth_sort_kernel<false>),
+                                    dim3(ctas), dim3(kCoopThreads), args, sizeof(CoopShared), st);
+  }
+  if (e == cudaErrorLaunchOutOfResources) e = cudaErrorCooperativeLaunchTooLarge;
+  return e;
+}
+
 int bits_for(long long count) {
   int b = 0;
   while (b < 32 && (1ll << b) < count) ++b;
@@ -2101,18 +2137,13 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
                      status_dev};
   // the visible rows' depth-bit range (complement of the smallest, largest)
   unsigned* range = reinterpret_cast<unsigned*>(w.counters + 12);
-  const int coop = n_rows <= kCoopRows ? coop_grid() : 0;
-  const SortedRows rows_sorted{w.rv[0], w.rv[1], coop ? nullptr : range};
   // scan blocks of 1,024 rows (4 per thread) keep many CTAs in flight when
   // few rows are visible; on large row counts 4,096-row blocks (16 per
   // thread) are faster
   // the projection's 8-bit packed rects (views of at most 255 tiles per side)
   const unsigned* rect8 = rect8_fits(ct) ? proj->rect8 : nullptr;
-  const bool small = n_rows <= (4ll << 20);
-  const int items = coop ? 1 : small ? 4 : 16;
-  const long long nb = (n_rows + kScanThreads * items - 1) / (kScanThreads * items);
-  if (n_rows > 0 && coop) {
-    // 1-3. in one launch
+  bool coop = n_rows > 0 && n_rows <= kCoopRows && coop_available();
+  if (coop) {
     CoopArgs a;
     a.rows = RadixRows{proj->depth, proj->tiles_touched, n_rows, n_vis};
     for (int i = 0; i < 2; ++i) {
@@ -2129,35 +2160,20 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     a.rect_sorted = w.rect_sorted;
     a.arrive = arrive + 1;
     a.co = co;
-    CamTable cams = ct;
-    void* args[] = {&a, &cams};
-    // a CTA per 1,024 rows, at most one per SM: fewer CTAs meet at a barrier sooner
-    int ctas = (int)std::min<long long>(coop, (n_rows + 1023) / 1024);
-    if (n_rows <= kClusterRows) {
-      int c = 1;  // (cluster sizes are powers of two)
-      while (c < kCoopCluster && c < ctas) c *= 2;
-      ctas = c;
-      GS_TRY_CUDA(allow_coop_smem<true>());
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(ctas);
-      cfg.blockDim = dim3(kCoopThreads);
-      cfg.dynamicSmemBytes = sizeof(CoopShared);
-      cfg.stream = st;
-      cudaLaunchAttribute at[1];
-      at[0].id = cudaLaunchAttributeClusterDimension;
-      at[0].val.clusterDim.x = ctas;
-      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-      cfg.attrs = at;
-      cfg.numAttrs = 1;
-      GS_TRY_CUDA(cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(depth_sort_kernel<true>),
-                                      args));
+    const cudaError_t e = launch_depth_sort(a, ct, st);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+      cudaGetLastError();
+      coop = false;
     } else {
-      GS_TRY_CUDA(allow_coop_smem<false>());
-      GS_TRY_CUDA(cudaLaunchCooperativeKernel(
-          reinterpret_cast<const void*>(depth_sort_kernel<false>), dim3(ctas), dim3(kCoopThreads),
-          args, sizeof(CoopShared), st));
+      GS_TRY_CUDA(e);
     }
-    count_launches(1);
+  }
+  const SortedRows rows_sorted{w.rv[0], w.rv[1], coop ? nullptr : range};
+  const bool small = n_rows <= (4ll << 20);
+  const int items = coop ? 1 : small ? 4 : 16;
+  const long long nb = (n_rows + kScanThreads * items - 1) / (kScanThreads * items);
+  if (n_rows > 0 && coop) {
+    count_launches(1);  // 1-3. in one launch (above)
   } else if (n_rows > 0) {
     // 1-2. stable depth sort of the visible rows (ties keep row order = id
     //    order) on the significant bits of their depth range; the first pass

