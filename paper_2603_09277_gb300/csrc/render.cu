@@ -57,14 +57,16 @@ namespace {
 // position is one byte in the per-warp entry lists).
 constexpr int kMaxBatch = 256;
 // Up to this many contributing lanes add directly; above, a warp reduction.  At
-// two pixels per thread 16 to 24 are the fastest (977 us on 8 views of 3M
-// Gaussians, 996 at 12, 1010 at 8), but every add into a large Gaussian's row
-// rounds: at 24 the colour and opacity gradients of a 1M-Gaussian view are up
-// to twice as far from their 64-bit values as at 12.  One pixel per thread runs
-// on few tiles, where the adds are few.
+// two pixels per thread 16 to 20 are the fastest (8 views of 3M Gaussians 985 and
+// 979 us, 996 at 12; 2,170 tiles of large opaque splats 94.7 and 96.6, 96.7 at
+// 12), but every add into a large Gaussian's row rounds: the colour gradients of
+// those splats are 5.7e-7 from their 64-bit values at 12, 6.9e-7 at 16 and 7.2e-7
+// at 20, and at 24 those of a 1M-Gaussian view can be twice as far as at 12.  (A
+// 16x4-pixel strip per warp at 24: 8.4e-7.)  One pixel per thread runs on few
+// tiles, where the adds are few.
 template <int PPT>
 struct DirectLanes {
-  static constexpr int value = PPT == 1 ? 24 : 12;
+  static constexpr int value = PPT == 1 ? 24 : 16;
 };
 constexpr unsigned kFull = 0xffffffffu;
 // A row coordinate this far from every mean makes the exponent -inf (f22 > 0),
