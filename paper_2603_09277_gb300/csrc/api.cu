@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(
     const float* __restrict__ entropy, const LossViews lv, long long P, float gamma,
     float l1_weight, float* __restrict__ dimg, float* __restrict__ dent,
     double* __restrict__ partials, int vec) {
+  behind_previous();
   float acc = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -283,6 +284,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(
 // ..., then a fixed shuffle tree and a fixed sum over the 8 warps.
 __global__ void __launch_bounds__(kLossThreads) loss_finalize_kernel(
     const double* __restrict__ partials, int n, double* __restrict__ out) {
+  behind_previous();
   double t = 0.0;
   for (int i = threadIdx.x; i < n; i += kLossThreads) t += partials[i];
 #pragma unroll
@@ -299,6 +301,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_finalize_kernel(
 
 // log s += ln(zeta), 16-byte accesses for the aligned body.
 __global__ void scale_reset_kernel(float* __restrict__ ls, long long n, float delta) {
+  behind_previous();
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   long long head = (long long)((16 - (reinterpret_cast<uintptr_t>(ls) & 15)) & 15) / 4;
@@ -501,9 +504,9 @@ int loss_impl(const float* image, const float* target, const float* entropy, con
   const int vec = aligned(image, 16) && aligned(target, 16) && aligned(dL_dimage, 16) &&
                   (gamma == 0.f || !entropy || aligned(entropy, 16)) &&
                   (!dL_dentropy || aligned(dL_dentropy, 16));
-  loss_kernel<<<nb, kLossThreads, 0, st>>>(image, target, gamma != 0.f ? entropy : nullptr, lv, P,
-                                           gamma, (float)(1.0 - (double)lambda), dL_dimage, dL_dentropy,
-                                           partials, vec);
+  launch_behind(loss_kernel, dim3(nb), kLossThreads, st, image, target,
+                gamma != 0.f ? entropy : nullptr, lv, P, gamma, (float)(1.0 - (double)lambda),
+                dL_dimage, dL_dentropy, partials, vec);
   count_launches(1);
   if (lambda > 0.f) {
     uintptr_t m = reinterpret_cast<uintptr_t>(partials + nb + ns);
@@ -511,7 +514,7 @@ int loss_impl(const float* image, const float* target, const float* entropy, con
     const int e = launch_ssim(image, target, ct, lambda, maps, partials + nb, dL_dimage, st);
     if (e != GS_OK) return e;
   }
-  loss_finalize_kernel<<<1, kLossThreads, 0, st>>>(partials, nb + ns, loss_dev);
+  launch_behind(loss_finalize_kernel, dim3(1), kLossThreads, st, partials, nb + ns, loss_dev);
   count_launches(1);
   return check_launch();
 }
@@ -595,7 +598,7 @@ int gs_scale_reset(float* log_scales, long long n, float zeta, gs_stream stream)
   if (n == 0) return GS_OK;
   const float delta = (float)log((double)zeta);
   unsigned grid = (unsigned)std::min<long long>((n / 4 + 255) / 256 + 1, 152ll * 8);
-  scale_reset_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(log_scales, n, delta);
+  launch_behind(scale_reset_kernel, dim3(grid), 256, (cudaStream_t)stream, log_scales, n, delta);
   count_launches(1);
   return check_launch();
 }

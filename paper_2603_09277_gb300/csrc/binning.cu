@@ -193,6 +193,7 @@ __device__ __forceinline__ void scan_counts_check_dev(const CountsOut& o, int nb
 
 __global__ void __launch_bounds__(kScanThreads) scan_counts_check_kernel(const CountsOut o,
                                                                          int nblocks) {
+  behind_previous();
   scan_counts_check_dev(o, nblocks);
 }
 
@@ -286,6 +287,7 @@ __global__ void __launch_bounds__(kScanThreads) rows_gather_kernel(
     const int* __restrict__ rect, const unsigned* __restrict__ rect8, int N, const CamTable ct,
     uint2* __restrict__ rect_sorted, unsigned long long* __restrict__ arrive,
     const CountsOut co) {
+  behind_previous();
   unsigned long long* sums_q = co.sums_q;
   unsigned long long* sums_p = co.sums_p;
   const unsigned* __restrict__ rows = sorted.get();
@@ -486,6 +488,7 @@ __device__ __forceinline__ void radix_load(const RadixPass& a, long long j, long
 }
 
 __global__ void __launch_bounds__(kRadixThreads) radix_upsweep_kernel(const RadixPass a) {
+  behind_previous();
   // the first pass over rows folds the key range in, so it cannot read the
   // plan: its digit is the low byte of the key
   const bool rows = a.from_rows();
@@ -567,6 +570,7 @@ __global__ void __launch_bounds__(kRadixThreads) radix_upsweep_kernel(const Radi
 // place (Ga = the pass's active CTAs) and writes the digit total to
 // totals[d].  G <= 1024.
 __global__ void __launch_bounds__(kScanThreads) radix_scan_kernel(const RadixPass a, int G) {
+  behind_previous();
   const RadixPlan pl = radix_plan(a.range, a.bits);
   if (a.pass >= pl.passes) return;
   unsigned* totals = a.digit_tot;
@@ -603,6 +607,7 @@ __global__ void __launch_bounds__(kScanThreads) radix_scan_kernel(const RadixPas
 #endif
 __global__ void __launch_bounds__(kRadixThreads, GS_RADIX_CTAS) radix_downsweep_kernel(
     const RadixPass a) {
+  behind_previous();
   const RadixPlan pl = radix_plan(a.range, a.bits);
   if (a.pass >= pl.passes) return;
   unsigned* __restrict__ keys_out = a.keys_out;
@@ -1232,6 +1237,7 @@ __global__ void __launch_bounds__(kScanThreads) rows_expand_kernel(
     const long long* __restrict__ q_eff, int N, unsigned n_magic, const CamTable ct,
     unsigned* __restrict__ skeys, unsigned* __restrict__ svals, int vec16, int packed,
     unsigned* __restrict__ hist, int hgrid, unsigned hmask) {
+  behind_previous();
   constexpr int RB = kScanThreads * ITEMS;
   __shared__ unsigned s_off[RB + 1];  // item offset of each row in the block (+ the total)
   // the super-tile sort's first-pass histogram (hist: [256][hgrid], zeroed):
@@ -1363,6 +1369,7 @@ __global__ void __launch_bounds__(256) ranges_kernel(const unsigned* __restrict_
                                                      const long long* __restrict__ p_eff,
                                                      unsigned kmask,
                                                      unsigned* __restrict__ ranges) {
+  behind_previous();
   const long long P = *p_eff;
   const long long groups = (P + 3) / 4;
   for (long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x; g < groups;
@@ -1433,6 +1440,7 @@ __global__ void __launch_bounds__(1024) st_segments_kernel(
     const uint2* __restrict__ st_ranges, int S, unsigned* __restrict__ seg_first,
     Segment* __restrict__ segs, unsigned* __restrict__ seg_st, const CamTable ct,
     long long* __restrict__ n_seg) {
+  behind_previous();
   __shared__ unsigned s_w[32];
   __shared__ unsigned s_carry;
   __shared__ Segment s_seg[1024];    // the super-tile's whole range, tile and shape
@@ -1556,6 +1564,7 @@ __global__ void __launch_bounds__(256) st_count_kernel(
     const CamTable ct, unsigned* __restrict__ desc, unsigned* __restrict__ hist,
     const unsigned* __restrict__ totals, const long long* __restrict__ q_eff, int S,
     unsigned* __restrict__ seg_first) {
+  behind_previous();
   __shared__ unsigned s_cnt[8][64];
   constexpr int kPer = kSeg / 8;  // items of a warp
   __shared__ __align__(16) unsigned short s_desc[8][kPer];
@@ -1681,6 +1690,7 @@ __global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* __restric
                                                        unsigned long long* __restrict__ arrive,
                                                        unsigned* __restrict__ tile_start,
                                                        unsigned* __restrict__ ranges) {
+  behind_previous();
   __shared__ uint4 s_part[64][16];
   const int s = blockIdx.x;
   const int k = threadIdx.x >> 4, q = threadIdx.x & 15;
@@ -1836,6 +1846,7 @@ __global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
     const long long* __restrict__ n_seg, const unsigned* __restrict__ hist,
     const unsigned* __restrict__ tile_start, const float* __restrict__ depth,
     unsigned* __restrict__ out_vals, unsigned long long* __restrict__ out_keys, long long cap) {
+  behind_previous();
   constexpr unsigned kRing = 128;  // at most 63 waiting + 32 new items
   __shared__ uint2 s_item[kSeg];                     // row, descriptor
   __shared__ __align__(16) uint2 s_ring[8][kRing];   // row, columns covered
@@ -1924,6 +1935,7 @@ __global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
 
 
 __global__ void set_value_kernel(long long* __restrict__ dst, long long v) {
+  behind_previous();
   if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
 
@@ -2058,9 +2070,10 @@ void radix_sort(unsigned* k[2], unsigned* v[2], const long long* n_dev, long lon
     a.pass = p;
     // (hist0_ready: the first pass's per-CTA digit counts are already in
     // hist, summed by the kernel that wrote the items)
-    if (p > 0 || !hist0_ready) radix_upsweep_kernel<<<grid, kRadixThreads, 0, st>>>(a);
-    radix_scan_kernel<<<kRadixBins, kScanThreads, 0, st>>>(a, grid);
-    radix_downsweep_kernel<<<grid, kRadixThreads, 0, st>>>(a);
+    if (p > 0 || !hist0_ready)
+      launch_behind(radix_upsweep_kernel, dim3(grid), kRadixThreads, st, a);
+    launch_behind(radix_scan_kernel, dim3(kRadixBins), kScanThreads, st, a, grid);
+    launch_behind(radix_downsweep_kernel, dim3(grid), kRadixThreads, st, a);
     count_launches(p > 0 || !hist0_ready ? 3 : 2);
   }
 }
@@ -2186,14 +2199,14 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     //    (its last CTA: the scans of Q and P over the blocks, the capacity
     //    check and the reported count)
     if (small)
-      rows_gather_kernel<4><<<(unsigned)nb, kScanThreads, 0, st>>>(
-          rows_sorted, n_vis, proj->rect, rect8, N, ct, w.rect_sorted, arrive + 1, co);
+      launch_behind(rows_gather_kernel<4>, dim3((unsigned)nb), kScanThreads, st, rows_sorted,
+                    n_vis, proj->rect, rect8, N, ct, w.rect_sorted, arrive + 1, co);
     else
-      rows_gather_kernel<16><<<(unsigned)nb, kScanThreads, 0, st>>>(
-          rows_sorted, n_vis, proj->rect, rect8, N, ct, w.rect_sorted, arrive + 1, co);
+      launch_behind(rows_gather_kernel<16>, dim3((unsigned)nb), kScanThreads, st, rows_sorted,
+                    n_vis, proj->rect, rect8, N, ct, w.rect_sorted, arrive + 1, co);
     count_launches(1);
   } else {
-    scan_counts_check_kernel<<<1, kScanThreads, 0, st>>>(co, 0);
+    launch_behind(scan_counts_check_kernel, dim3(1), kScanThreads, st, co, 0);
     count_launches(1);
   }
   GS_TRY_CUDA(cudaGetLastError());
@@ -2250,17 +2263,17 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     unsigned* h = hist0 ? w.hist : nullptr;
     const unsigned hmask = (1u << radix_plan_bits(0u, sbits).d0) - 1u;
     if (coop)
-      rows_expand_kernel<1><<<(unsigned)nb, kScanThreads, 0, st>>>(
-          rows_sorted, w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N),
-          ct, sk[0], sv[0], vec16, packed, h, sgrid, hmask);
+      launch_behind(rows_expand_kernel<1>, dim3((unsigned)nb), kScanThreads, st, rows_sorted,
+                    w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N), ct,
+                    sk[0], sv[0], vec16, packed, h, sgrid, hmask);
     else if (small)
-      rows_expand_kernel<4><<<(unsigned)nb, kScanThreads, 0, st>>>(
-          rows_sorted, w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N),
-          ct, sk[0], sv[0], vec16, packed, h, sgrid, hmask);
+      launch_behind(rows_expand_kernel<4>, dim3((unsigned)nb), kScanThreads, st, rows_sorted,
+                    w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N), ct,
+                    sk[0], sv[0], vec16, packed, h, sgrid, hmask);
     else
-      rows_expand_kernel<16><<<(unsigned)nb, kScanThreads, 0, st>>>(
-          rows_sorted, w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N),
-          ct, sk[0], sv[0], vec16, packed, h, sgrid, hmask);
+      launch_behind(rows_expand_kernel<16>, dim3((unsigned)nb), kScanThreads, st, rows_sorted,
+                    w.rect_sorted, n_vis, w.block_sums, q_eff, N, div_magic_host((unsigned)N), ct,
+                    sk[0], sv[0], vec16, packed, h, sgrid, hmask);
     count_launches(1);
   }
   // 5. stable sort of the super-pairs by super-tile id
@@ -2277,23 +2290,22 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
   } else if (spasses > 1) {
     GS_TRY_CUDA(cudaMemsetAsync(w.st_ranges, 0, 2 * sizeof(unsigned) * (size_t)S, st));
     const unsigned gq = (unsigned)std::min<long long>((q_bound + 1023) / 1024, 152ll * 16);
-    ranges_kernel<<<gq, 256, 0, st>>>(sp_keys, q_eff, packed ? 0xffffu : 0xffffffffu,
-                                      w.st_ranges);
+    launch_behind(ranges_kernel, dim3(gq), 256, st, sp_keys, q_eff, packed ? 0xffffu : 0xffffffffu,
+                  w.st_ranges);
     count_launches(1);
   }
   if (spasses > 1) {  // (else st_count_kernel forms the segments)
-    st_segments_kernel<<<1, 1024, 0, st>>>(reinterpret_cast<const uint2*>(w.st_ranges), S,
-                                           w.seg_first, w.segs, packed ? nullptr : w.seg_st, ct,
-                                           n_seg);
+    launch_behind(st_segments_kernel, dim3(1), 1024, st,
+                  reinterpret_cast<const uint2*>(w.st_ranges), S, w.seg_first, w.segs,
+                  packed ? nullptr : w.seg_st, ct, n_seg);
     count_launches(1);
   }
   const unsigned gs = (unsigned)std::min<long long>(max_segments(q_bound, S), 152ll * 8);
-  st_count_kernel<<<gs, 256, 0, st>>>(sp_keys, sp_rows, w.segs, w.seg_st, n_seg, packed,
-                                      proj->rect, N, ct, desc, w.seg_hist, st_totals, q_eff, S,
-                                      w.seg_first);
-  st_scan_kernel<<<(unsigned)S, 1024, 0, st>>>(w.seg_first, ct,
-                                               reinterpret_cast<uint4*>(w.seg_hist), w.tile_cnt,
-                                               arrive + 2, w.tile_start, ranges);
+  launch_behind(st_count_kernel, dim3(gs), 256, st, sp_keys, sp_rows, w.segs, w.seg_st, n_seg,
+                packed, proj->rect, N, ct, desc, w.seg_hist, st_totals, q_eff, S, w.seg_first);
+  launch_behind(st_scan_kernel, dim3((unsigned)S), 1024, st, w.seg_first, ct,
+                reinterpret_cast<uint4*>(w.seg_hist), w.tile_cnt, arrive + 2, w.tile_start,
+                ranges);
   // 7. every row into the lists of the tiles it covers, in depth order
   {
     const int e = stage_event(GS_STAGE_EXPANSION, false, st);
@@ -2301,13 +2313,11 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
   }
   const unsigned ge = (unsigned)std::min<long long>(max_segments(q_bound, S), kEmitGrid);
   if (sorted_keys)
-    st_emit_kernel<true><<<ge, 256, 0, st>>>(sp_keys, sp_rows, desc, packed, w.segs, n_seg,
-                                             w.seg_hist, w.tile_start, proj->depth, sorted_vals,
-                                             sorted_keys, cap);
+    launch_behind(st_emit_kernel<true>, dim3(ge), 256, st, sp_keys, sp_rows, desc, packed, w.segs,
+                  n_seg, w.seg_hist, w.tile_start, proj->depth, sorted_vals, sorted_keys, cap);
   else
-    st_emit_kernel<false><<<ge, 256, 0, st>>>(sp_keys, sp_rows, desc, packed, w.segs, n_seg,
-                                              w.seg_hist, w.tile_start, proj->depth, sorted_vals,
-                                              nullptr, cap);
+    launch_behind(st_emit_kernel<false>, dim3(ge), 256, st, sp_keys, sp_rows, desc, packed, w.segs,
+                  n_seg, w.seg_hist, w.tile_start, proj->depth, sorted_vals, nullptr, cap);
   {
     const int e = stage_event(GS_STAGE_EXPANSION, true, st);
     if (e != GS_OK) return e;
@@ -2322,6 +2332,7 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
 namespace {
 __global__ void queue_keys_kernel(const unsigned* __restrict__ ranges, long long T,
                                   unsigned* __restrict__ keys, unsigned* __restrict__ vals) {
+  behind_previous();
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < T;
        t += (long long)gridDim.x * blockDim.x) {
     unsigned len = ranges[2 * t + 1] - ranges[2 * t];
@@ -2350,11 +2361,11 @@ int launch_tile_queue(const unsigned* ranges, long long T, unsigned* order, void
   long long* n_dev = reinterpret_cast<long long*>(p);
   p += align256(sizeof(long long) * 2);
   unsigned* hist = reinterpret_cast<unsigned*>(p);
-  set_value_kernel<<<1, 32, 0, st>>>(n_dev, T);
+  launch_behind(set_value_kernel, dim3(1), 32, st, n_dev, T);
   count_launches(1);
   unsigned grid = (unsigned)std::min<long long>((T + 255) / 256, 1024);
   // 4 passes (even): the result ends in the first buffer, i.e. `order`
-  queue_keys_kernel<<<grid, 256, 0, st>>>(ranges, T, k0, order);
+  launch_behind(queue_keys_kernel, dim3(grid), 256, st, ranges, T, k0, order);
   count_launches(1);
   unsigned* k[2] = {k0, k1};
   unsigned* v[2] = {order, v1};

@@ -256,6 +256,16 @@ __device__ __forceinline__ int find_view_of_pixel(const CamTable& ct, long long 
 
 }  // namespace gs
 
+// First statement of a kernel launched with launch_behind: lets the stream's next
+// kernel place its blocks once all of this one's run (those blocks wait here until
+// this kernel has ended), and waits until the previous kernel has ended and its
+// writes are visible.  No memory is touched before it.
+namespace gs {
+__device__ __forceinline__ void behind_previous() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+}  // namespace gs
+
 // ---------------------------------------------------------------------------
 // Host-side helpers shared by the translation units (defined in api.cu).
 // ---------------------------------------------------------------------------
@@ -264,6 +274,31 @@ int set_cuda_error(cudaError_t e);
 int set_error_text_and_status(const char* msg, int status);
 void count_launches(int n);
 int check_launch();
+
+// Launch of a kernel whose first statement is behind_previous(): issued to a
+// stream, its blocks are placed while the stream's previous kernel still runs its
+// last ones (programmatic dependent launch), which hides the launch and the
+// previous kernel's drain: three views' lists 234 -> 220 us (10 launches), a
+// blending with its adjoint 158 -> 146 (5), D-SSIM on two views 214 -> 205 (4), a
+// 1920x1080 render 383 -> 376.  Into a graph the launch is a plain one: a
+// replay starts plain kernel nodes as fast, and with programmatic edges a captured
+// step of 10k Gaussians took 194 instead of 176 us, of 1M 615 instead of 608.
+// (An error is picked up by check_launch.)
+template <class... P, class... A>
+void launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, A... args) {
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+  cudaStreamIsCapturing(st, &capture);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 // tile: the tile side (0 means 16); fov_clamp comes from prm (1.3 if NULL).
 bool build_cam_table(const gs_camera* cams, int V, const gs_params* prm, int tile, CamTable* ct);
 RenderConsts render_consts(const gs_params* prm);

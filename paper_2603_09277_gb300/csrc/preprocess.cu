@@ -483,6 +483,7 @@ __global__ void __launch_bounds__(256, pre_ctas_per_sm<DEG>()) preprocess_kernel
     const float* __restrict__ quats, const float* __restrict__ opacity_logits,
     const float* __restrict__ sh, int N, const CamTable ct, float dilation, float near_z,
     const ShPtr shp, gs_proj out) {
+  behind_previous();
   int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= N) return;
   Activated a = activate(means, log_scales, quats, opacity_logits, g);
@@ -953,6 +954,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
     const float* __restrict__ sh, int N, const CamTable ct, float dilation, const ShPtr shp,
     int chunk, float* __restrict__ grad2d, float* __restrict__ g_means, float* __restrict__ g_ls,
     float* __restrict__ g_quats, float* __restrict__ g_opac, float* __restrict__ g_sh) {
+  behind_previous();
   __shared__ unsigned s_any[kAdjChunk / 32];
   __shared__ unsigned short s_idx[kAdjChunk];
   __shared__ unsigned s_n;
@@ -1000,13 +1002,13 @@ void launch_adjoint(const float* means, const float* log_scales, const float* qu
   const int chunk = (int)std::min<long long>(kAdjChunk, (per + kAdjThreads - 1) / kAdjThreads * kAdjThreads);
   const unsigned grid = (unsigned)(((long long)N + chunk - 1) / chunk);
   if (prm->attr_dtype == GS_ATTR_F32)
-    preprocess_bwd_kernel<DEG, true><<<grid, kAdjThreads, 0, st>>>(
-        means, log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
-        chunk, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
+    launch_behind(preprocess_bwd_kernel<DEG, true>, dim3(grid), kAdjThreads, st, means, log_scales,
+                  quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N), chunk,
+                  grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
   else
-    preprocess_bwd_kernel<DEG, false><<<grid, kAdjThreads, 0, st>>>(
-        means, log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
-        chunk, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
+    launch_behind(preprocess_bwd_kernel<DEG, false>, dim3(grid), kAdjThreads, st, means,
+                  log_scales, quats, opacity_logits, sh, N, ct, prm->dilation, sh_ptr(sh, prm, N),
+                  chunk, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
 }
 
 // The 2D gradients of Suppl. C per row from the moment rows of the blending
@@ -1018,6 +1020,7 @@ __global__ void __launch_bounds__(256) grad2d_attr_kernel(const void* __restrict
                                                           const unsigned* __restrict__ tiles_touched,
                                                           const float* __restrict__ grad2d,
                                                           long long rows, float* __restrict__ out) {
+  behind_previous();
   for (long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x; row < rows;
        row += (long long)gridDim.x * blockDim.x) {
     float o[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -1055,16 +1058,16 @@ int launch_grad2d_attributes(const gs_proj* proj, long long rows, const gs_param
   const unsigned grid = (unsigned)std::min<long long>((rows + 255) / 256, 152ll * 8);
   switch (prm->attr_dtype) {
     case GS_ATTR_F32:
-      grad2d_attr_kernel<GS_ATTR_F32><<<grid, 256, 0, st>>>(proj->records, proj->tiles_touched,
-                                                            grad2d, rows, out);
+      launch_behind(grad2d_attr_kernel<GS_ATTR_F32>, dim3(grid), 256, st, proj->records,
+                    proj->tiles_touched, grad2d, rows, out);
       break;
     case GS_ATTR_F16:
-      grad2d_attr_kernel<GS_ATTR_F16><<<grid, 256, 0, st>>>(proj->records, proj->tiles_touched,
-                                                            grad2d, rows, out);
+      launch_behind(grad2d_attr_kernel<GS_ATTR_F16>, dim3(grid), 256, st, proj->records,
+                    proj->tiles_touched, grad2d, rows, out);
       break;
     case GS_ATTR_BF16:
-      grad2d_attr_kernel<GS_ATTR_BF16><<<grid, 256, 0, st>>>(proj->records, proj->tiles_touched,
-                                                             grad2d, rows, out);
+      launch_behind(grad2d_attr_kernel<GS_ATTR_BF16>, dim3(grid), 256, st, proj->records,
+                    proj->tiles_touched, grad2d, rows, out);
       break;
     default:
       return GS_ERR_INVALID_ARG;
@@ -1078,10 +1081,9 @@ void launch_preprocess_dt(int deg, dim3 grid, dim3 block, const float* means,
                           const float* log_scales, const float* quats,
                           const float* opacity_logits, const float* sh, int N, const CamTable& ct,
                           const gs_params* prm, const gs_proj& o, cudaStream_t st) {
-#define GS_PRE_LAUNCH(D)                                                                   \
-  preprocess_kernel<DT, D><<<grid, block, 0, st>>>(means, log_scales, quats, opacity_logits, \
-                                                   sh, N, ct, prm->dilation, prm->near_z,    \
-                                                   sh_ptr(sh, prm, N), o)
+#define GS_PRE_LAUNCH(D)                                                              \
+  launch_behind(preprocess_kernel<DT, D>, grid, block, st, means, log_scales, quats,  \
+                opacity_logits, sh, N, ct, prm->dilation, prm->near_z, sh_ptr(sh, prm, N), o)
   switch (deg) {
     case 0: GS_PRE_LAUNCH(0); break;
     case 1: GS_PRE_LAUNCH(1); break;

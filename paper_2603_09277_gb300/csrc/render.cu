@@ -422,6 +422,7 @@ __global__ void __launch_bounds__(TS * TS / PPT) render_fwd_kernel(const CamTabl
                                                                     const RenderConsts rc,
                                                                     const FwdArgs a,
                                                                     int persistent) {
+  behind_previous();
   unsigned long long nb = 0, ne = 0;
   if (a.zero) zero_stripe(a.zero, a.zero_n16);
   if (persistent) {
@@ -820,6 +821,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, (TS == 16 && PPT != 4) ? 4 * PP
                                                                     const RenderConsts rc,
                                                                     const BwdArgs a,
                                                                     int persistent) {
+  behind_previous();
   if (persistent) {
     __shared__ unsigned s_t;
     for (;;) {
@@ -849,16 +851,19 @@ void launch_fwd_b(const CamTable& ct, const RenderConsts& rc, const FwdArgs& a, 
   const int grid = ctas > 0 ? ctas : ct.total_tiles;
   const int pers = ctas > 0 ? 1 : 0;
   if (a.stats)
-    render_fwd_kernel<DT, TS, PPT, B, true><<<grid, TS * TS / PPT, 0, st>>>(ct, rc, a, pers);
+    launch_behind(render_fwd_kernel<DT, TS, PPT, B, true>, dim3(grid), TS * TS / PPT, st, ct, rc,
+                  a, pers);
   else
-    render_fwd_kernel<DT, TS, PPT, B, false><<<grid, TS * TS / PPT, 0, st>>>(ct, rc, a, pers);
+    launch_behind(render_fwd_kernel<DT, TS, PPT, B, false>, dim3(grid), TS * TS / PPT, st, ct, rc,
+                  a, pers);
 }
 
 template <int DT, int TS, int PPT, int B>
 void launch_bwd_b(const CamTable& ct, const RenderConsts& rc, const BwdArgs& a, int ctas,
                   cudaStream_t st) {
   const int grid = ctas > 0 ? ctas : ct.total_tiles;
-  render_bwd_kernel<DT, TS, PPT, B><<<grid, TS * TS / PPT, 0, st>>>(ct, rc, a, ctas > 0 ? 1 : 0);
+  launch_behind(render_bwd_kernel<DT, TS, PPT, B>, dim3(grid), TS * TS / PPT, st, ct, rc, a,
+                ctas > 0 ? 1 : 0);
 }
 
 // The 128-record batch exists for F32 records on 16-pixel tiles only (the

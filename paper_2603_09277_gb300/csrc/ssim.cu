@@ -121,6 +121,7 @@ __device__ __forceinline__ ChannelRange channels_of(unsigned parts, unsigned par
 __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     float* __restrict__ maps /* 15 planes of P */, long long P, double* __restrict__ partials) {
+  behind_previous();
   __shared__ __align__(16) float2 s_xy[kSsimS][kSsimP];
   __shared__ __align__(16) float2 s_m[2 * kQS][kSsimB];  // horizontal sums of (x, y)
   __shared__ __align__(16) float2 s_q[2 * kQS][kSsimB];  // of (x^2, y^2)
@@ -245,6 +246,7 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
 __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
     const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
     const float* __restrict__ maps, long long P, float* __restrict__ dimg) {
+  behind_previous();
   __shared__ __align__(16) float2 s_ab[kSsimS][kSsimP];  // (a - 2 (mu_x - c) b - (mu_y - c') e, b)
   __shared__ __align__(16) float s_e[kSsimS][kSsimP];
   __shared__ __align__(16) float2 s_hab[kSsimS][kSsimB];  // horizontal sums
@@ -389,8 +391,9 @@ int launch_ssim(const float* image, const float* target, const CamTable& ct, flo
   if (nb == 0) return GS_OK;
   const long long P = ct.c[ct.V - 1].pix_off + (long long)ct.c[ct.V - 1].W * ct.c[ct.V - 1].H;
   const dim3 grid(nb, ssim_parts(nb));
-  ssim_fwd_kernel<<<grid, kSsimThreads, 0, st>>>(image, target, sv, maps, P, partials);
-  ssim_bwd_kernel<<<grid, kSsimThreads, 0, st>>>(image, target, sv, maps, P, dimg);
+  launch_behind(ssim_fwd_kernel, dim3(grid), kSsimThreads, st, image, target, sv, maps, P,
+                partials);
+  launch_behind(ssim_bwd_kernel, dim3(grid), kSsimThreads, st, image, target, sv, maps, P, dimg);
   count_launches(2);
   return check_launch();
 }
