@@ -30,9 +30,11 @@
 // All kernels read their element counts from device memory and use grids
 // sized from host-known upper bounds (blocks beyond the actual counts leave
 // at once), so the whole sequence can be captured in a CUDA graph (no host
-// synchronisation needed).  None of them waits on another block: where a
-// single-block scan follows a kernel, the kernel's last block to finish runs
-// it (each block counts its arrival after a __threadfence).
+// synchronisation needed).  Up to 2M rows steps 1 to 3 are one cooperative
+// launch whose blocks meet at grid barriers with bounded waits
+// (depth_sort_kernel); no other kernel waits on another block: where a
+// single-block scan follows one, its last block to finish runs the scan (each
+// block counts its arrival after a __threadfence).
 #include <cuda.h>
 
 #include <algorithm>
