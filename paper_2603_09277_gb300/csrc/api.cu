@@ -217,10 +217,10 @@ __device__ __forceinline__ int view_of_pixel(const LossViews& lv, long long i) {
 // vec (every array 16-byte aligned) a thread takes 4 pixels at a time with
 // 16-byte loads and stores; the last P mod 4 pixels go through block 0.
 __global__ void __launch_bounds__(kLossThreads) loss_kernel(
-    const float* __restrict__ image, const float* __restrict__ target,
-    const float* __restrict__ entropy, const LossViews lv, long long P, float gamma,
-    float l1_weight, float* __restrict__ dimg, float* __restrict__ dent,
-    double* __restrict__ partials, int vec) {
+    const float* image, const float* target,
+    const float* entropy, const LossViews lv, long long P, float gamma,
+    float l1_weight, float* dimg, float* dent,
+    double* partials, int vec) {
   behind_previous();
   float acc = 0.f;
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_kernel(
 // Sums the block partials in a fixed order: thread t adds partials t, t+256,
 // ..., then a fixed shuffle tree and a fixed sum over the 8 warps.
 __global__ void __launch_bounds__(kLossThreads) loss_finalize_kernel(
-    const double* __restrict__ partials, int n, double* __restrict__ out) {
+    const double* partials, int n, double* out) {
   behind_previous();
   double t = 0.0;
   for (int i = threadIdx.x; i < n; i += kLossThreads) t += partials[i];
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kLossThreads) loss_finalize_kernel(
 }
 
 // log s += ln(zeta), 16-byte accesses for the aligned body.
-__global__ void scale_reset_kernel(float* __restrict__ ls, long long n, float delta) {
+__global__ void scale_reset_kernel(float* ls, long long n, float delta) {
   behind_previous();
   const long long stride = (long long)gridDim.x * blockDim.x;
   const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -214,7 +214,7 @@ __device__ __forceinline__ void scan_counts_check_dev(const CountsOut& o, int nb
 // ----------------------------------------------------------------------------
 static_assert(kSuperTile == 8, "super-tile masks hold 8x8 tiles");
 
-__device__ __forceinline__ int4 view_rect(const int* __restrict__ rect, unsigned row, int N,
+__device__ __forceinline__ int4 view_rect(const int* rect, unsigned row, int N,
                                           const CamTable& ct) {
   int4 r = reinterpret_cast<const int4*>(rect)[row];
   const CamInfo& c = ct.c[row / (unsigned)N];
@@ -285,14 +285,14 @@ struct SortedRows {
 // capacity check (scan_counts_check_dev).
 template <int ITEMS>
 __global__ void __launch_bounds__(kScanThreads) rows_gather_kernel(
-    const SortedRows sorted, const long long* __restrict__ n_dev,
-    const int* __restrict__ rect, const unsigned* __restrict__ rect8, int N, const CamTable ct,
-    uint2* __restrict__ rect_sorted, unsigned long long* __restrict__ arrive,
+    const SortedRows sorted, const long long* n_dev,
+    const int* rect, const unsigned* rect8, int N, const CamTable ct,
+    uint2* rect_sorted, unsigned long long* arrive,
     const CountsOut co) {
   behind_previous();
   unsigned long long* sums_q = co.sums_q;
   unsigned long long* sums_p = co.sums_p;
-  const unsigned* __restrict__ rows = sorted.get();
+  const unsigned* rows = sorted.get();
   const long long n = *n_dev;
   const long long base = (long long)blockIdx.x * (kScanThreads * ITEMS);
   if (base >= n) {  // (the whole CTA) no rows: zero sums
@@ -400,7 +400,7 @@ __host__ __device__ __forceinline__ RadixPlan radix_plan_bits(unsigned kmin, int
 // 256, which leaves the low byte of (key - kmin) equal to that of the key;
 // the later passes take the remaining significant bits of (key - kmin) in
 // digits of equal width.  There is always at least the first pass.
-__device__ __forceinline__ RadixPlan radix_plan(const unsigned* __restrict__ range, int bits) {
+__device__ __forceinline__ RadixPlan radix_plan(const unsigned* range, int bits) {
   if (!range) return radix_plan_bits(0u, bits);
   RadixPlan p;
   p.kmin = 0u;
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kRadixThreads) radix_upsweep_kernel(const Radi
   }
   const int shift = radix_shift(pl, a.pass);
   const unsigned mask = radix_mask(pl, a.pass);
-  unsigned* __restrict__ hist = a.hist;  // [256][nblocks]
+  unsigned* hist = a.hist;  // [256][nblocks]
   __shared__ unsigned s_h[kRadixWarps][kRadixBins];
   __shared__ unsigned s_kmin[kRadixWarps], s_kmax[kRadixWarps];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -612,10 +612,10 @@ __global__ void __launch_bounds__(kRadixThreads, GS_RADIX_CTAS) radix_downsweep_
   behind_previous();
   const RadixPlan pl = radix_plan(a.range, a.bits);
   if (a.pass >= pl.passes) return;
-  unsigned* __restrict__ keys_out = a.keys_out;
-  unsigned* __restrict__ vals_out = a.vals_out;
-  const unsigned* __restrict__ offsets = a.hist;
-  const unsigned* __restrict__ totals = a.digit_tot;
+  unsigned* keys_out = a.keys_out;
+  unsigned* vals_out = a.vals_out;
+  const unsigned* offsets = a.hist;
+  const unsigned* totals = a.digit_tot;
   const int shift = radix_shift(pl, a.pass);
   const unsigned mask = radix_mask(pl, a.pass);
   const bool wkeys = a.keys_last || a.pass + 1 < pl.passes;
@@ -1234,11 +1234,11 @@ __device__ __forceinline__ int div_small(int a, int d) {
 
 template <int ITEMS>
 __global__ void __launch_bounds__(kScanThreads) rows_expand_kernel(
-    const SortedRows sorted, const uint2* __restrict__ rect_sorted,
-    const long long* __restrict__ n_dev, const unsigned long long* __restrict__ block_items,
-    const long long* __restrict__ q_eff, int N, unsigned n_magic, const CamTable ct,
-    unsigned* __restrict__ skeys, unsigned* __restrict__ svals, int vec16, int packed,
-    unsigned* __restrict__ hist, int hgrid, unsigned hmask) {
+    const SortedRows sorted, const uint2* rect_sorted,
+    const long long* n_dev, const unsigned long long* block_items,
+    const long long* q_eff, int N, unsigned n_magic, const CamTable ct,
+    unsigned* skeys, unsigned* svals, int vec16, int packed,
+    unsigned* hist, int hgrid, unsigned hmask) {
   behind_previous();
   constexpr int RB = kScanThreads * ITEMS;
   __shared__ unsigned s_off[RB + 1];  // item offset of each row in the block (+ the total)
@@ -1272,7 +1272,7 @@ __global__ void __launch_bounds__(kScanThreads) rows_expand_kernel(
   __syncthreads();
   const unsigned total = (unsigned)tot;
   const long long gbase = (long long)block_items[blockIdx.x];
-  const unsigned* __restrict__ rows = sorted.get();
+  const unsigned* rows = sorted.get();
   // the sort's chunk of a position: div_magic by the chunk (Q < 2^32)
   const unsigned hchunk = hist ? (unsigned)radix_chunk(Q, hgrid) : 1u;
   const unsigned hmagic = hist ? (unsigned)(0x100000000ull / hchunk) : 0u;
@@ -1367,10 +1367,10 @@ __global__ void __launch_bounds__(kScanThreads) rows_expand_kernel(
 // Per-key [start, end) from sorted u32 keys: each thread reads 4
 // consecutive keys with one 16-byte load (the array is 256-byte aligned) plus
 // its neighbours, and marks where the key changes.
-__global__ void __launch_bounds__(256) ranges_kernel(const unsigned* __restrict__ tkeys,
-                                                     const long long* __restrict__ p_eff,
+__global__ void __launch_bounds__(256) ranges_kernel(const unsigned* tkeys,
+                                                     const long long* p_eff,
                                                      unsigned kmask,
-                                                     unsigned* __restrict__ ranges) {
+                                                     unsigned* ranges) {
   behind_previous();
   const long long P = *p_eff;
   const long long groups = (P + 3) / 4;
@@ -1428,8 +1428,8 @@ struct __align__(16) Segment {
   __device__ __forceinline__ int rows() const { return (int)(shape >> 20); }
 };
 
-__device__ __forceinline__ Segment load_segment(const Segment* __restrict__ segs, long long g) {
-  const uint4 v = __ldg(reinterpret_cast<const uint4*>(segs + g));
+__device__ __forceinline__ Segment load_segment(const Segment* segs, long long g) {
+  const uint4 v = *reinterpret_cast<const uint4*>(segs + g);
   return Segment{v.x, v.y, (int)v.z, v.w};
 }
 
@@ -1439,9 +1439,9 @@ __device__ __forceinline__ Segment load_segment(const Segment* __restrict__ segs
 // One CTA of 1024 threads; for more than 256 super-tiles (up to that many
 // st_count_kernel forms the segments itself).
 __global__ void __launch_bounds__(1024) st_segments_kernel(
-    const uint2* __restrict__ st_ranges, int S, unsigned* __restrict__ seg_first,
-    Segment* __restrict__ segs, unsigned* __restrict__ seg_st, const CamTable ct,
-    long long* __restrict__ n_seg) {
+    const uint2* st_ranges, int S, unsigned* seg_first,
+    Segment* segs, unsigned* seg_st, const CamTable ct,
+    long long* n_seg) {
   behind_previous();
   __shared__ unsigned s_w[32];
   __shared__ unsigned s_carry;
@@ -1507,7 +1507,7 @@ __global__ void __launch_bounds__(1024) st_segments_kernel(
 
 // Rect of row `row` inside the super-tile with tile origin (ox, oy), as a
 // descriptor (0 when it covers no tile of it).
-__device__ __forceinline__ unsigned st_desc(const int* __restrict__ rect, unsigned row, int N,
+__device__ __forceinline__ unsigned st_desc(const int* rect, unsigned row, int N,
                                             const CamTable& ct, int ox, int oy) {
   const int4 r = view_rect(rect, row, N, ct);
   const int x0 = r.x - ox, x1 = r.z - ox, y0 = r.y - oy, y1 = r.w - oy;
@@ -1560,12 +1560,12 @@ __device__ __forceinline__ unsigned block_scan256(unsigned x, unsigned* s_w) {
 }
 
 __global__ void __launch_bounds__(256) st_count_kernel(
-    const unsigned* __restrict__ sp_keys, const unsigned* __restrict__ sp_rows,
-    Segment* __restrict__ segs, const unsigned* __restrict__ seg_st,
-    long long* __restrict__ n_seg, int packed, const int* __restrict__ rect, int N,
-    const CamTable ct, unsigned* __restrict__ desc, unsigned* __restrict__ hist,
-    const unsigned* __restrict__ totals, const long long* __restrict__ q_eff, int S,
-    unsigned* __restrict__ seg_first) {
+    const unsigned* sp_keys, const unsigned* sp_rows,
+    Segment* segs, const unsigned* seg_st,
+    long long* n_seg, int packed, const int* rect, int N,
+    const CamTable ct, unsigned* desc, unsigned* hist,
+    const unsigned* totals, const long long* q_eff, int S,
+    unsigned* seg_first) {
   behind_previous();
   __shared__ unsigned s_cnt[8][64];
   constexpr int kPer = kSeg / 8;  // items of a warp
@@ -1677,21 +1677,21 @@ __global__ void __launch_bounds__(256) st_count_kernel(
 // One CTA per super-tile, 64 groups of segments x 16 quads of tiles: exclusive
 // scan of every tile's counts over the super-tile's segments (in place), and
 // the tile's total list length.
-__device__ __forceinline__ void tile_scan_dev(const unsigned* __restrict__ tile_cnt, int T,
-                                              unsigned* __restrict__ tile_start,
-                                              unsigned* __restrict__ ranges);
+__device__ __forceinline__ void tile_scan_dev(const unsigned* tile_cnt, int T,
+                                              unsigned* tile_start,
+                                              unsigned* ranges);
 
 __device__ __forceinline__ uint4 add4(uint4 a, uint4 b) {
   return make_uint4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
-__global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* __restrict__ seg_first,
+__global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* seg_first,
                                                        const CamTable ct,
-                                                       uint4* __restrict__ hist,
-                                                       unsigned* __restrict__ tile_cnt,
-                                                       unsigned long long* __restrict__ arrive,
-                                                       unsigned* __restrict__ tile_start,
-                                                       unsigned* __restrict__ ranges) {
+                                                       uint4* hist,
+                                                       unsigned* tile_cnt,
+                                                       unsigned long long* arrive,
+                                                       unsigned* tile_start,
+                                                       unsigned* ranges) {
   behind_previous();
   __shared__ uint4 s_part[64][16];
   const int s = blockIdx.x;
@@ -1749,9 +1749,9 @@ __global__ void __launch_bounds__(1024) st_scan_kernel(const unsigned* __restric
 // threads, 4 consecutive tiles per thread and round): list starts, and ranges
 // [start, end) ((0, 0) for an empty list).  Run by the last CTA of
 // st_scan_kernel (tile_cnt read through L2; it is padded to whole 16 bytes).
-__device__ __forceinline__ void tile_scan_dev(const unsigned* __restrict__ tile_cnt, int T,
-                                              unsigned* __restrict__ tile_start,
-                                              unsigned* __restrict__ ranges) {
+__device__ __forceinline__ void tile_scan_dev(const unsigned* tile_cnt, int T,
+                                              unsigned* tile_start,
+                                              unsigned* ranges) {
   __shared__ unsigned s_w[2][32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   unsigned carry = 0u;
@@ -1843,11 +1843,11 @@ constexpr int kEmitCtas = 4;
 constexpr long long kEmitGrid = 152ll * 64;
 template <bool KEYS>
 __global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
-    const unsigned* __restrict__ sp_keys, const unsigned* __restrict__ sp_rows,
-    const unsigned* __restrict__ desc, int packed, const Segment* __restrict__ segs,
-    const long long* __restrict__ n_seg, const unsigned* __restrict__ hist,
-    const unsigned* __restrict__ tile_start, const float* __restrict__ depth,
-    unsigned* __restrict__ out_vals, unsigned long long* __restrict__ out_keys, long long cap) {
+    const unsigned* sp_keys, const unsigned* sp_rows,
+    const unsigned* desc, int packed, const Segment* segs,
+    const long long* n_seg, const unsigned* hist,
+    const unsigned* tile_start, const float* depth,
+    unsigned* out_vals, unsigned long long* out_keys, long long cap) {
   behind_previous();
   constexpr unsigned kRing = 128;  // at most 63 waiting + 32 new items
   __shared__ uint2 s_item[kSeg];                     // row, descriptor
@@ -1855,7 +1855,7 @@ __global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const unsigned lt = (1u << lane) - 1u;
   const long long G = *n_seg;
-  const unsigned* __restrict__ keys = packed ? sp_keys : desc;
+  const unsigned* keys = packed ? sp_keys : desc;
   for (long long g = blockIdx.x; g < G; g += gridDim.x) {
     const Segment si = load_segment(segs, g);
     const int n = (int)(si.e - si.b);
@@ -1936,7 +1936,7 @@ __global__ void __launch_bounds__(256, kEmitCtas) st_emit_kernel(
 }
 
 
-__global__ void set_value_kernel(long long* __restrict__ dst, long long v) {
+__global__ void set_value_kernel(long long* dst, long long v) {
   behind_previous();
   if (threadIdx.x == 0 && blockIdx.x == 0) *dst = v;
 }
@@ -2332,8 +2332,8 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
 // Tile queue: global tile ids ordered by list length, longest first.
 // ----------------------------------------------------------------------------
 namespace {
-__global__ void queue_keys_kernel(const unsigned* __restrict__ ranges, long long T,
-                                  unsigned* __restrict__ keys, unsigned* __restrict__ vals) {
+__global__ void queue_keys_kernel(const unsigned* ranges, long long T,
+                                  unsigned* keys, unsigned* vals) {
   behind_previous();
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < T;
        t += (long long)gridDim.x * blockDim.x) {

@@ -146,7 +146,7 @@ __device__ __forceinline__ void for_sh_block(const float* sh, long long g, const
 #pragma unroll
     for (int i = 0; i < 12; ++i) {
       if (4 * i < 3 * K) {
-        const float4 t = __ldg(reinterpret_cast<const float4*>(p) + i);
+        const float4 t = reinterpret_cast<const float4*>(p)[i];
         f(4 * i, t.x);
         if (4 * i + 1 < 3 * K) f(4 * i + 1, t.y);
         if (4 * i + 2 < 3 * K) f(4 * i + 2, t.z);
@@ -158,9 +158,9 @@ __device__ __forceinline__ void for_sh_block(const float* sh, long long g, const
     for (int k = 0; k < 16; ++k) {
       if (k < K) {
         const float* q = sh + g * L.gs + k * L.ks;
-        f(3 * k, __ldg(q));
-        f(3 * k + 1, __ldg(q + 1));
-        f(3 * k + 2, __ldg(q + 2));
+        f(3 * k, q[0]);
+        f(3 * k + 1, q[1]);
+        f(3 * k + 2, q[2]);
       }
     }
   }
@@ -187,11 +187,11 @@ __device__ __forceinline__ Activated activate(const float* means, const float* l
                                               const float* quats, const float* opacity_logits,
                                               int g) {
   Activated a;
-  a.mean[0] = __ldg(means + 3ll * g);
-  a.mean[1] = __ldg(means + 3ll * g + 1);
-  a.mean[2] = __ldg(means + 3ll * g + 2);
-  for (int k = 0; k < 3; ++k) a.s[k] = expf(__ldg(log_scales + 3ll * g + k));
-  float4 q = __ldg(reinterpret_cast<const float4*>(quats) + g);
+  a.mean[0] = means[3ll * g];
+  a.mean[1] = means[3ll * g + 1];
+  a.mean[2] = means[3ll * g + 2];
+  for (int k = 0; k < 3; ++k) a.s[k] = expf(log_scales[3ll * g + k]);
+  float4 q = reinterpret_cast<const float4*>(quats)[g];
   float n2 = q.x * q.x + q.y * q.y + q.z * q.z + q.w * q.w;
   a.qnorm = sqrtf(n2);
   float inv = rsqrtf(n2);
@@ -206,7 +206,7 @@ __device__ __forceinline__ Activated activate(const float* means, const float* l
   a.Sig[3] = M[3] * M[3] + M[4] * M[4] + M[5] * M[5];
   a.Sig[4] = M[3] * M[6] + M[4] * M[7] + M[5] * M[8];
   a.Sig[5] = M[6] * M[6] + M[7] * M[7] + M[8] * M[8];
-  float o = __ldg(opacity_logits + g);
+  float o = opacity_logits[g];
   a.sigma = 1.f / (1.f + expf(-o));
   return a;
 }
@@ -479,9 +479,9 @@ constexpr int pre_ctas_per_sm() {
 }
 template <int DT, int DEG>
 __global__ void __launch_bounds__(256, pre_ctas_per_sm<DEG>()) preprocess_kernel(
-    const float* __restrict__ means, const float* __restrict__ log_scales,
-    const float* __restrict__ quats, const float* __restrict__ opacity_logits,
-    const float* __restrict__ sh, int N, const CamTable ct, float dilation, float near_z,
+    const float* means, const float* log_scales,
+    const float* quats, const float* opacity_logits,
+    const float* sh, int N, const CamTable ct, float dilation, float near_z,
     const ShPtr shp, gs_proj out) {
   behind_previous();
   int g = blockIdx.x * blockDim.x + threadIdx.x;
@@ -500,6 +500,9 @@ __global__ void __launch_bounds__(256, pre_ctas_per_sm<DEG>()) preprocess_kernel
   for (int v = 0; v < ct.V; ++v) {
     const CamInfo& c = ct.c[v];
     long long row = (long long)v * N + g;
+    // (read again per view, from L1: holding it across the view's SH sum spills)
+    if (DEG >= 2 && v > 0)
+      for (int k = 0; k < 3; ++k) a.mean[k] = means[3ll * g + k];
     float depth = depth_of(c, a.mean);
     out.depth[row] = depth;
     bool vis = depth > near_z;
@@ -627,12 +630,12 @@ struct ShCoef {
   static constexpr int K = (DEG + 1) * (DEG + 1);
   static constexpr bool kCached = DEG == 0;
   float c[kCached ? 3 * K : 1];
-  __device__ __forceinline__ void load(const float* __restrict__ sh, long long g, const ShPtr& L) {
+  __device__ __forceinline__ void load(const float* sh, long long g, const ShPtr& L) {
     if constexpr (kCached) for_sh_block(sh, g, L, K, [&](int e, float v) { c[e] = v; });
   }
   // f(e, value) for e < 3K, like for_sh_block
   template <typename F>
-  __device__ __forceinline__ void each(const float* __restrict__ sh, long long g, const ShPtr& L,
+  __device__ __forceinline__ void each(const float* sh, long long g, const ShPtr& L,
                                        F&& f) const {
     if constexpr (kCached) {
 #pragma unroll
@@ -648,9 +651,9 @@ struct ShCoef {
 // the Gaussian stores, later ones add.
 template <int DEG, bool SHREG, bool WHITE>
 __device__ __forceinline__ void adjoint_view(
-    int g, int v, const Activated& a, const float* __restrict__ sh, int N, const CamTable& ct,
-    float dilation, const ShPtr& shp, float* __restrict__ grad2d,
-    AdjAcc<SHREG ? DEG : 0>& acc, bool first_view, bool vec_out, float* __restrict__ g_sh,
+    int g, int v, const Activated& a, const float* sh, int N, const CamTable& ct,
+    float dilation, const ShPtr& shp, float* grad2d,
+    AdjAcc<SHREG ? DEG : 0>& acc, bool first_view, bool vec_out, float* g_sh,
     const ShCoef<DEG>& shc) {
   constexpr int sh_deg = DEG;
   constexpr int K = AdjAcc<DEG>::K;
@@ -836,8 +839,8 @@ __device__ __forceinline__ void adjoint_view(
 template <int DEG, bool SHREG>
 __device__ __forceinline__ void adjoint_finish(
     int g, const Activated& a, const AdjAcc<DEG>& acc, const ShPtr& shp, bool vec_out,
-    float* __restrict__ g_means, float* __restrict__ g_ls, float* __restrict__ g_quats,
-    float* __restrict__ g_opac, float* __restrict__ g_sh) {
+    float* g_means, float* g_ls, float* g_quats,
+    float* g_opac, float* g_sh) {
   constexpr int K = AdjAcc<DEG>::K;
   constexpr int kSectorFloats = (3 * K + 7) / 8 * 8;  // 3K rounded up to 32 bytes
   float* gsh = g_sh + (long long)g * shp.gs;  // (vec_out: layout 0, the block's start)
@@ -889,7 +892,7 @@ __device__ __forceinline__ void adjoint_finish(
 // marked in a bitmap: bit row % 32 of the third pad float (float 10) of
 // grad2d's row row / 32, zeroed with grad2d.
 __device__ __forceinline__ unsigned touched_word(const float* grad2d, long long word) {
-  return __ldg(reinterpret_cast<const unsigned*>(grad2d) + 12 * word + 10);
+  return reinterpret_cast<const unsigned*>(grad2d)[12 * word + 10];
 }
 
 // Adjoint of Gaussian g: sums its parts over the views whose blending touched
@@ -897,11 +900,11 @@ __device__ __forceinline__ unsigned touched_word(const float* grad2d, long long 
 // zeroes them), so the Gaussians no pixel met keep zeros.
 template <int DEG, bool WHITE>
 __device__ __forceinline__ void adjoint_gaussian(
-    int g, const float* __restrict__ means, const float* __restrict__ log_scales,
-    const float* __restrict__ quats, const float* __restrict__ opacity_logits,
-    const float* __restrict__ sh, int N, const CamTable& ct, float dilation, const ShPtr& shp,
-    float* __restrict__ grad2d, float* __restrict__ g_means, float* __restrict__ g_ls,
-    float* __restrict__ g_quats, float* __restrict__ g_opac, float* __restrict__ g_sh) {
+    int g, const float* means, const float* log_scales,
+    const float* quats, const float* opacity_logits,
+    const float* sh, int N, const CamTable& ct, float dilation, const ShPtr& shp,
+    float* grad2d, float* g_means, float* g_ls,
+    float* g_quats, float* g_opac, float* g_sh) {
   const bool vec_out = shp.vec && (reinterpret_cast<uintptr_t>(g_sh) & 15) == 0;
   const Activated a = activate(means, log_scales, quats, opacity_logits, g);
   constexpr bool SHREG = DEG < 3;
@@ -951,11 +954,11 @@ constexpr int adj_ctas_per_sm() { return DEG == 2 ? 3 : GS_ADJ_CTAS; }
 
 template <int DEG, bool WHITE>
 __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preprocess_bwd_kernel(
-    const float* __restrict__ means, const float* __restrict__ log_scales,
-    const float* __restrict__ quats, const float* __restrict__ opacity_logits,
-    const float* __restrict__ sh, int N, const CamTable ct, float dilation, const ShPtr shp,
-    int chunk, float* __restrict__ grad2d, float* __restrict__ g_means, float* __restrict__ g_ls,
-    float* __restrict__ g_quats, float* __restrict__ g_opac, float* __restrict__ g_sh) {
+    const float* means, const float* log_scales,
+    const float* quats, const float* opacity_logits,
+    const float* sh, int N, const CamTable ct, float dilation, const ShPtr shp,
+    int chunk, float* grad2d, float* g_means, float* g_ls,
+    float* g_quats, float* g_opac, float* g_sh) {
   behind_previous();
   __shared__ unsigned s_any[kAdjChunk / 32];
   __shared__ unsigned short s_idx[kAdjChunk];
@@ -1018,10 +1021,10 @@ void launch_adjoint(const float* means, const float* log_scales, const float* qu
 // (F^T F = log2(e) / 2 conic, F lower triangular): a = 2 ln 2 (f11^2 + f21^2),
 // b = 2 ln 2 f21 f22, c = 2 ln 2 f22^2.
 template <int DT>
-__global__ void __launch_bounds__(256) grad2d_attr_kernel(const void* __restrict__ recs,
-                                                          const unsigned* __restrict__ tiles_touched,
-                                                          const float* __restrict__ grad2d,
-                                                          long long rows, float* __restrict__ out) {
+__global__ void __launch_bounds__(256) grad2d_attr_kernel(const void* recs,
+                                                          const unsigned* tiles_touched,
+                                                          const float* grad2d,
+                                                          long long rows, float* out) {
   behind_previous();
   for (long long row = (long long)blockIdx.x * blockDim.x + threadIdx.x; row < rows;
        row += (long long)gridDim.x * blockDim.x) {

@@ -218,7 +218,7 @@ struct FwdArgs {
 // the memory bandwidth mostly idle, so this costs a few issue slots where a
 // separate zeroing kernel (even on a second stream: the forward's CTAs fill
 // the register file, nothing runs beside them) added its whole duration.
-__device__ __forceinline__ void zero_stripe(uint4* __restrict__ z, unsigned long long n16) {
+__device__ __forceinline__ void zero_stripe(uint4* z, unsigned long long n16) {
   const unsigned long long per = (n16 + gridDim.x - 1) / gridDim.x;
   const unsigned long long b = (unsigned long long)blockIdx.x * per;
   const unsigned long long e = min(n16, b + per);

@@ -119,8 +119,8 @@ __device__ __forceinline__ ChannelRange channels_of(unsigned parts, unsigned par
 }
 
 __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
-    const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
-    float* __restrict__ maps /* 15 planes of P */, long long P, double* __restrict__ partials) {
+    const float* image, const float* target, const SsimViews sv,
+    float* maps /* 15 planes of P */, long long P, double* partials) {
   behind_previous();
   __shared__ __align__(16) float2 s_xy[kSsimS][kSsimP];
   __shared__ __align__(16) float2 s_m[2 * kQS][kSsimB];  // horizontal sums of (x, y)
@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(kSsimThreads, 4) ssim_fwd_kernel(
 }
 
 __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
-    const float* __restrict__ image, const float* __restrict__ target, const SsimViews sv,
-    const float* __restrict__ maps, long long P, float* __restrict__ dimg) {
+    const float* image, const float* target, const SsimViews sv,
+    const float* maps, long long P, float* dimg) {
   behind_previous();
   __shared__ __align__(16) float2 s_ab[kSsimS][kSsimP];  // (a - 2 (mu_x - c) b - (mu_y - c') e, b)
   __shared__ __align__(16) float s_e[kSsimS][kSsimP];
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
   for (int ch = cr.first; ch < cr.end; ++ch) {
     // block constants: the image and target at the block's first pixel
     const float cx = image[p0 + ch], cy = target[p0 + ch];
-    const float* __restrict__ mp = maps + (long long)(5 * ch) * P;
+    const float* mp = maps + (long long)(5 * ch) * P;
     for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
       const int r = i / kSsimS, c = i - r * kSsimS;
       const int yy = k.by - kSsimR + r, xx = k.bx - kSsimR + c;
