@@ -244,7 +244,9 @@ int gs_preprocess(const float* means, const float* log_scales, const float* quat
  * Up to 2^21 rows part of the work is one cooperative launch whose blocks meet
  * at grid barriers; should a barrier's bounded wait (about a second) run out,
  * the call reports GS_ERR_TIMEOUT (in *status_dev, and as its return value with
- * num_pairs_host), with no pairs. */
+ * num_pairs_host): every range is empty and *num_pairs_dev and *num_pairs_host
+ * are 0, which is not a size to regrow the buffers to; the next call starts
+ * afresh. */
 int gs_bin_sort(const gs_proj* proj, int N, const gs_camera* cams_host, int V, int tile_size,
                 void* workspace, size_t workspace_bytes, long long pair_capacity,
                 unsigned* sorted_vals, unsigned long long* sorted_keys, unsigned* tile_ranges,

@@ -801,6 +801,7 @@ struct CoopArgs {
   unsigned* cnt;    // [grid] visible rows per CTA
   unsigned* range;  // [~smallest, largest] visible key (zero)
   unsigned* bar;    // barrier arrivals (zero)
+  int polls;        // reads of bar after which a barrier's wait gives up
   const int* rect;
   const unsigned* rect8;
   int N;
@@ -839,7 +840,7 @@ __device__ __forceinline__ bool coop_barrier(const CoopArgs& a, CoopShared& s, u
       __threadfence();  // (after the block barrier: covers the whole CTA's writes)
       atomicAdd(a.bar, 1u);
       int ok = 0;
-      for (int i = 0; i < (1 << 21) && !ok; ++i) {  // (about a second)
+      for (int i = 0; i < a.polls && !ok; ++i) {
         unsigned x;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(a.bar) : "memory");
         ok = x >= want;
@@ -1171,6 +1172,16 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
     counts_check(a.co, (long long)grand, (long long)pp);
   }
 }
+
+// A barrier's wait, about a second.  The bounds-checked debug build lets a test
+// shorten it for the calling thread's next calls (gs_debug_sort_polls).
+constexpr int kBarrierPolls = 1 << 21;
+#ifdef GS_DEBUG_BOUNDS
+thread_local int g_barrier_polls = kBarrierPolls;
+int barrier_polls() { return g_barrier_polls; }
+#else
+int barrier_polls() { return kBarrierPolls; }
+#endif
 
 template <bool CLUSTER>
 cudaError_t allow_coop_smem() {
@@ -2126,6 +2137,12 @@ int bits_for(long long count) {
 
 GS_BOUNDS_READER(bounds_status_binning)
 
+#ifdef GS_DEBUG_BOUNDS
+extern "C" void gs_debug_sort_polls(int polls) {
+  g_barrier_polls = polls >= 0 ? polls : kBarrierPolls;
+}
+#endif
+
 size_t bin_sort_workspace_size(long long n_rows, long long cap, long long total_tiles) {
   return carve(nullptr, n_rows, cap, total_tiles).bytes;
 }
@@ -2169,6 +2186,7 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     a.cnt = w.hist + (size_t)kRadixMaxPasses * kCoopGrid * kRadixBins;
     a.range = range;
     a.bar = reinterpret_cast<unsigned*>(w.counters + 11);
+    a.polls = barrier_polls();
     a.rect = proj->rect;
     a.rect8 = rect8;
     a.N = N;

@@ -56,8 +56,11 @@ def capture_step(fn, device="cuda"):
     stream and returns the graph; graph.replay() reruns the step with the
     buffers' current contents.  Run the step once eagerly first (the pair
     buffers are sized there); list construction inside the graph keeps the
-    pair count on the device (bin_sort(sync=False)): after a replay, a nonzero
-    status_dev means the pair buffers overflowed."""
+    pair count on the device (bin_sort(sync=False)): after a replay, read
+    status_dev.  gs.GS_ERR_CAPACITY: the pair buffers overflowed and
+    num_pairs_dev holds the count to regrow them to.  gs.GS_ERR_TIMEOUT: the
+    sort's bounded wait ran out, the lists are empty and num_pairs_dev is 0 (no
+    size to regrow to): replay again."""
     g = torch.cuda.CUDAGraph()
     s = torch.cuda.Stream(device=device)
     s.wait_stream(torch.cuda.current_stream(device))
