@@ -459,14 +459,17 @@ struct BwdArgs {
   unsigned* counter;
   unsigned long long rows, pixels;  // extents of the record and per-pixel arrays
   ZeroRegions zero;                 // zeroed by the kernel's CTAs
+  unsigned blend_ctas;              // CTAs that blend; any beyond them only zero
 };
 
-// A CTA's stripes of the regions (16-byte stores; the first CTA also takes the
-// ends off 16-byte boundaries).  The backward's CTAs zero the parameter
+// Stripe `part` of `parts` of the regions (16-byte stores; the first also takes
+// the ends off 16-byte boundaries).  The backward's CTAs zero the parameter
 // gradients this way after their tiles: the stores drain while other CTAs
 // blend, which is bound by instruction issue, and no memsets (five, on a
-// second stream forked and joined by events) stand beside the kernel.
-__device__ __forceinline__ void zero_regions(const ZeroRegions& z) {
+// second stream forked and joined by events) stand beside the kernel.  Where few
+// CTAs blend, further ones take the zeroing (see kZeroBlendCtas).
+__device__ __forceinline__ void zero_regions(const ZeroRegions& z, unsigned part,
+                                             unsigned parts) {
 #pragma unroll 1
   for (int r = 0; r < ZeroRegions::kMax; ++r) {
     float* p = z.p[r];
@@ -475,12 +478,12 @@ __device__ __forceinline__ void zero_regions(const ZeroRegions& z) {
     const unsigned long long head =
         min(n, (unsigned long long)((0u - (unsigned)(reinterpret_cast<uintptr_t>(p) >> 2)) & 3u));
     const unsigned long long n16 = (n - head) / 4;
-    const unsigned long long per = (n16 + gridDim.x - 1) / gridDim.x;
-    const unsigned long long b = (unsigned long long)blockIdx.x * per, e = min(n16, b + per);
+    const unsigned long long per = (n16 + parts - 1) / parts;
+    const unsigned long long b = (unsigned long long)part * per, e = min(n16, b + per);
     uint4* q = reinterpret_cast<uint4*>(p + head);
     for (unsigned long long i = b + threadIdx.x; i < e; i += blockDim.x)
       __stcs(q + i, make_uint4(0u, 0u, 0u, 0u));
-    if (blockIdx.x == 0) {
+    if (part == 0) {
       if (threadIdx.x < head) p[threadIdx.x] = 0.f;
       const unsigned long long t0 = head + 4 * n16;
       if (t0 + threadIdx.x < n) p[t0 + threadIdx.x] = 0.f;  // (at most 3)
@@ -822,6 +825,8 @@ __global__ void __launch_bounds__(TS * TS / PPT, (TS == 16 && PPT != 4) ? 4 * PP
                                                                     const BwdArgs a,
                                                                     int persistent) {
   behind_previous();
+  if (blockIdx.x >= a.blend_ctas)
+    return zero_regions(a.zero, blockIdx.x - a.blend_ctas, gridDim.x - a.blend_ctas);
   if (persistent) {
     __shared__ unsigned s_t;
     for (;;) {
@@ -836,7 +841,7 @@ __global__ void __launch_bounds__(TS * TS / PPT, (TS == 16 && PPT != 4) ? 4 * PP
     const int t = blockIdx.x;
     bwd_tile<DT, TS, PPT, B>(ct, rc, a, a.order ? (int)a.order[t] : t);
   }
-  zero_regions(a.zero);
+  if (gridDim.x == a.blend_ctas) zero_regions(a.zero, blockIdx.x, gridDim.x);
 }
 
 int record_event(void* ev, cudaStream_t st) {
@@ -858,10 +863,25 @@ void launch_fwd_b(const CamTable& ct, const RenderConsts& rc, const FwdArgs& a, 
                   a, pers);
 }
 
+// Zeroing the parameter gradients in stripes after the tiles wants many CTAs: with
+// few, the rest of the chip stands idle while those store (a one-tile view of 1M
+// Gaussians, 236 MB: 3772 us).  Up to two blending CTAs per SM the grid gets two more
+// per SM that only zero, beside the blending.  Measured (adjoint and projection
+// adjoint, us, zeroing after the tiles / in CTAs of its own):
+//             1 tile       16         64         144        256        320        475
+//   10k    244 / 209   142 / 140   99 / 97    80 / 80    70 / 69    70 / 70    89 / 87
+//   1M    3772 / 229   462 / 263  263 / 227  212 / 211  209 / 202  201 / 190  201 / 212
+//   3M   10904 / 283  1068 / 459  418 / 336  324 / 324  351 / 339  359 / 327  340 / 382
+// (Five memsets on a second stream, for 3M Gaussians: 555, 829, 564, -, 505, -, 466.)
+// Four CTAs per SM that zero take the same to 6 % longer.
+constexpr int kZeroBlendCtas = 2 * 152, kZeroCtas = 2 * 152;
+
 template <int DT, int TS, int PPT, int B>
-void launch_bwd_b(const CamTable& ct, const RenderConsts& rc, const BwdArgs& a, int ctas,
+void launch_bwd_b(const CamTable& ct, const RenderConsts& rc, BwdArgs a, int ctas,
                   cudaStream_t st) {
-  const int grid = ctas > 0 ? ctas : ct.total_tiles;
+  const int blend = ctas > 0 ? ctas : ct.total_tiles;
+  a.blend_ctas = (unsigned)blend;
+  const int grid = blend + (blend <= kZeroBlendCtas ? kZeroCtas : 0);
   launch_behind(render_bwd_kernel<DT, TS, PPT, B>, dim3(grid), TS * TS / PPT, st, ct, rc, a,
                 ctas > 0 ? 1 : 0);
 }
