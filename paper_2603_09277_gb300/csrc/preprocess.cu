@@ -932,20 +932,36 @@ __device__ __forceinline__ void adjoint_gaussian(
                                          g_sh);
 }
 
-// The adjoint over the touched Gaussians.  A CTA takes `chunk` consecutive
-// Gaussians: it merges the views' bitmap words of its range in shared memory,
-// compacts the touched ones, and its threads take one each.  On dense scenes
-// most visible rows lie behind the pixels' last blended entries: reading the
-// moment rows and parameters of every visible Gaussian was most of this
-// kernel (8 views of 3M Gaussians, where the blending reaches about 1 % of the 24 M
-// visible rows: 453 -> 51 us).  Compacting by chunk instead of into one list keeps
-// the parameter reads and gradient writes of neighbours together and needs no
-// launch of its own.
 constexpr int kAdjThreads = 128;
 constexpr int kAdjChunk = 2048;  // most Gaussians of a CTA
-// CTAs per SM the register budget allows.  Measured inside the step: 8 views of 3M
-// Gaussians (degree 0) 63.6 us at 4, 59.1 at 5, 60.6 at 6; a 1M-Gaussian view
-// (degree 3) 33.4, 33.3 and 34.6.
+constexpr int kAdjRun = 128;     // of which this many are consecutive
+
+// First Gaussian of word w of a CTA's chunk (see preprocess_bwd_kernel).
+__device__ __forceinline__ long long adj_first(int w) {
+  constexpr int kWords = kAdjRun / 32;
+  return ((long long)(w / kWords) * gridDim.x + blockIdx.x) * kAdjRun + 32 * (w % kWords);
+}
+
+// The adjoint over the touched Gaussians.  A CTA takes `chunk` Gaussians: it merges
+// the views' bitmap words of its Gaussians in shared memory, compacts the touched
+// ones, and its threads take one each.  On dense scenes most visible rows lie behind
+// the pixels' last blended entries: reading the moment rows and parameters of every
+// visible Gaussian was most of this kernel (8 views of 3M Gaussians, where the
+// blending reaches about 1 % of the 24 M visible rows: 454 -> 52 us in a captured
+// step).  Compacting by chunk instead of into one list needs no launch of its own.
+//
+// The chunk is runs of 128 consecutive Gaussians, a grid's stride apart: the runs
+// keep the parameter reads and gradient writes of neighbours together, and the stride
+// deals the touched Gaussians out evenly where the ids follow space (sorted or grown
+// scenes, whose views touch a few ranges of ids).  With consecutive chunks those
+// ranges were left to a few CTAs.  Measured (captured, us, ids at random / in Morton
+// order): 1M clusters, degree 3, one view 47 / 86 with consecutive chunks, 48 / 37
+// with runs; 4 views 198 / 208, 180 / 134; 8 views of 3M 50 / 94, 52 / 45 (runs of
+// 256 there: 52 / 48).
+//
+// CTAs per SM the register budget allows.  Measured under stage events in eager
+// steps: 8 views of 3M Gaussians (degree 0) 63.6 us at 4, 59.1 at 5, 60.6 at 6; a
+// 1M-Gaussian view (degree 3) 33.4, 33.3 and 34.6.
 #ifndef GS_ADJ_CTAS
 #define GS_ADJ_CTAS 5
 #endif
@@ -964,8 +980,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
   __shared__ unsigned short s_idx[kAdjChunk];
   __shared__ unsigned s_n;
   const int tid = threadIdx.x;
-  const long long g0 = (long long)blockIdx.x * chunk;
-  const int n = (int)min((long long)chunk, N - g0), words = (n + 31) / 32;
+  const int words = chunk / 32;
   for (int i = tid; i < words; i += kAdjThreads) s_any[i] = 0u;
   if (tid == 0) s_n = 0u;
   __syncthreads();
@@ -973,11 +988,13 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
 #pragma unroll 4
   for (int i = tid; i < ct.V * words; i += kAdjThreads) {
     const int v = i / words, w = i - v * words;
-    const long long r0 = (long long)v * N + g0 + 32 * w;  // the word's first row
+    const long long g = adj_first(w);
+    if (g >= N) continue;
+    const long long r0 = (long long)v * N + g;  // the word's first row
     const unsigned lo = touched_word(grad2d, r0 >> 5);
     const unsigned hi = (r0 | 31) + 1 < rows ? touched_word(grad2d, (r0 >> 5) + 1) : 0u;
     unsigned m = __funnelshift_r(lo, hi, (unsigned)(r0 & 31));
-    if (n - 32 * w < 32) m &= (1u << (n - 32 * w)) - 1u;  // (rows of the next view)
+    if (N - g < 32) m &= (1u << (int)(N - g)) - 1u;  // (rows of the next view)
     if (m) atomicOr(&s_any[w], m);
   }
   __syncthreads();
@@ -990,7 +1007,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
   __syncthreads();
   const int cnt = (int)s_n;
   for (int i = tid; i < cnt; i += kAdjThreads) {
-    const long long g = g0 + s_idx[i];
+    const long long g = adj_first(s_idx[i] >> 5) + (s_idx[i] & 31);
     if (!GS_IN_BOUNDS(g, N, 301)) continue;
     adjoint_gaussian<DEG, WHITE>((int)g, means, log_scales, quats, opacity_logits, sh, N, ct,
                                  dilation, shp, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
@@ -1002,9 +1019,10 @@ void launch_adjoint(const float* means, const float* log_scales, const float* qu
                     const float* opacity_logits, const float* sh, int N, const CamTable& ct,
                     const gs_params* prm, float* grad2d, float* g_means, float* g_ls,
                     float* g_quats, float* g_opac, float* g_sh, cudaStream_t st) {
-  // a chunk per resident CTA, in whole warps' words, at most kAdjChunk
+  // a chunk per resident CTA, in whole runs, at most kAdjChunk
   const long long per = ((long long)N + 152 * GS_ADJ_CTAS - 1) / (152 * GS_ADJ_CTAS);
-  const int chunk = (int)std::min<long long>(kAdjChunk, (per + kAdjThreads - 1) / kAdjThreads * kAdjThreads);
+  const int chunk = (int)std::min<long long>(kAdjChunk, (per + kAdjRun - 1) / kAdjRun * kAdjRun);
+  static_assert(kAdjChunk % kAdjRun == 0 && kAdjRun % 32 == 0, "whole runs of whole words");
   const unsigned grid = (unsigned)(((long long)N + chunk - 1) / chunk);
   if (prm->attr_dtype == GS_ATTR_F32)
     launch_behind(preprocess_bwd_kernel<DEG, true>, dim3(grid), kAdjThreads, st, means, log_scales,
