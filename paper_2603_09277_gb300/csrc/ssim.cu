@@ -263,8 +263,10 @@ __global__ void __launch_bounds__(kSsimThreads, 5) ssim_bwd_kernel(
   const ChannelRange cr = channels_of(gridDim.y, blockIdx.y);
 #pragma unroll 1
   for (int ch = cr.first; ch < cr.end; ++ch) {
-    // block constants: the image and target at the middle pixel
-    const float cx = image[p0 + ch], cy = target[p0 + ch];
+    // block constants: the image and target at the middle pixel (0 in place of one
+    // that is not finite, which would spread over the whole block)
+    const float ix = image[p0 + ch], iy = target[p0 + ch];
+    const float cx = isfinite(ix) ? ix : 0.f, cy = isfinite(iy) ? iy : 0.f;
     const float* mp = maps + (long long)(5 * ch) * P;
     for (int i = threadIdx.x; i < kSsimS * kSsimS; i += kSsimThreads) {
       const int r = i / kSsimS, c = i - r * kSsimS;
