@@ -699,6 +699,11 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
   }
   const float2 ry2 = make_float2(tg.ry0, tg.ry0 + 1.f);
   float U1 = -gH[0] * Rent[0];  // (one pixel per thread)
+  // lanes that add directly: any number where the warp holds a gradient that is not
+  // finite, which stays with the entries its pixel blends that way (in the warp's sum
+  // a lane that takes no part of an entry would add 0 times that gradient)
+  const int direct = PPT == 1 && __any_sync(kFull, !isfinite(gr[0] + gg[0] + gb[0] + gH[0]))
+                         ? 32 : DirectLanes<PPT>::value;
   if (tid == 0) s_max = 0u;
   __syncthreads();
   if (mylast) atomicMax(&s_max, mylast);
@@ -797,7 +802,7 @@ __device__ __forceinline__ void bwd_tile(const CamTable& ct, const RenderConsts&
       if constexpr (PPT > 2) who = __ballot_sync(kFull, contrib);
       if (who) {
         float* G = a.grad2d + 12ll * s_row[k];
-        if (__popc(who) <= DirectLanes<PPT>::value) {
+        if (__popc(who) <= direct) {
           // few contributing lanes: each adds its own values (three vector
           // atomics) instead of the 12-shuffle warp reduction
           if (contrib) {
