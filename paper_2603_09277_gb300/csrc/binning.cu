@@ -766,11 +766,24 @@ __device__ __forceinline__ int radix_result(const unsigned* range, int bits) {
 // they are 13 launches of 4 to 10 us each whatever the rows, most of it
 // launching, filling and draining the chip and re-reading arguments: 10k rows
 // took about 75 us, 1M rows of which 70k are visible about 110 us.  Here the
-// counts a phase needs from all CTAs are summed by each CTA for itself, and a
-// pass's scatter also counts the next pass's digits (one reduction per item
-// into the chunk that will own it), so a pass is one phase.  Above kCoopRows the
-// passes are long enough for the separate kernels, whose three CTAs per SM hide
-// more latency.
+// counts a phase needs from all CTAs are summed by each CTA for itself, and up to
+// kCountAhead visible rows a pass's scatter also counts the next pass's digits (one
+// reduction per item into the chunk that will own it), so a pass is one phase.
+// Beyond, those reductions collide in L2 and a CTA counts its own chunk in shared
+// memory instead, a phase more.  Above kCoopRows the passes are long enough for the
+// separate kernels, whose three CTAs per SM hide more latency.
+//
+// Measured, whole list construction replayed from a graph, us:
+//   counted ahead / counted in the pass, all rows visible: 20k 66 / 66, 60k 76 / 76,
+//   80k 76 / 75, 200k 90 / 87, 1M 168 / 152, 2.1M 281 / 247; 7 % visible (8k: 560 rows)
+//   51 / 56, 50k 62 / 64, 1M (70k visible) 86 / 84.
+//   one launch / separate kernels, all rows visible: 100k 80 / 80, 1M 152 / 148, 1.5M
+//   197 / 182, 2.1M 247 / 239, 2.6M 295 / 270, 6M 560 / 479; 30 % visible: 1M 98 / 113,
+//   2.1M 139 / 150, 6M 270 / 253; 7 %: 1M 84 / 105, 2.1M 94 / 127, 6M 162 / 177.
+//   (The host knows the rows, not how many are visible: the line lies where the one
+//   launch costs at most 8 % with all of them visible and gains a quarter with few.)
+//   one cluster / the grid, all rows visible: 2k 55 / 60, 16k 66 / 68, 32,768 70 / 72,
+//   40k (two tiles per CTA of the cluster) 88 / 74; 7 % visible: 32,768 58 / 62.
 //
 // Every CTA is resident (cooperative launch).  The barrier's wait is bounded:
 // when it runs out, the CTA reports GS_ERR_TIMEOUT and leaves, the others run
@@ -791,6 +804,7 @@ constexpr int kCoopCluster = 8;
 constexpr long long kClusterRows = (long long)kCoopCluster * kCoopTile;
 static_assert(kClusterRows / (kCoopCluster * kCoopWarps) <= 32 * kCoopGroups,
               "a warp's rows of the cluster form fit");
+constexpr unsigned kCountAhead = 65536;
 static_assert(kCoopTile == 1 << kCoopShift, "chunks are whole tiles");
 
 struct CoopArgs {
@@ -945,13 +959,16 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
   const int bits = n && hi > lo ? 32 - __clz(hi - lo) : 0;
   const RadixPlan pl = radix_plan_bits(base, bits);
   const unsigned dmask = (1u << pl.dbits) - 1u;  // (dbits 0: no pass)
-  // chunks of whole tiles, a power of two of them: chunk = position >> shift
-  int shift = kCoopShift;
-  while (((unsigned long long)G << shift) < n) ++shift;
+  // chunks of `tiles` whole tiles: the chunk of tile t is t / tiles, by a reciprocal
+  // that is exact below 2^16 / tiles tiles (here at most kCoopRows / kCoopTile)
+  const unsigned tiles = max(1u, (n + (unsigned)G * kCoopTile - 1u) / ((unsigned)G * kCoopTile));
+  const unsigned per_chunk = 65536u / tiles + 1u, chunk = tiles * kCoopTile;
   auto count = [&](int pass, unsigned pos, unsigned k) {
-    atomicAdd(a.hist + ((long long)pass * G + (pos >> shift)) * kRadixBins +
+    const unsigned c = ((pos >> kCoopShift) * per_chunk) >> 16;
+    atomicAdd(a.hist + ((long long)pass * G + c) * kRadixBins +
                   (((k - base) >> (pass * pl.dbits)) & dmask), 1u);
   };
+  const bool ahead = n <= kCountAhead;  // (see the top)
   int buf = pl.passes & 1;  // (the result lands in buffer 0)
   {
     unsigned at = before + woff;
@@ -965,7 +982,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
         const unsigned k = __float_as_uint(a.rows.depth[j]), pos = at + __popc(m & lt);
         if (pl.passes) {
           ko[pos] = k;
-          count(0, pos, k);
+          if (ahead) count(0, pos, k);
         }
         vo[pos] = (unsigned)j;
       }
@@ -974,12 +991,39 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
   }
   if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
   // C. stable passes over the digits, as radix_downsweep_kernel
-  const int chunks = (int)((n + (1u << shift) - 1u) >> shift);
+  const int chunks = (int)((n + chunk - 1u) / chunk);
   for (int pass = 0; pass < pl.passes; ++pass, buf ^= 1) {
+    if (!ahead) {  // this chunk's digit counts
+      if (cta < chunks) {
+        const unsigned c0 = (unsigned)cta * chunk, c1 = min(n, c0 + chunk);
+        for (int i = tid; i < kCoopWarps * (kRadixBins + 1); i += kCoopThreads) (&s.wc[0][0])[i] = 0u;
+        __syncthreads();
+        for (unsigned t0 = c0; t0 < c1; t0 += kCoopTile) {
+          unsigned kk[kRadixIpt];
+#pragma unroll
+          for (int i = 0; i < kRadixIpt; ++i) {
+            const unsigned p = t0 + tid + kCoopThreads * i;
+            kk[i] = p < c1 ? __ldcg(a.k[buf] + p) : 0u;
+          }
+#pragma unroll
+          for (int i = 0; i < kRadixIpt; ++i)
+            if (t0 + tid + kCoopThreads * i < c1)
+              atomicAdd(&s.wc[w][((kk[i] - base) >> (pass * pl.dbits)) & dmask], 1u);
+        }
+        __syncthreads();
+        if (tid < kRadixBins) {
+          unsigned sum = 0u;
+#pragma unroll
+          for (int ww = 0; ww < kCoopWarps; ++ww) sum += s.wc[ww][tid];
+          a.hist[((long long)pass * G + cta) * kRadixBins + tid] = sum;
+        }
+      }
+      if (!coop_barrier<CLUSTER>(a, s, phase++)) return;
+    }
     if (cta < chunks) {
       const unsigned* __restrict__ ki = a.k[buf];
       const unsigned* __restrict__ vi = a.v[buf];
-      const unsigned c0 = (unsigned)cta << shift, c1 = min(n, c0 + (1u << shift));
+      const unsigned c0 = (unsigned)cta * chunk, c1 = min(n, c0 + chunk);
       // (a tile's items are requested while the one before is ranked)
       unsigned nk[kRadixIpt], nv[kRadixIpt];
       auto request = [&](unsigned t0) {
@@ -1092,7 +1136,7 @@ __global__ void __launch_bounds__(kCoopThreads, 1) depth_sort_kernel(const CoopA
           if (!GS_IN_BOUNDS(pos, n, 202)) continue;
           if (more) {
             ko[pos] = kk;
-            count(pass + 1, pos, kk);
+            if (ahead) count(pass + 1, pos, kk);
           }
           vo[pos] = s.val[i];
         }
