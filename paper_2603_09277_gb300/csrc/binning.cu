@@ -1628,11 +1628,11 @@ __global__ void __launch_bounds__(256) st_count_kernel(
   __shared__ unsigned s_start[256], s_first[257];  // (totals) items, segments before a super-tile
   __shared__ unsigned s_w[8];
   __shared__ __align__(16) Segment s_seg[256];  // (totals) the CTA's segments
-  __shared__ unsigned char s_st[256];           // and their super-tiles
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int t = lane & 3, q = lane >> 2;  // the lane's four items of 16; its tile row and column
   const int sr = 14 - q, sc = 6 - q;      // moves its bits to bit 14 (a rotation by -1 for column 7)
   long long G;
+  static_assert(kRadixBins == 256, "one digit per thread: S <= 256 where the segments are formed here");
   const bool own = totals || S == 1;  // the segments are formed here
   if (own) {
     const unsigned items = tid < S ? (S == 1 ? (unsigned)*q_eff : totals[tid]) : 0u;
@@ -1677,15 +1677,14 @@ __global__ void __launch_bounds__(256) st_count_kernel(
         si.shape = (unsigned)c.TX | (unsigned)min(kSuperTile, c.TX - ox) << 16 |
                    (unsigned)min(kSuperTile, c.TY - oy) << 20;
         s_seg[tid] = si;
-        s_st[tid] = (unsigned char)s;
         segs[gt] = si;
       }
       __syncthreads();
     }
     const Segment si = own ? s_seg[it & 255] : load_segment(segs, g);
-    const int s = packed ? 0 : own ? (int)s_st[it & 255] : (int)seg_st[g];
     int ox = 0, oy = 0;
-    if (!packed) {
+    if (!packed) {  // (over 65,536 super-tiles or 8,000 tiles a side: not own)
+      const int s = (int)seg_st[g];
       const CamInfo& c = ct.c[view_of_st(ct, s)];
       ox = ((s - c.st_off) % c.STX) * kSuperTile;
       oy = ((s - c.st_off) / c.STX) * kSuperTile;
