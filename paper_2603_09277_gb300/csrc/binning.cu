@@ -6,10 +6,11 @@
 // P pairs, the sort works on rows and on row x super-tile items (a
 // super-tile is 8x8 tiles), and the pairs are only ever written once, into
 // their final slots:
-//   1. compact the visible rows (scan of a visibility flag);
+//   1. drop the rows without tiles (an ordered compaction in the one-launch sort;
+//      above 2M rows the depth sort's first pass reads the rows and leaves them out);
 //   2. stable LSD radix sort of the visible rows by FP32 depth bits, on the
-//      bits that vary over the visible rows (up to 9-bit digits: 3 passes
-//      for a range of up to 27 bits; ties keep row order = Gaussian id order);
+//      bits that vary over the visible rows (digits of up to 8 bits: 3 passes
+//      for a range of up to 24 bits; ties keep row order = Gaussian id order);
 //   3. gather every row's rect in depth order (16-bit packed); block scans
 //      give the pair count P and each block's first super-tile item (count
 //      Q <= P);
@@ -17,7 +18,7 @@
 //      (super-tile, row) for the super-tiles each rect meets, in depth order
 //      (4 consecutive items per thread, owners by binary search);
 //   5. stable radix sort of the items by super-tile id (one pass for up to
-//      512 super-tiles), so every super-tile holds its rows in depth order;
+//      256 super-tiles), so every super-tile holds its rows in depth order;
 //   6. per segment of 1024 rows of a super-tile: each row's rect within the
 //      super-tile and per-tile counts; scans over segments and over all
 //      tiles give every tile's list start (the ranges);
@@ -105,9 +106,10 @@ __device__ __forceinline__ unsigned long long block_sum(unsigned long long x) {
 
 // A CTA's arrival at the end of a kernel whose last CTA goes on to a step
 // over every CTA's results (a scan of the block sums, say), in place of a
-// separate single-CTA launch.  Each CTA makes its results visible
-// (a fence by one thread behind a block barrier) before it counts itself, so the CTA that counts last sees
-// all of them; it reads them through L2 (__ldcg).  No CTA waits for another.
+// separate single-CTA launch.  Each CTA makes its results visible (a fence by one
+// thread behind a block barrier) before it counts itself, so the CTA that counts
+// last sees all of them; it reads them through L2 (__ldcg).  No CTA waits for
+// another.
 // The counter is zeroed with the pipeline's counters before the launch.
 // Returns true in every thread of the last CTA.
 __device__ __forceinline__ bool last_block_arrives(unsigned long long* counter,
@@ -2212,9 +2214,6 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
                      status_dev};
   // the visible rows' depth-bit range (complement of the smallest, largest)
   unsigned* range = reinterpret_cast<unsigned*>(w.counters + 12);
-  // scan blocks of 1,024 rows (4 per thread) keep many CTAs in flight when
-  // few rows are visible; on large row counts 4,096-row blocks (16 per
-  // thread) are faster
   // the projection's 8-bit packed rects (views of at most 255 tiles per side)
   const unsigned* rect8 = rect8_fits(ct) ? proj->rect8 : nullptr;
   bool coop = n_rows > 0 && n_rows <= kCoopRows && coop_available();
@@ -2245,6 +2244,10 @@ int launch_bin_sort(const gs_proj* proj, int N, const CamTable& ct, void* worksp
     }
   }
   const SortedRows rows_sorted{w.rv[0], w.rv[1], coop ? nullptr : range};
+  // scan blocks: 256 rows (one per thread) behind the one-launch sort, whose warps
+  // count them; in the separate kernels 1,024 rows (4 per thread), which keep many
+  // CTAs in flight when few rows are visible, and above 4M rows 4,096 (16 per thread),
+  // which are faster there
   const bool small = n_rows <= (4ll << 20);
   const int items = coop ? 1 : small ? 4 : 16;
   const long long nb = (n_rows + kScanThreads * items - 1) / (kScanThreads * items);

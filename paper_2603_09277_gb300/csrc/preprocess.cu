@@ -12,9 +12,10 @@
 // coalesced across the warp; quaternions and SH rows use 16-byte loads.
 //
 // Backward: hand-derived adjoint of the same steps, one thread per Gaussian
-// that the blending adjoint touched in some view, summing over views; the covariance part runs through the Cholesky factor of the
-// 2D covariance (whitened form) and accumulates the log-scale and
-// rotation-matrix gradients over views, pushed to the quaternion once.
+// that the blending adjoint touched in some view, summing over views; the
+// covariance part runs through the Cholesky factor of the 2D covariance
+// (whitened form) and accumulates the log-scale and rotation-matrix gradients
+// over views, pushed to the quaternion once.
 #include <algorithm>
 
 #include "gs_internal.cuh"

@@ -33,11 +33,12 @@
 //   projection's adjoint applies 1 / sigma, the conic and the signs once per
 //   Gaussian.
 // The thread sums the 9 per-Gaussian values (6 moments, 3 colour weights)
-// over its pixels.  When few lanes of the warp contribute, each of them adds its values to grad2d with three vector atomics;
-// otherwise the warp sums them with a split-transpose shuffle reduction (12
-// shuffles leave one of the 9 totals in each of 9 lane pairs) and 9 lanes
-// add them with one atomic instruction.  (All 32 lanes adding to one address
-// in one instruction serialise in L2: the threshold stays below 32.)
+// over its pixels.  When few lanes of the warp contribute, each of them adds its
+// values to grad2d with three vector atomics; otherwise the warp sums them with a
+// split-transpose shuffle reduction (12 shuffles leave one of the 9 totals in each of
+// 9 lane pairs) and 9 lanes add them with one atomic instruction.  (All 32 lanes
+// adding to one address in one instruction serialise in L2: the threshold stays
+// below 32.)
 // With two pixels per thread both pixels go through packed FP32 (f32x2)
 // arithmetic, in the forward as well.
 //
