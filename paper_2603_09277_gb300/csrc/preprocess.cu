@@ -938,9 +938,9 @@ constexpr int kAdjChunk = 2048;  // most Gaussians of a CTA
 constexpr int kAdjRun = 128;     // of which this many are consecutive
 
 // First Gaussian of word w of a CTA's chunk (see preprocess_bwd_kernel).
-__device__ __forceinline__ long long adj_first(int w) {
-  constexpr int kWords = kAdjRun / 32;
-  return ((long long)(w / kWords) * gridDim.x + blockIdx.x) * kAdjRun + 32 * (w % kWords);
+__device__ __forceinline__ unsigned adj_first(unsigned w) {
+  constexpr unsigned kWords = kAdjRun / 32;
+  return ((w / kWords) * gridDim.x + blockIdx.x) * (unsigned)kAdjRun + 32u * (w % kWords);
 }
 
 // The adjoint over the touched Gaussians.  A CTA takes `chunk` Gaussians: it merges
@@ -957,8 +957,8 @@ __device__ __forceinline__ long long adj_first(int w) {
 // scenes, whose views touch a few ranges of ids).  With consecutive chunks those
 // ranges were left to a few CTAs.  Measured (captured, us, ids at random / in Morton
 // order): 1M clusters, degree 3, one view 47 / 86 with consecutive chunks, 48 / 37
-// with runs; 4 views 198 / 208, 180 / 134; 8 views of 3M 50 / 94, 52 / 45 (runs of
-// 256 there: 52 / 48).
+// with runs; 4 views 193 / 203, 186 / 140; 8 views of 3M 51 / 92, 51 / 40; 100k of
+// degree 1 7.9 / 10.8, 8.1 / 10.5.
 //
 // CTAs per SM the register budget allows.  Measured under stage events in eager
 // steps: 8 views of 3M Gaussians (degree 0) 63.6 us at 4, 59.1 at 5, 60.6 at 6; a
@@ -978,7 +978,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
     float* g_quats, float* g_opac, float* g_sh) {
   behind_previous();
   __shared__ unsigned s_any[kAdjChunk / 32];
-  __shared__ unsigned short s_idx[kAdjChunk];
+  __shared__ unsigned s_idx[kAdjChunk];
   __shared__ unsigned s_n;
   const int tid = threadIdx.x;
   const int words = chunk / 32;
@@ -989,13 +989,13 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
 #pragma unroll 4
   for (int i = tid; i < ct.V * words; i += kAdjThreads) {
     const int v = i / words, w = i - v * words;
-    const long long g = adj_first(w);
-    if (g >= N) continue;
-    const long long r0 = (long long)v * N + g;  // the word's first row
+    const unsigned g = adj_first((unsigned)w);
+    const bool in = g < (unsigned)N;
+    const long long r0 = in ? (long long)v * N + g : 0;  // the word's first row
     const unsigned lo = touched_word(grad2d, r0 >> 5);
     const unsigned hi = (r0 | 31) + 1 < rows ? touched_word(grad2d, (r0 >> 5) + 1) : 0u;
-    unsigned m = __funnelshift_r(lo, hi, (unsigned)(r0 & 31));
-    if (N - g < 32) m &= (1u << (int)(N - g)) - 1u;  // (rows of the next view)
+    unsigned m = in ? __funnelshift_r(lo, hi, (unsigned)(r0 & 31)) : 0u;
+    if (in && (unsigned)N - g < 32u) m &= (1u << ((unsigned)N - g)) - 1u;  // (rows of the next view)
     if (m) atomicOr(&s_any[w], m);
   }
   __syncthreads();
@@ -1003,12 +1003,12 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<DEG>()) preproces
     unsigned m = s_any[w];
     if (!m) continue;
     unsigned at = atomicAdd(&s_n, (unsigned)__popc(m));
-    for (; m; m &= m - 1u) s_idx[at++] = (unsigned short)(32 * w + __ffs((int)m) - 1);
+    for (; m; m &= m - 1u) s_idx[at++] = adj_first((unsigned)w) + (unsigned)__ffs((int)m) - 1u;
   }
   __syncthreads();
   const int cnt = (int)s_n;
   for (int i = tid; i < cnt; i += kAdjThreads) {
-    const long long g = adj_first(s_idx[i] >> 5) + (s_idx[i] & 31);
+    const unsigned g = s_idx[i];
     if (!GS_IN_BOUNDS(g, N, 301)) continue;
     adjoint_gaussian<DEG, WHITE>((int)g, means, log_scales, quats, opacity_logits, sh, N, ct,
                                  dilation, shp, grad2d, g_means, g_ls, g_quats, g_opac, g_sh);
