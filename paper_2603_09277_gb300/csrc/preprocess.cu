@@ -470,16 +470,15 @@ __device__ __forceinline__ Projected project_adjoint(const CamInfo& c, const Act
 // Templated on the staging dtype and the SH degree in use: with the degree a
 // constant the basis values and the coefficient loop stay in registers (a
 // runtime degree put them in local memory).
-// Resident projection CTAs per SM the register budget targets: 4 (64
-// registers, no spills) up to SH degree 1, 5 (48 registers) above.  Measured
-// on cfg3 (degree 0): 562 us at 5, 486 us at 4; on cfg2 (degree 3): 43.7 us
-// at 5, 47.5 us at 4.
-template <int DEG>
-constexpr int pre_ctas_per_sm() {
-  return DEG <= 1 ? 4 : 5;
-}
+// Resident projection CTAs per SM the register budget targets: 4 (64 registers; no
+// spills up to degree 1, 32 to 40 bytes above).  Measured (captured, us, 5 CTAs per SM
+// of 48 registers / 4): degree 3, 1M Gaussians of which 7 % are visible, one view
+// 41.0 / 40.9, four views 109 / 107 (eager, with the 2D attributes, 132 / 122), 300k all
+// visible in three views 51 / 47, BF16 records at 1080p 38.6 / 39.7; degree 2, 600k in
+// two views 45.6 / 40.7; degree 0, 8 views of 3M 562 / 486.
+constexpr int kPreCtas = 4;
 template <int DT, int DEG>
-__global__ void __launch_bounds__(256, pre_ctas_per_sm<DEG>()) preprocess_kernel(
+__global__ void __launch_bounds__(256, kPreCtas) preprocess_kernel(
     const float* means, const float* log_scales,
     const float* quats, const float* opacity_logits,
     const float* sh, int N, const CamTable ct, float dilation, float near_z,
