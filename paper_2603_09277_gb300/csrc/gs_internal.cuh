@@ -268,9 +268,10 @@ __device__ __forceinline__ int find_view_of_pixel(const CamTable& ct, long long 
 // that nothing writes during the kernel's life, such a kernel and the device
 // functions it calls take no __restrict__ pointers (the memory clobber does not order
 // accesses through those) and use no __ldg: plain loads, or __ldcg / __ldcs.  Measured
-// against the same kernels with both (and plain launches): captured steps 0.996 to
-// 1.005 of the time; the projection, whose rematerialised loads had to be written out,
-// 136 us with dependent launches, 141 without.
+// against the same kernels with both, launched plainly: captured steps at 0.993 to
+// 1.005 of the speed; a captured projection of 1M Gaussians into one view at degree 3
+// 40.9 us instead of 38.9, at degree 1 35.1 instead of 39.5; eager calls faster (see
+// launch_behind).
 namespace gs {
 __device__ __forceinline__ void behind_previous() {
   asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
@@ -289,9 +290,9 @@ int check_launch();
 // Launch of a kernel whose first statement is behind_previous(): issued to a
 // stream, its blocks are placed while the stream's previous kernel still runs its
 // last ones (programmatic dependent launch), which hides the launch and the
-// previous kernel's drain: three views' lists 234 -> 220 us (10 launches), a
-// blending with its adjoint 158 -> 146 (5), D-SSIM on two views 214 -> 205 (4), a
-// 1920x1080 render 383 -> 376.  Into a graph the launch is a plain one: a
+// previous kernel's drain: three views' lists 215 -> 200 us (10 launches), a
+// blending with its adjoint 171 -> 159 (5), D-SSIM on two views 212 -> 205 (4), a
+// 1920x1080 render 367 -> 363.  Into a graph the launch is a plain one: a
 // replay starts plain kernel nodes as fast, and with programmatic edges a captured
 // step of 10k Gaussians took 194 instead of 176 us, of 1M 615 instead of 608.
 // (An error is picked up by check_launch.)
